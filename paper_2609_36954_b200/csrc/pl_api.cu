@@ -48,6 +48,9 @@ struct pl_schedule_s {
   bool pipelined_reduce = false;  // bulk-copy datapath: every reduce op is plain, run the 12-warp variant
   bool stage_ahead = false;       // double-buffered staging: two scratch halves and flag sets, chosen by launch parity
   uint64_t scratch_half = 0;      // bytes of one half (all ranks)
+  bool layer_kernel = false;      // layered direct-fused all-reduce with one op per queue and layer: layer executor
+  bool layer_cluster = false;     // ... as one thread-block cluster
+  int layer_break_layer = -1, layer_break_queue = -1;  // test hook (pl_schedule_debug_break_wait without flag words)
   int packet_ctas_per_rank = 0;   // > 0: packet datapath (layered one-shot all-reduce), CTAs per rank
   long long packet_break_op = -1; // test hook (pl_schedule_debug_break_wait on a packet schedule)
   size_t off_trace = 0;
@@ -402,6 +405,17 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   }
   pol = default_policy(rq, capacity);
   if (requested > capacity) return PL_ERR_OVERSUBSCRIBED;
+  LayerShape layers{0, 0, false};
+  const uint64_t layer_bytes = rq.count_per_rank * (uint64_t)elem_size(comm->dtype);
+  if (rq.n_layers > 1 && rq.algo == PL_ALGO_DIRECT_FUSED && pol.datapath == PL_DP_LDST && requested == 0 && !rq.staged && comm->dtype != PL_U8 &&
+      (!opts || (opts->threads == 0 && opts->slice_bytes == 0)) && layer_bytes > 0 && layer_bytes % (16 * (uint64_t)comm->R) == 0) {
+    layers = layer_shape(comm->R, layer_bytes, capacity, true);
+    if (layers.cluster && !comm->planner && !layers_cluster_fits(comm->dtype, comm->R, hook != 0, layers.ctas_per_rank * comm->R, layers.threads))
+      layers = layer_shape(comm->R, layer_bytes, capacity, false);
+    pol.n_ctas = layers.ctas_per_rank * comm->R;
+    pol.threads = layers.threads;
+    rq.layer_ctas_per_rank = layers.ctas_per_rank;
+  }
   if (pol.n_ctas > capacity) return PL_ERR_OVERSUBSCRIBED;
   rq.pol = pol;
 
@@ -417,6 +431,8 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   S->stage_ahead = (flags & PL_OPT_STAGE_AHEAD) != 0;
   S->out_scale = out_scale;
   S->hook = hook;
+  S->layer_kernel = layers.ctas_per_rank > 0;
+  S->layer_cluster = layers.cluster;
   std::string err;
   pl_status_t st = lower(rq, &S->L, &err);
   if (st != PL_OK) {
@@ -959,6 +975,11 @@ pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index) {
     s->packet_break_op = (long long)op_index;
     return PL_OK;
   }
+  if (s->layer_kernel) {  // reads no wait entries: told which op is to miss a signal
+    s->layer_break_layer = h.layer;
+    s->layer_break_queue = h.queue;
+    return PL_OK;
+  }
   const size_t pos = (size_t)s->topo_to_dev[op_index];
   DevWait& w = s->waits[pos * s->wait_stride];
   w.need += 1;  // one more signal than the schedule will ever produce
@@ -1084,7 +1105,16 @@ pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
   P.overlap_launch = s->overlap_launch ? 1u : 0u;
   P.pipelined_reduce = s->pipelined_reduce ? 1u : 0u;
   P.bcast_copies = s->bcast_copies ? 1u : 0u;
-  cudaError_t le = s->pol.datapath == PL_DP_TMA
+  LayerParams Y;
+  if (s->layer_kernel) {
+    Y.in_stride = s->L.message_bytes;
+    Y.out_stride = s->info.out_bytes[0] / (uint64_t)s->L.n_layers;
+    Y.n_layers = (uint32_t)s->L.n_layers;
+    Y.break_layer = s->layer_break_layer;
+    Y.break_queue = s->layer_break_queue;
+  }
+  cudaError_t le = s->layer_kernel ? launch_layers(s->comm->dtype, P, Y, s->pol.n_ctas, s->pol.threads, s->layer_cluster, static_cast<cudaStream_t>(stream))
+                   : s->pol.datapath == PL_DP_TMA
                        ? launch_exec_tma(s->comm->dtype, P, s->sm_window ? s->comm->sm_count : s->pol.n_ctas, static_cast<cudaStream_t>(stream))
                        : launch_exec(s->comm->dtype, P, s->pol.n_ctas, s->pol.threads, static_cast<cudaStream_t>(stream));
   if (le != cudaSuccess) return PL_ERR_CUDA;

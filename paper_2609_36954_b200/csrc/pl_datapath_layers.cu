@@ -1,0 +1,284 @@
+// Datapath for layered direct-fused all-reduces (the decode shape: L small all-reduces in one
+// launch) whose grid is left to the library.
+//
+// Such a schedule is regular: every queue holds exactly one op per layer, the ops of layer l
+// read and write the same slice of every rank's buffers l messages further on, and every op of
+// layer l + 1 waits for every op of layer l.  The register executor runs it too, but pays on
+// every layer for being able to run anything: descriptors through shared memory, 512 threads at
+// two CTA barriers whatever the slice needs, input lines that come from DRAM only after the flag.
+// A layer is a serial chain (flag seen -> inputs -> sum -> outputs acknowledged -> flag), so what
+// counts is what sits on that chain:
+//   - a CTA has as many threads as its slice has 16-byte units (32 at the small end), one unit per
+//     thread, addresses from the kernel parameters;
+//   - the lines of a later layer's inputs are asked into L2 while the flag of this layer travels
+//     (a prefetch is not a read: the values are loaded after the flag, from the point of
+//     coherence);
+//   - CLUSTER: when the whole schedule fits 16 CTAs, they form one thread-block cluster and the
+//     flag is the cluster barrier (release / acquire): one hop instead of an increment in L2 and a
+//     poll that has to see it.
+// What bounds it: at the small end the chain (outputs acknowledged by L2 about 0.6 us, barrier or
+// flag 0.3-0.6 us, inputs from L2 0.4 us), at 1 MiB the chain plus 16 MiB of L2 traffic per layer
+// (2.6 us at DRAM rate, which the prefetch and the write-back overlap with the chain).
+// Measured on B200, R = 8, bf16, 80 layers in one launch, three sets of buffers in turn, us per
+// layer, register executor -> this kernel: 8 KiB 2.10 -> 1.32, 16 KiB 2.40 -> 1.32-1.51 (cluster);
+// 64 KiB 3.20 -> 1.96, 128 KiB 3.28 -> 2.00, 512 KiB 3.86 -> 2.63, 1 MiB 4.99 -> 3.64 (flags).
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <type_traits>
+
+#include "pl_device.cuh"
+#include "pl_internal.h"
+#include "pl_kernels.h"
+
+namespace pl {
+namespace {
+
+using namespace dev;
+
+constexpr int kMaxThreads = kLayerThreads, kMaxClusterThreads = kLayerClusterThreads;  // threads that move data; CLUSTER adds one warp that asks for lines ahead
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// One unit (16 bytes of every source) of a layer: NR bounds the ranks, all loads before the adds.
+template <int DT, int NR, bool HOOK>
+__device__ __forceinline__ void layer_unit(const ExecParams& P, uint64_t in_off, uint64_t out_off) {
+  const int R = P.n_ranks;
+  uint4 q[NR];
+#pragma unroll
+  for (int s = 0; s < NR; ++s)
+    if (s < R) q[s] = ld16(static_cast<const char*>(P.base[kSlotIn + s]) + in_off);
+  uint4 second[HOOK ? NR : 1];
+  if constexpr (HOOK) {
+    if (P.hook & PL_HOOK_RESIDUAL) {
+#pragma unroll
+      for (int s = 0; s < NR; ++s)
+        if (s < R) second[s] = ld16(static_cast<const char*>(P.base[kSlotAux + s]) + in_off);
+    }
+  }
+  Acc<DT> acc;
+  acc.zero();
+#pragma unroll
+  for (int s = 0; s < NR; ++s)
+    if (s < R) {
+      if constexpr (DT == PL_BF16) acc.add_bf16(q[s]);
+      else acc.add(q[s]);
+    }
+  if constexpr (HOOK) {
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+      if (k < R) store_final_q<DT>(acc, P.out_scale, P.hook, static_cast<char*>(P.base[kSlotOut + k]) + out_off, second[k]);
+  } else {
+    uint4 r;
+    if constexpr (DT == PL_BF16) r = acc.to_bf16(P.out_scale);
+    else r = acc.result(P.out_scale);
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+      if (k < R) st16(static_cast<char*>(P.base[kSlotOut + k]) + out_off, r);
+  }
+}
+
+// Lines of one layer's operands for this CTA's slice into L2: line j of rank s by the thread with
+// number j * NR + s modulo n.  The slice starts on a 16-byte boundary, so it can touch one line
+// more than its bytes fill; that one is left to the load.
+template <int NR>
+__device__ __forceinline__ void ask_for_layer(const ExecParams& P, uint64_t in_off, uint32_t units, uint32_t t, uint32_t n) {
+  const uint32_t lines = (units + 7u) >> 3;
+  const bool residual = P.hook & PL_HOOK_RESIDUAL;
+  for (uint32_t j = t; j < lines * NR; j += n) {
+    const uint32_t line = j / NR, s = j % NR;
+    if (s >= (uint32_t)P.n_ranks) continue;
+    const uint64_t off = in_off + (uint64_t)line * 128u;
+    prefetch_l2(static_cast<const char*>(P.base[kSlotIn + s]) + off);
+    if (residual) prefetch_l2(static_cast<const char*>(P.base[kSlotAux + s]) + off);
+  }
+}
+
+template <int DT, int NR, bool HOOK, bool CLUSTER>
+__global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThreads) pl_layers_kernel(const __grid_constant__ ExecParams P,
+                                                                                  const __grid_constant__ LayerParams Y) {
+  __shared__ int s_abort;
+  const uint32_t tid = threadIdx.x, q = blockIdx.x, nq = P.n_queues;
+  pdl_launch_dependents();
+  // descriptors are immutable: read before the wait for the launch in front
+  const DevOp* const op0 = P.ops + q;
+  const uint64_t in_off0 = P.srcs[(uint64_t)q * P.src_stride] & 0xFFFFFFFFFFFFull;  // the same in every rank's input
+  const uint64_t out_off0 = op0->dst & 0xFFFFFFFFFFFFull;
+  const uint32_t units = (uint32_t)(op0->count / Acc<DT>::kElems);
+  const uint32_t out_unit = (HOOK && DT == PL_BF16 && (P.hook & PL_HOOK_F32_OUT)) ? 32u : 16u;
+  if (tid == 0) s_abort = 0;
+  uint32_t topo = op0->topo;
+  pdl_wait();
+
+  if constexpr (CLUSTER) {
+    const uint32_t movers = blockDim.x - 32u;
+    for (uint32_t l = 0; l < Y.n_layers; ++l) {
+      if ((int)l == Y.break_layer) {
+        // test hook: a wait that nothing satisfies.  Every CTA leaves here; the one whose op was
+        // broken gives up after the time limit and says so.
+        if ((int)q == Y.break_queue && tid == 0) {
+          const unsigned long long t0 = globaltimer_ns();
+          while (globaltimer_ns() - t0 <= P.timeout_ns) {}
+          record_timeout(P, (int)q, topo, op0->signal + l - 1u, nq, 0);
+        }
+        break;
+      }
+      const uint64_t in_off = in_off0 + l * Y.in_stride, out_off = out_off0 + l * Y.out_stride;
+      if (P.trace && tid == 0) P.trace[2ull * topo] = globaltimer_ns();
+      if (tid < movers) {
+        for (uint32_t u = tid; u < units; u += movers) layer_unit<DT, NR, HOOK>(P, in_off + u * 16ull, out_off + (uint64_t)u * out_unit);
+      } else if (l + 1 < Y.n_layers) {
+        ask_for_layer<NR>(P, in_off + Y.in_stride, units, tid - movers, 32u);
+      }
+      if (l + 1 < Y.n_layers) {
+        if (P.trace) {
+          __syncthreads();
+          if (tid == 0) P.trace[2ull * topo + 1] = globaltimer_ns();
+        }
+        __syncwarp();
+        cluster_arrive_release();
+        cluster_wait_acquire();
+      } else if (P.trace) {
+        __syncthreads();
+        if (tid == 0) P.trace[2ull * topo + 1] = globaltimer_ns();
+      }
+      topo += nq;
+    }
+  } else {
+    const unsigned long long epoch = *reinterpret_cast<volatile unsigned long long*>(P.epoch) + 1ull;
+    bool aborted = false;
+    unsigned long long* flag = P.flags + op0->signal;  // this layer's; the next layer's is the next word
+    for (uint32_t l = 0; l < Y.n_layers; ++l) {
+      if (l > 0) {
+        if (tid == 0) {
+          // every CTA signals once per layer; acquire, bounded by the time limit
+          const unsigned long long need = epoch * (gridDim.x + (((int)l == Y.break_layer && (int)q == Y.break_queue) ? 1ull : 0ull));
+          unsigned long long seen = ld_acquire_u64(flag);
+          if (seen < need) {
+            const unsigned long long t0 = globaltimer_ns();
+            uint32_t spins = 0;
+            while ((seen = ld_acquire_u64(flag)) < need) {
+              if ((++spins & 63u) == 0) {
+                if (ld_volatile_s32(P.status + 8)) { s_abort = 1; break; }
+                if (globaltimer_ns() - t0 > P.timeout_ns) {
+                  record_timeout(P, (int)q, topo, (uint32_t)(flag - P.flags), need, seen);
+                  s_abort = 1;
+                  break;
+                }
+              }
+            }
+          }
+        }
+        ++flag;
+        __syncthreads();
+        if (s_abort) { aborted = true; break; }
+      }
+      const uint64_t in_off = in_off0 + l * Y.in_stride, out_off = out_off0 + l * Y.out_stride;
+      if (P.trace && tid == 0) P.trace[2ull * topo] = globaltimer_ns();
+      for (uint32_t u = tid; u < units; u += blockDim.x) layer_unit<DT, NR, HOOK>(P, in_off + u * 16ull, out_off + (uint64_t)u * out_unit);
+      if (l + 1 < Y.n_layers || P.trace) {
+        __syncthreads();  // every thread's writes are done
+        if (tid == 0) {
+          if (P.trace) P.trace[2ull * topo + 1] = globaltimer_ns();
+          // cumulative: covers the other threads' stores, observed through the barrier
+          if (l + 1 < Y.n_layers) red_release_add_u64(flag, 1ull);
+        }
+      }
+      if (l + 1 < Y.n_layers) {
+        topo += nq;
+        // while the flag travels (asking two layers ahead measured the same)
+        ask_for_layer<NR>(P, in_off + Y.in_stride, units, tid, blockDim.x);
+      }
+    }
+    __syncthreads();
+    if (tid == 0 && !aborted) {
+      // last CTA to finish advances the epoch for the next execute
+      const unsigned long long prev = atomicAdd(P.epoch + 1, 1ull);
+      if (prev == (unsigned long long)gridDim.x - 1ull) {
+        P.epoch[1] = 0ull;
+        __threadfence();
+        *reinterpret_cast<volatile unsigned long long*>(P.epoch) = epoch;
+      }
+    }
+  }
+}
+
+template <int DT, int NR, bool HOOK, bool CLUSTER>
+cudaError_t prepare_t(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int grid, int threads, bool overlap) {
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)(threads + (CLUSTER ? 32 : 0)));
+  int na = 0;
+  if (CLUSTER) {
+    // up to 16 CTAs: more than the portable 8 needs the opt-in (a per-device attribute of the function)
+    if (grid > 8) {
+      const cudaError_t e = cudaFuncSetAttribute(pl_layers_kernel<DT, NR, HOOK, CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = (unsigned)grid;
+    attr[na].val.clusterDim.y = 1;
+    attr[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  if (overlap) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = na;
+  return cudaSuccess;
+}
+
+template <int DT, int NR, bool HOOK, bool CLUSTER>
+cudaError_t launch_t(const ExecParams& P, const LayerParams& Y, int grid, int threads, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  const cudaError_t e = prepare_t<DT, NR, HOOK, CLUSTER>(cfg, attr, grid, threads, P.overlap_launch);
+  if (e != cudaSuccess) return e;
+  cfg.stream = stream;
+  return cudaLaunchKernelEx(&cfg, pl_layers_kernel<DT, NR, HOOK, CLUSTER>, P, Y);
+}
+
+template <int DT, int NR, bool HOOK>
+bool cluster_fits_t(int grid, int threads) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (prepare_t<DT, NR, HOOK, true>(cfg, attr, grid, threads, false) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, pl_layers_kernel<DT, NR, HOOK, true>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n >= 1;
+}
+
+// f(dtype, rank bound, hook) over the instantiations; int32 has no hooks.
+template <typename F>
+auto pick(int dtype, int R, bool hook, F f) {
+  auto ranks = [&](auto dt, auto hk) {
+    if (R <= 4) return f(dt, std::integral_constant<int, 4>{}, hk);
+    if (R <= 8) return f(dt, std::integral_constant<int, 8>{}, hk);
+    return f(dt, std::integral_constant<int, PL_MAX_RANKS>{}, hk);
+  };
+  if (dtype == PL_BF16) return hook ? ranks(std::integral_constant<int, PL_BF16>{}, std::true_type{}) : ranks(std::integral_constant<int, PL_BF16>{}, std::false_type{});
+  if (dtype == PL_F32) return hook ? ranks(std::integral_constant<int, PL_F32>{}, std::true_type{}) : ranks(std::integral_constant<int, PL_F32>{}, std::false_type{});
+  return ranks(std::integral_constant<int, PL_I32>{}, std::false_type{});
+}
+
+}  // namespace
+
+cudaError_t launch_layers(int dtype, const ExecParams& P, const LayerParams& Y, int grid, int threads, bool cluster, cudaStream_t stream) {
+  if (dtype == PL_U8 || (dtype == PL_I32 && P.hook)) return cudaErrorInvalidValue;
+  return pick(dtype, P.n_ranks, P.hook != 0, [&](auto dt, auto nr, auto hk) {
+    return cluster ? launch_t<dt(), nr(), hk(), true>(P, Y, grid, threads, stream) : launch_t<dt(), nr(), hk(), false>(P, Y, grid, threads, stream);
+  });
+}
+
+bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads) {
+  return pick(dtype, R, hook, [&](auto dt, auto nr, auto hk) { return cluster_fits_t<dt(), nr(), hk()>(grid, threads); });
+}
+
+}  // namespace pl

@@ -107,6 +107,14 @@ struct ExecParams {
   uint32_t pipelined_reduce;  // host side only: every reduce op is plain (element-typed operands), use the 12-warp variant
 };
 
+// What the layer executor needs on top of ExecParams (see pl_datapath_layers.cu): the distance from
+// a layer's operands to the next layer's, in bytes.
+struct LayerParams {
+  uint64_t in_stride, out_stride;
+  uint32_t n_layers;
+  int32_t break_layer, break_queue;  // test hook of the cluster variant (no wait entries to break), -1 = none
+};
+
 // Parameters of the packet executor (layered one-shot all-reduce, see pl_datapath_packet.cu).
 struct PacketParams {
   const void* in[PL_MAX_RANKS];
@@ -120,6 +128,15 @@ struct PacketParams {
   long long break_op;                 // test hook: index of an op whose polls can never be satisfied, -1 = none
   int n_ranks, n_layers, ctas_per_rank;
   float out_scale;
+};
+
+// Shape of a layered direct-fused all-reduce on the layer executor.
+constexpr int kLayerThreads = 512, kLayerClusterThreads = 256;  // most threads a CTA of it has
+constexpr int kLayerClusterCtas = 16; // most CTAs of one thread-block cluster
+struct LayerShape {
+  int ctas_per_rank;  // slices a rank's partition is cut into, one queue each
+  int threads;
+  bool cluster;       // the whole grid is one thread-block cluster
 };
 
 struct Policy {
@@ -154,6 +171,7 @@ struct BuildRequest {
   int root;                  // rooted collectives
   bool staged;               // stage through schedule-owned memory (ordinary application buffers)
   uint64_t staging_bytes;    // staging capacity per rank (0 = default)
+  int layer_ctas_per_rank;   // > 0: layered direct-fused all-reduce, one op per queue and layer, this many queues per rank
   int packet_ctas_per_rank;  // > 0: layered all-reduce on the packet datapath with this many CTAs per rank
   uint32_t hook;             // PL_HOOK_* bits
   bool stage_ahead;          // PL_OPT_STAGE_AHEAD
@@ -172,6 +190,7 @@ int level_width(const Lowered& L, int R);
 // bulk_datapath: the schedule runs on the bulk-copy executor, where program order on one queue
 // orders less than on the register executor (see validate()).
 pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapath);
+LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster);
 Policy default_policy(const BuildRequest& rq, int max_resident_ctas);
 
 }  // namespace pl

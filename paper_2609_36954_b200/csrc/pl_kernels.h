@@ -19,6 +19,11 @@ int exec_tma_max_ctas_per_sm(int dtype, int stages, uint32_t stage_bytes);
 int exec_tma_threads(bool pipelined);
 size_t exec_tma_smem_bytes(int stages, uint32_t stage_bytes);
 
+// layered direct-fused all-reduces with one op per queue and layer (`cluster`: the grid is one
+// thread-block cluster and the cluster barrier takes the place of the flags)
+cudaError_t launch_layers(int dtype, const ExecParams& P, const LayerParams& Y, int grid, int threads, bool cluster, cudaStream_t stream);
+bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads);
+
 // packet executor (latency path): rank = cluster of ctas_per_rank CTAs
 cudaError_t launch_exec_packet(int dtype, const PacketParams& P, int threads, bool overlap, cudaStream_t stream);
 int exec_packet_max_groups(int dtype, int ctas_per_rank, int threads);

@@ -402,6 +402,33 @@ void ar_fused(Emitter& em, const Geo& g, int layer, uint64_t in_off, uint64_t ou
     }
 }
 
+// One layer of a direct-fused all-reduce cut for the layer executor: rank k's partition in `slices`
+// equal parts of whole 16-byte vectors (the last one may be shorter), slice j on the rank's queue j
+// in every layer.
+void ar_fused_sliced(Emitter& em, const Geo& g, int slices, int layer, uint64_t base_off, const LayerEdges& le) {
+  const uint64_t vec = 16 / g.es, vecs = g.P / vec;
+  uint64_t per = (vecs + slices - 1) / slices;
+  if (per >= 16) per = (per + 7) / 8 * 8;  // as layer_shape() counted them
+  per *= vec;
+  for (int k = 0; k < g.R; ++k)
+    for (uint64_t b = 0, j = 0; b < g.P; b += per, ++j) {
+      HostOp op;
+      op.kind = PL_OP_REDUCE;
+      op.exec_rank = k;
+      op.layer = layer;
+      op.count = std::min(per, g.P - b);
+      const uint64_t off = base_off + (k * g.P + b) * g.es;
+      op.dst = ref(k, PL_BUF_OUT, g.dtype, off);
+      op.bcast = true;
+      for (int p = 0; p < g.R; ++p) op.src.push_back(ref(p, PL_BUF_IN, g.dtype, off));
+      op.waits = waits_on(&le, all_ranks(g.R));
+      op.signal = le.done[0];
+      op.queue = (int)j * g.R + k;
+      em.L->ops.push_back(std::move(op));
+    }
+  em.L->queues_preassigned = true;
+}
+
 // all-reduce, direct two-shot = compose<reduce-scatter, all-gather> in one launch
 // (Algorithm 1 without the staging role): rank k reduces chunk c of partition k into its own
 // output and publishes reduced(k,c) to all ranks; every other rank then copies that chunk.
@@ -765,6 +792,24 @@ void a2a_direct_staged(Emitter& em, const Geo& g, uint64_t capacity) {
 
 }  // namespace
 
+// One cluster while it has at most 256 KiB of inputs to read per layer (16 KiB per CTA): at
+// R = 8 a 16 KiB layer takes 1.32-1.45 us as a cluster and 1.66 us with flags, 32 KiB 1.59-2.03
+// (the two values are two B200s) against 1.95, 64 KiB 2.16-2.24 against 1.96.  With flags as many
+// CTAs as there are slices of at least 32 units: 16, 32, 64 or 128 made no difference at 64 KiB
+// and above as long as every SM has a slice at the large end (1 MiB: 128 CTAs 3.6 us, 64 CTAs 5 us).
+LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster) {
+  LayerShape s;
+  const uint64_t units = std::max<uint64_t>(1, message_bytes / (uint64_t)R / 16);  // vectors of a rank's partition
+  s.cluster = allow_cluster && (uint64_t)R * message_bytes <= (256u << 10);
+  uint64_t k = s.cluster ? (uint64_t)(kLayerClusterCtas / R) : std::min<uint64_t>((uint64_t)std::max(1, capacity / R), std::max<uint64_t>(1, units / 32));
+  k = std::min(k, units);
+  uint64_t per = (units + k - 1) / k;
+  if (per >= 16) per = (per + 7) / 8 * 8;  // whole 128-byte lines
+  s.ctas_per_rank = (int)((units + per - 1) / per);
+  s.threads = (int)std::min<uint64_t>(s.cluster ? kLayerClusterThreads : kLayerThreads, (per + 31) / 32 * 32);
+  return s;
+}
+
 // Default knobs for sm_100a ("codesign policy", Sec. 3.2-3.3).  Called twice by the build:
 // first with max_resident_ctas == 0 to settle the datapath and its shared-memory ring (which
 // decide how many CTAs fit on an SM), then with the resulting capacity to settle the grid.
@@ -1087,7 +1132,8 @@ pl_status_t lower_collective(const BuildRequest& rq, Lowered* L, std::string* er
             }
           }
           const uint64_t off = (uint64_t)l * bytes;
-          if (rq.algo == PL_ALGO_ONESHOT) ar_oneshot(em, gw, l, off, off, &le);
+          if (rq.layer_ctas_per_rank > 0) ar_fused_sliced(em, gp, rq.layer_ctas_per_rank, l, off, le);
+          else if (rq.algo == PL_ALGO_ONESHOT) ar_oneshot(em, gw, l, off, off, &le);
           else if (rq.algo == PL_ALGO_DIRECT) ar_direct(em, gp, l, off, off, &le);
           else ar_fused(em, gp, l, off, off, &le);
           le.pub = le.done;
