@@ -222,7 +222,8 @@ typedef struct {
  * when the kernel in front of it on the stream is another execute, its CTAs may be set up
  * while that one drains (the kernel waits for the completion of everything in front of it
  * before it reads anything an earlier launch wrote, so stream order is kept as seen by the
- * data).  Shortens back-to-back executes; no effect after any other kind of work.  The paper
+ * data).  Shortens back-to-back executes; no effect after any other kind of work.  The register and
+ * packet datapaths are launched this way in any case; the option is for the bulk-copy datapath.  The paper
  * has no counterpart (it measures calls inside a CUDA graph, Sec. 5). */
 #define PL_OPT_OVERLAP_LAUNCH 16u
 /* Epoch-parity double buffering of the staging memory (Sec. 4.1-4.2: two staging buffers
