@@ -10,7 +10,11 @@
  *                  list of chunk-granular copy / reduce / copy-reduce ops with wait and
  *                  signal edges (Sec. 3.2, Listing 2, Algorithm 1) -> pl_schedule_build*;
  *   datapath       how bytes move: one persistent sm_100a kernel interprets the per-CTA op
- *                  queues (Sec. 3.3, Listing 3, Algorithm 2) -> pl_execute.
+ *                  queues (Sec. 3.3, Listing 3, Algorithm 2) -> pl_execute.  A schedule whose ops
+ *                  neither wait nor signal needs no queues: with grid, datapath, slices, ring and
+ *                  trace left to the library its ops are laid end to end and executed in tiles, one
+ *                  CTA per tile (same operands, same order of additions; pl_schedule_info reports
+ *                  grid, threads and tile bytes of that launch, n_queues those of the op list).
  *
  * R logical ranks are R sets of buffers in ONE GPU's memory; every rank's buffers are
  * visible to every other rank, i.e. the executor is the paper's variant that skips the
@@ -351,7 +355,9 @@ pl_status_t pl_comm_destroy(pl_comm_t comm);
 /* Measure, on this communicator's GPU, with how many CTAs and on WHICH SMs the write-dominated
  * direct schedules of the bulk-copy datapath (all-gather, all-gather-v, broadcast: 1 read : R
  * writes) run fastest, and make the result the default of later builds on this communicator
- * (opts.n_ctas / opts.idle_sm_count still override; schedules already built keep theirs).  Such
+ * (opts.n_ctas / opts.idle_sm_count still override; schedules already built keep theirs; it
+ * concerns builds that ask for PL_DP_TMA: left to the library these schedules run without queues
+ * and have no grid to tune).  Such
  * a stream is served best with fewer than all SMs writing, and with the right ones sitting out:
  * 16-20 idle SMs taken from SM ids 0-31 or 64-79 gave 97-103 us for the 8 x 64 MiB all-gather on
  * every B200 tried, the same number anywhere else 108-116 us; which SMs a plain launch of fewer

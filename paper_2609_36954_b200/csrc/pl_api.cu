@@ -51,6 +51,9 @@ struct pl_schedule_s {
   bool layer_kernel = false;      // layered direct-fused all-reduce with one op per queue and layer: layer executor
   bool layer_cluster = false;     // ... as one thread-block cluster
   int layer_break_layer = -1, layer_break_queue = -1;  // test hook (pl_schedule_debug_break_wait without flag words)
+  bool flat = false;              // no flags, everything left to the library: one CTA per tile (pl_datapath_flat.cu)
+  FlatLaunch flat_launch{};
+  std::vector<FlatSpan> flat_spans;  // uploaded in place of op list and flags
   int packet_ctas_per_rank = 0;   // > 0: packet datapath (layered one-shot all-reduce), CTAs per rank
   long long packet_break_op = -1; // test hook (pl_schedule_debug_break_wait on a packet schedule)
   size_t off_trace = 0;
@@ -142,6 +145,13 @@ void fill_info(pl_schedule_s* S, int R) {
   I.stages = S->pol.stages;
   I.stage_bytes = S->pol.stage_bytes;
   I.slice_bytes = S->pol.slice_bytes;
+  if (S->flat) {
+    I.grid = (int32_t)S->flat_launch.blocks;
+    I.threads = S->flat_launch.threads;
+    I.smem_bytes = (int32_t)S->flat_launch.smem_bytes;
+    I.stages = 1;
+    I.stage_bytes = S->flat_launch.tile * 16u;
+  }
 }
 
 // Flatten the lowered ops into the device arrays (host side): op i of queue q at index
@@ -195,6 +205,12 @@ void flatten(pl_schedule_s* S, int dtype) {
 }
 
 pl_status_t upload(pl_schedule_s* S, int R) {
+  if (S->flat) {
+    S->blob_bytes = S->flat_spans.size() * sizeof(FlatSpan);
+    if (cudaMalloc(&S->d_blob, S->blob_bytes) != cudaSuccess) { cudaGetLastError(); return PL_ERR_OOM; }
+    if (cudaMemcpy(S->d_blob, S->flat_spans.data(), S->blob_bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
+    return PL_OK;
+  }
   size_t off = 0;
   auto place = [&](size_t bytes) {
     size_t o = off;
@@ -480,6 +496,25 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   }
   for (const HostOp& op : S->L.ops)
     if (op.kind == PL_OP_COPY && op.bcast) S->bcast_copies = true;
+  // No flags and nothing about the launch asked for: no queues.  Planner communicators keep the
+  // queues, which is what their schedules are inspected for.
+  if (!comm->planner && rq.n_layers <= 1 && S->L.n_flags == 0 && !rq.staged && !S->trace && !S->layer_kernel &&
+      (!opts || (opts->n_ctas == 0 && opts->threads == 0 && opts->datapath == PL_DP_AUTO && opts->stages == 0 && opts->stage_bytes == 0 &&
+                 opts->slice_bytes == 0 && !idle_asked))) {
+    bool reduce = false, all = false;
+    if (flat_plan(S->L, comm->R, comm->dtype, &S->flat_spans, &reduce, &all)) {
+      uint64_t units = 0, blocks = 0;
+      for (const FlatSpan& f : S->flat_spans) units += f.units;
+      S->flat_launch = flat_launch(comm->R, reduce, all, pol.datapath == PL_DP_TMA, hook, units);
+      for (FlatSpan& f : S->flat_spans) {
+        f.first_block = (uint32_t)blocks;
+        blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;
+      }
+      S->flat_launch.blocks = (uint32_t)blocks;
+      S->flat = blocks <= 0x7FFFFFFFull;
+      if (S->flat) S->pol.idle_count = 0;
+    }
+  }
   // A window of idle SMs needs: the bulk-copy datapath with one CTA per SM, no flags (a queue
   // may be claimed late, so no queue may wait for another), one staging buffer, at most 160 SMs,
   // and ordinary launches: the claim words serve one launch at a time, and only a launch that
@@ -502,7 +537,7 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
       if (sm < S->pol.idle_first || sm >= S->pol.idle_first + S->pol.idle_count) S->sm_mask[sm >> 5] |= 1u << (sm & 31);
   }
   fill_info(S, comm->R);
-  flatten(S, comm->dtype);
+  if (!S->flat) flatten(S, comm->dtype);
   if (!comm->planner) {
     st = upload(S, comm->R);
     if (st != PL_OK) {
@@ -831,7 +866,7 @@ pl_status_t pl_comm_reset(pl_comm_t comm, void* stream) {
   if (cudaMemsetAsync(comm->d_status, 0, kStatusWords * sizeof(int), st) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
   std::lock_guard<std::mutex> g(comm->mu);
   for (pl_schedule_s* S : comm->schedules) {
-    if (S->d_blob && cudaMemsetAsync(S->d_blob + S->off_flags, 0, S->sync_bytes, st) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
+    if (S->d_blob && S->sync_bytes && cudaMemsetAsync(S->d_blob + S->off_flags, 0, S->sync_bytes, st) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
     // packet tags restart with the epoch: old packets must not match them
     if (S->packet_ctas_per_rank && S->d_scratch && cudaMemsetAsync(S->d_scratch, 0, S->scratch_total, st) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
   }
@@ -1077,9 +1112,32 @@ pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
     g_launches.fetch_add(1);
     return PL_OK;
   }
+  const int R = s->comm->R;
+  if (s->flat) {
+    FlatParams F;
+    for (int r = 0; r < R; ++r) {
+      F.in[r] = bufs->in[r];
+      F.out[r] = bufs->out[r];
+      F.aux[r] = s->info.aux_bytes[r] ? bufs->aux[r] : nullptr;
+    }
+    F.spans = reinterpret_cast<const FlatSpan*>(s->d_blob);
+    F.n_spans = (uint32_t)s->flat_spans.size();
+    F.tile = s->flat_launch.tile;
+    F.n_ranks = R;
+    F.hook = s->hook;
+    F.hints = s->no_l2_hints ? 0u : (2u | (s->inputs_last_use ? 1u : 0u));
+    F.out_scale = s->out_scale;
+    F.status = s->comm->d_status;
+    F.timeout_ns = s->timeout_ns;
+    if (launch_flat(s->comm->dtype, F, s->flat_launch, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
+      cudaGetLastError();
+      return PL_ERR_CUDA;
+    }
+    g_launches.fetch_add(1);
+    return PL_OK;
+  }
   ExecParams P;
   std::memset(&P, 0, sizeof(P));
-  const int R = s->comm->R;
   for (int r = 0; r < R; ++r) {
     P.base[kSlotIn + r] = const_cast<void*>(bufs->in[r]);
     P.base[kSlotOut + r] = bufs->out[r];

@@ -107,6 +107,36 @@ struct ExecParams {
   uint32_t pipelined_reduce;  // host side only: every reduce op is plain (element-typed operands), use the 12-warp variant
 };
 
+// ---- flat execution of a schedule without flags (pl_datapath_flat.cu) ------------------------
+constexpr int kFlatThreads = 256, kFlatBulkThreads = 128;
+// A run of units (16 bytes of every operand): a copy from one rank's input, or the sum of every
+// rank's input at one offset in ascending rank order, to one rank's output or to all of them.
+struct alignas(16) FlatSpan {
+  uint64_t src_off, dst_off;  // units into the input(s) / into the output(s)
+  uint64_t units;
+  uint32_t first_block;       // CTAs of the spans in front
+  uint32_t ranks;             // source rank | destination rank << 8, 255 = every rank
+};
+static_assert(sizeof(FlatSpan) == 32, "FlatSpan layout");
+struct FlatParams {
+  const void* in[PL_MAX_RANKS];
+  void* out[PL_MAX_RANKS];
+  const void* aux[PL_MAX_RANKS];
+  const FlatSpan* spans;
+  uint32_t n_spans, tile;  // tile: units per CTA
+  int n_ranks;
+  uint32_t hook, hints;    // as in ExecParams
+  float out_scale;
+  int* status;
+  unsigned long long timeout_ns;
+};
+struct FlatLaunch {  // host side: which kernel, how many CTAs
+  bool reduce, all, bulk;  // all: every rank is a destination
+  int units = 1;           // units per thread of a register copy
+  uint32_t tile, blocks = 0, smem_bytes;
+  int threads;
+};
+
 // What the layer executor needs on top of ExecParams (see pl_datapath_layers.cu): the distance from
 // a layer's operands to the next layer's, in bytes.
 struct LayerParams {
@@ -190,6 +220,9 @@ int level_width(const Lowered& L, int R);
 // bulk_datapath: the schedule runs on the bulk-copy executor, where program order on one queue
 // orders less than on the register executor (see validate()).
 pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapath);
+// The ops of a schedule without flags as spans; false if they are not of the forms a span describes.
+// `reduce` / `all` receive the one kind of op the schedule holds.  first_block is left to the caller.
+bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all);
 LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster);
 Policy default_policy(const BuildRequest& rq, int max_resident_ctas);
 

@@ -24,6 +24,10 @@ size_t exec_tma_smem_bytes(int stages, uint32_t stage_bytes);
 cudaError_t launch_layers(int dtype, const ExecParams& P, const LayerParams& Y, int grid, int threads, bool cluster, cudaStream_t stream);
 bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads);
 
+// schedules without flags, one CTA per tile
+FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units);
+cudaError_t launch_flat(int dtype, const FlatParams& P, const FlatLaunch& F, cudaStream_t stream);
+
 // packet executor (latency path): rank = cluster of ctas_per_rank CTAs
 cudaError_t launch_exec_packet(int dtype, const PacketParams& P, int threads, bool overlap, cudaStream_t stream);
 int exec_packet_max_groups(int dtype, int ctas_per_rank, int threads);

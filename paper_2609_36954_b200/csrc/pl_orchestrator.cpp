@@ -1227,6 +1227,42 @@ void assign_queues(Lowered* L, int R, int n_queues, bool by_level) {
   }
 }
 
+bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all) {
+  spans->clear();
+  if (L.ops.empty() || L.n_flags != 0) return false;
+  *reduce = L.ops[0].kind == PL_OP_REDUCE;
+  *all = L.ops[0].bcast;
+  // runs by (ranks, distance from source to destination), in the order in which the ops name them
+  std::map<std::pair<uint32_t, int64_t>, size_t> group_of;
+  std::vector<std::vector<FlatSpan>> groups;
+  for (const HostOp& op : L.ops) {
+    if (op.kind != (*reduce ? PL_OP_REDUCE : PL_OP_COPY) || op.bcast != *all || op.dst.buf != PL_BUF_OUT) return false;
+    const uint64_t unit = *reduce ? 16 / elem_size(dtype) : 16;  // elements (bytes of a copy) per unit
+    const uint64_t out_b = *reduce ? unit * elem_size(op.dst.dtype) : 16;
+    if (op.src.size() != (*reduce ? (size_t)R : 1u)) return false;
+    for (size_t k = 0; k < op.src.size(); ++k) {
+      const pl_ref_t& s = op.src[k];
+      if (s.buf != PL_BUF_IN || s.offset != op.src[0].offset) return false;
+      if (*reduce && (s.rank != (int)k || s.dtype != dtype)) return false;
+    }
+    if (op.count % unit || op.src[0].offset % 16 || op.dst.offset % out_b) return false;
+    if (op.count == 0) continue;
+    const FlatSpan f{op.src[0].offset / 16, op.dst.offset / out_b, op.count / unit, 0,
+                     (*reduce ? 255u : (uint32_t)op.src[0].rank) | (*all ? 255u : (uint32_t)op.dst.rank) << 8};
+    const auto at = group_of.emplace(std::make_pair(f.ranks, (int64_t)(f.dst_off - f.src_off)), groups.size());
+    if (at.second) groups.emplace_back();
+    groups[at.first->second].push_back(f);
+  }
+  for (auto& g : groups) {
+    std::sort(g.begin(), g.end(), [](const FlatSpan& a, const FlatSpan& b) { return a.src_off < b.src_off; });
+    for (const FlatSpan& f : g) {
+      if (&f != &g[0] && spans->back().src_off + spans->back().units == f.src_off) spans->back().units += f.units;
+      else spans->push_back(f);
+    }
+  }
+  return !spans->empty();
+}
+
 int level_width(const Lowered& L, int R) {
   // level of an op = length of the longest chain of flag edges that ends in it
   std::vector<int> flag_level(L.n_flags, 0);

@@ -1,0 +1,87 @@
+"""Schedules without flags with everything left to the library (one CTA per tile, no queues) against
+the same schedule on the op queues: the same bits, at the edges of tiles, in both forms."""
+import pytest
+import torch
+
+from gpu_harness import DT, stream_handle
+from paper_2609_36954_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+SIZE = {"bf16": 2, "f32": 4, "i32": 4, "u8": 1}
+MIB = 1 << 20
+
+
+def values(nbytes, dtype, gen):
+    if dtype in ("bf16", "f32"):
+        return torch.randn(nbytes // SIZE[dtype], generator=gen, device="cuda").to({"bf16": torch.bfloat16, "f32": torch.float32}[dtype])
+    return torch.randint(0, 256, (nbytes,), generator=gen, device="cuda", dtype=torch.uint8)
+
+
+def same_bits(R, dtype, build, **both):
+    """`build` makes a schedule from (comm, opts); runs it flat and on the queues, compares all outputs."""
+    comm = B.pl_comm_create(R, DT[dtype])
+    flat, queues = build(comm, B.make_opts(**both)), build(comm, B.make_opts(datapath=B.PL_DP_LDST, **both))
+    try:
+        info = B.pl_schedule_info(flat)
+        gen = torch.Generator(device="cuda").manual_seed(3)
+        sizes = [[int(a[r]) for r in range(R)] for a in (info.in_bytes, info.out_bytes, info.aux_bytes)]
+        ins = [values(max(16, n), dtype, gen) for n in sizes[0]]
+        aux = [values(max(16, n), dtype, gen) for n in sizes[2]]
+        outs = []
+        for s in (flat, queues):
+            out = [torch.full((max(16, n) + 16,), 0x5A, dtype=torch.uint8, device="cuda") for n in sizes[1]]
+            bufs = B.make_bufs([t.data_ptr() for t in ins], [t.data_ptr() for t in out], sizes[0], sizes[1], [t.data_ptr() for t in aux], sizes[2])
+            for _ in range(2):
+                B.pl_execute(s, bufs, stream_handle())
+            torch.cuda.synchronize()
+            outs.append(out)
+        assert B.pl_comm_status(comm).code == B.PL_OK
+        for r in range(R):
+            assert torch.equal(outs[0][r], outs[1][r]), r   # the 16 bytes behind the output included
+            assert bool((outs[0][r][sizes[1][r]:] == 0x5A).all())
+        return info
+    finally:
+        B.pl_schedule_destroy(flat)
+        B.pl_schedule_destroy(queues)
+        B.pl_comm_destroy(comm)
+
+
+# units (16 bytes) of a partition: a single one, around 128, 256 and 512 (tiles of the forms), and
+# sizes that stream (bulk-copy form) with a ragged end
+@pytest.mark.parametrize("R,dtype", [(2, "f32"), (3, "bf16"), (4, "i32"), (5, "f32"), (8, "bf16"), (16, "bf16"), (16, "f32")])
+@pytest.mark.parametrize("units", [1, 127, 129, 257, 1025, "stream"])
+def test_fixed_size_collectives(R, dtype, units):
+    part = 16 * units if units != "stream" else (288 * MIB // (2 * R * R) // 16 + 37) * 16
+    n = part // SIZE[dtype]
+    for coll, algo, count in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n * R), (B.PL_ALLREDUCE, B.PL_ALGO_ONESHOT, n),
+                              (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, n * R), (B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n),
+                              (B.PL_ALLTOALL, B.PL_ALGO_DIRECT, n * R)):
+        for flags in (0, B.PL_OPT_INPUTS_LAST_USE):
+            info = same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, count, 64 * 1024, o), flags=flags)
+        if units == "stream" and algo == B.PL_ALGO_DIRECT_FUSED:
+            assert info.datapath == B.PL_DP_TMA
+
+
+@pytest.mark.parametrize("R,dtype", [(2, "bf16"), (4, "f32"), (8, "bf16"), (8, "f32"), (16, "bf16")])
+@pytest.mark.parametrize("units", [1, 257, "stream"])
+def test_processing_phase(R, dtype, units):
+    part = 16 * units if units != "stream" else (288 * MIB // (2 * R * R) // 16 + 37) * 16
+    n = part // SIZE[dtype] * R
+    hooks = [B.PL_HOOK_RESIDUAL] + ([B.PL_HOOK_F32_OUT, B.PL_HOOK_RESIDUAL | B.PL_HOOK_F32_OUT] if dtype == "bf16" else [])
+    for hook in hooks:
+        for coll, algo in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED), (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT)):
+            same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, n, 64 * 1024, o), hook=hook, out_scale=0.375)
+
+
+@pytest.mark.parametrize("scale", [1, 3000])
+def test_variable_sizes_and_rooted(scale):
+    R = 8
+    counts = [[0 if (p + r) % 3 == 0 else 8 * (1 + (5 * p + 11 * r) % 67) * scale for r in range(R)] for p in range(R)]
+    same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, counts, 4096, o))
+    for coll in (B.PL_ALLGATHERV, B.PL_REDUCE_SCATTERV):
+        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_v(c, coll, B.PL_ALGO_DIRECT, counts[2], 4096, o))
+    for coll in (B.PL_BROADCAST, B.PL_REDUCE, B.PL_SCATTER, B.PL_GATHER):
+        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_rooted(c, coll, 5, 8 * R * 77 * scale, 4096, o))
+    # 256 spans, those between different ranks a single vector
+    one = [[8 if p != r else 8 * 50 * scale for r in range(16)] for p in range(16)]
+    same_bits(16, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, one, 4096, o))
