@@ -362,8 +362,15 @@ def pl_comm_host_sync(comm):
     _check(load().pl_comm_host_sync(comm), "pl_comm_host_sync")
 
 
+_ptr_types = {n: C.c_void_p * n for n in range(1, PL_MAX_RANKS + 1)}  # building the type costs more than filling it
+
+
 def _ptr_array(addrs):
-    return (C.c_void_p * len(addrs))(*[int(a) if a else None for a in addrs])
+    T = _ptr_types.get(len(addrs)) or C.c_void_p * len(addrs)
+    try:
+        return T(*addrs)  # plain ints and None
+    except TypeError:
+        return T(*[int(a) if a else None for a in addrs])
 
 
 def pl_moe_plan_create(comm, tokens_per_rank, hidden, n_experts, topk, recv_capacity_rows):

@@ -6,7 +6,8 @@
 // source rank: exclusive prefix sums over its blocks, totals per expert and destination) ->
 // place (segment bases in (source rank, expert, token) order, row index of every
 // (token, slot), receive metadata) -> move (each token row is read once into
-// shared memory by a bulk async copy and written to its K destinations by K bulk stores).
+// shared memory by a bulk async copy and written to its K destinations by K bulk stores);
+// with up to 1024 routing entries per source all of it in one launch (moe_small_kernel).
 // combine = gate-weighted fp32 sum of the K expert rows of every token, ascending slot.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -27,7 +28,7 @@ namespace {
 constexpr int kTB = 256;             // tokens per count/place block
 constexpr int kMaskWords = kTB / 32;
 constexpr int kMaxTopk = 32;
-constexpr uint32_t kMaxTile = 16384;  // bytes of a row moved per bulk copy
+constexpr int kCombineThreads = 256, kCombinePartThreads = 128;
 
 struct DispatchPtrs {
   const void* x[PL_MAX_RANKS];
@@ -42,8 +43,8 @@ struct CombinePtrs {
 };
 struct MoeGeo {
   int R, T, E, K, NB, epr;
-  uint32_t row_bytes, tile_bytes, n_tiles, slots;
-  uint32_t rows_per_item, slot_bytes;  // mover: consecutive token rows per bulk load, bytes per ring slot
+  uint32_t row_bytes;
+  uint32_t move_rows, move_parts;  // mover: token rows per tile, or tiles per row
   unsigned long long cap;
   int32_t* blockcnt;   // [R][NB][E]: per-block counts, turned into exclusive block offsets by scan
   long long* counts;   // [R][R]
@@ -53,6 +54,7 @@ struct MoeGeo {
   int* flags;          // [0] overflow, [1] invalid expert id, [2] copy engine wait gave up, [3] grid barrier gave up (sticky)
   unsigned int* sync;  // fused bookkeeping: [0] CTAs that reached the grid barrier, [1] CTAs that left the kernel
   const int32_t* slotmask;  // optional [R][T][K]: written into the metadata instead of the slot index
+  int epr_shift;            // log2(epr), -1 if it is no power of two
   int gates_are_logits;     // combine: the gate input holds the K selected logits; softmax them first
 };
 
@@ -359,127 +361,376 @@ __global__ void __launch_bounds__(256) moe_derive_ranks_kernel(const __grid_cons
   }
 }
 
-// One warp per CTA drives a ring of `slots` shared-memory tiles: lane 0 issues the bulk loads
-// (prime, then refill as tiles drain: the paper's Algorithm 2 with the processing step being
-// "store to K places"), the lanes share the bulk stores.  A work item is a group of `rows`
-// consecutive token rows of one source rank, which are contiguous in its input: one bulk load of
-// up to 56 KiB, then rows x K bulk stores of one row each (rows wider than 16 KiB are moved in
-// tiles, one row per item).  The write-dominated stream this kernel is runs fastest with large
-// loads and 128-136 CTAs on this GPU (1 read : 8 writes through the same ring: 6.15-6.3 TB/s with
-// 128-136 CTAs and 32-64 KiB tiles, 5.65-5.73 TB/s with 140-148 CTAs, 5.55 TB/s with 296 CTAs and
-// 14 KiB tiles), so the grid is a property of the GPU's memory system, not of the row count.
-__global__ void __launch_bounds__(32) moe_move_kernel(const __grid_constant__ DispatchPtrs P, const __grid_constant__ MoeGeo g) {
+// ---- small dispatches in one launch --------------------------------------------------------
+// A CTA takes `rows` consecutive tokens of one source rank: it asks for their rows first, works out
+// where its own rows go from the routing of everybody while they travel, and stores them.
+// Each CTA reads all routing in front of its own (16 KiB of indices at 8 x 64 tokens x 8 slots),
+// so nothing is counted, published and read back between launches or across a grid barrier.  A
+// dispatch of this size is bound by its chain (indices from DRAM, counting, rows out) and by the
+// launches (B200, R = 8, 7168 x bf16, top-8, two launches -> one: 1 token per rank 15.6 -> 6.4 us,
+// 64 tokens 25.4 -> 18 us; deduplicated 31 -> 16 us).  The line lies where a CTA's share of the
+// routing costs more than the grid barrier (256 tokens: 57 us in two launches, 70 us in one).
+// The row of (p, t, j) at rank r = entries of sources before p that go to r, plus entries of p that
+// go to r with a lower expert, or with the same expert and an earlier token.
+// DEDUP: an entry is (token, destination rank); the row is the number of earlier tokens, over
+// sources and then tokens, with a slot on r.
+constexpr int kSmallThreads = 256;
+constexpr int kSmallOwn = 1024;       // most entries (T x K) of a source in a plan dispatched this way
+constexpr int kSmallExperts = 1024;
+constexpr int kSmallTargets = 64;     // most (token, slot) pairs of one CTA
+
+struct SmallParams {
+  uint32_t rows;            // tokens per CTA
+  int K0, epr0;             // DEDUP: slots per token and experts per rank of the routing
+  int32_t* ridx;            // DEDUP: distinct destination ranks per token, padded with -1, and the slots on each
+  int32_t* rmask;
+};
+
+// Bounded wait for the first phase of `bar` (a CTA's rows have landed).
+__device__ __forceinline__ bool wait_rows(uint64_t* bar) {
+  if (ptx::mbar_try_wait(bar, 0)) return true;
+  unsigned long long t0, t1;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+  for (uint32_t tries = 1;; ++tries) {
+    if (ptx::mbar_try_wait(bar, 0)) return true;
+    if ((tries & 1023u) == 0) {
+      asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
+      if (t1 - t0 > 2000000000ull) return false;
+    }
+  }
+}
+// Adds one to rank r's 8-bit field (r < 16); a thread adds at most 255 entries.
+__device__ __forceinline__ void count_rank(unsigned long long (&c)[2], int r) {
+  const unsigned long long one = 1ull << ((r & 7) * 8);
+  if (r < 8) c[0] += one;
+  else c[1] += one;
+}
+// Sums the CTA's per-thread fields into s_cnt[16] (zeroed, a barrier before the call; none after).
+__device__ __forceinline__ void sum_ranks(const unsigned long long (&c)[2], int R, int32_t* s_cnt) {
+  const unsigned long long m = 0x00FF00FF00FF00FFull;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (h * 8 >= R) break;
+    unsigned long long even = c[h] & m, odd = (c[h] >> 8) & m;  // 16-bit fields: a warp's 32 x 255 fit
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+      even += __shfl_xor_sync(0xFFFFFFFFu, even, d);
+      odd += __shfl_xor_sync(0xFFFFFFFFu, odd, d);
+    }
+    const int lane = threadIdx.x & 31;
+    if (lane < 8) {
+      const int v = (int)(((lane & 1 ? odd : even) >> ((lane >> 1) * 16)) & 0xFFFFull);
+      if (v) atomicAdd(&s_cnt[h * 8 + lane], v);
+    }
+  }
+}
+// Ranks that token `idx` (K slots) sends to, as a bit mask (dropping slots that name no expert).
+__device__ __forceinline__ uint32_t rank_set(const int32_t* idx, int K, int epr, int R) {
+  uint32_t set = 0;
+  for (int j0 = 0; j0 < K; j0 += 8) {
+    int ev[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < K) ? __ldg(&idx[j0 + k]) : -1;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (ev[k] >= 0 && ev[k] < epr * R) set |= 1u << (ev[k] / epr);
+  }
+  return set;
+}
+
+template <bool DEDUP>
+__global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_constant__ DispatchPtrs P, const __grid_constant__ MoeGeo g,
+                                                                  const __grid_constant__ SmallParams Q) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const int lane = threadIdx.x;
-  const uint32_t S = g.slots;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
-  unsigned char* tiles = smem + 128;
-  if (lane == 0) {
-    for (uint32_t s = 0; s < S; ++s) ptx::mbar_init(full + s, 1);
+  unsigned char* tile = smem + 128;
+  __shared__ int32_t s_cnt[16], s_total[16];
+  __shared__ int32_t s_before[kSmallTargets];          // per target: this source's rows in front of it
+  __shared__ int32_t s_set[kSmallTargets];             // DEDUP: rank sets of the CTA's tokens
+  __shared__ int32_t s_own[DEDUP ? 1 : kSmallOwn];     // the source's routing
+  __shared__ int32_t s_hist[DEDUP ? 1 : kSmallExperts];
+  __shared__ int s_bad;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, R = g.R, T = g.T, K = DEDUP ? Q.K0 : g.K, TK = T * K;
+  const uint32_t groups = ((uint32_t)T + Q.rows - 1) / Q.rows;
+  const int p = (int)(blockIdx.x / groups), t0 = (int)((blockIdx.x - (uint32_t)p * groups) * Q.rows);
+  const int nrows = min((int)Q.rows, T - t0), Kd = g.K, n_tgt = nrows * Kd;  // Kd: entries per token (DEDUP: ranks)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid < 16) s_cnt[tid] = s_total[tid] = 0;
+  if (tid == 0) {
+    s_bad = 0;
+    ptx::mbar_init(full, 1);
     ptx::mbar_init_fence();
   }
-  __syncwarp();
-  // launched with programmatic stream serialization: set up above while the bookkeeping kernel
-  // drains, wait here for it to complete before anything it wrote (pos, prank) is read
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const uint32_t rows = g.rows_per_item;  // > 1 only when a row is one tile
-  const unsigned long long groups_per_rank = ((unsigned long long)g.T + rows - 1) / rows;
-  const unsigned long long n_items = (unsigned long long)g.R * groups_per_rank * g.n_tiles;
-  const unsigned long long c = blockIdx.x, G = gridDim.x;
-  if (c >= n_items) return;
-  const unsigned long long n_my = (n_items - c + G - 1) / G;
-  constexpr int L = 2;  // store groups allowed to be still reading shared memory
-
-  // item n of this CTA: tokens [tok, tok + nrows) of one rank, bytes [off, off + bytes) of each row
-  auto item = [&](unsigned long long n, unsigned long long& tok, uint32_t& nrows, uint32_t& off, uint32_t& bytes) {
-    const unsigned long long w = c + n * G;
-    const unsigned long long grp = w / g.n_tiles;
-    const uint32_t tile = (uint32_t)(w % g.n_tiles);
-    const unsigned long long p = grp / groups_per_rank, t0 = (grp % groups_per_rank) * rows;
-    tok = p * g.T + t0;
-    nrows = (uint32_t)min((unsigned long long)rows, (unsigned long long)g.T - t0);
-    off = tile * g.tile_bytes;
-    bytes = (rows > 1) ? g.row_bytes : min(g.tile_bytes, g.row_bytes - off);
-  };
-  auto issue_load = [&](unsigned long long n) {
-    unsigned long long tok;
-    uint32_t nrows, off, bytes;
-    item(n, tok, nrows, off, bytes);
-    const int p = (int)(tok / g.T);
-    const unsigned long long t = tok % g.T;
-    const char* src = static_cast<const char*>(P.x[p]) + t * g.row_bytes + off;
-    const uint32_t s = (uint32_t)(n % S);
-    ptx::mbar_expect_tx(full + s, nrows * bytes);
-    ptx::bulk_g2s_hint(tiles + (size_t)s * g.slot_bytes, src, nrows * bytes, full + s, ptx::policy_evict_first());
-  };
-
-  unsigned long long issued = 0;
-  if (lane == 0)
-    for (; issued < n_my && issued < S; ++issued) issue_load(issued);
-  issued = min(n_my, (unsigned long long)S);
-  bool failed = false;
-  unsigned long long n = 0;
-  for (; n < n_my; ++n) {
-    unsigned long long tok;
-    uint32_t nrows, off, bytes;
-    item(n, tok, nrows, off, bytes);
-    // this lane's first store of the item: (row i of the group, slot j); fetched before the wait
-    const uint32_t n_st = nrows * (uint32_t)g.K;
-    int row = -1, r = 0;
-    if ((uint32_t)lane < n_st) {
-      row = g.pos[tok * g.K + lane];
-      r = g.prank[tok * g.K + lane];
+  if (tid == 0) {
+    const uint32_t bytes = (uint32_t)nrows * g.row_bytes;
+    ptx::mbar_expect_tx(full, bytes);
+    ptx::bulk_g2s_hint(tile, static_cast<const char*>(P.x[p]) + (size_t)t0 * g.row_bytes, bytes, full, ptx::policy_evict_first());
+  }
+  const int32_t* own = P.idx[p];
+  auto rank_of = [&](int e) { return g.epr_shift >= 0 ? e >> g.epr_shift : e / g.epr; };
+  // entries per rank of the sources [0, n), in this thread's 8-bit fields
+  auto count_sources = [&](int n, unsigned long long (&into)[2], bool check) {
+    bool vec = (TK & 3) == 0;
+    for (int q = 0; q < n; ++q) vec = vec && ((uintptr_t)P.idx[q] & 15) == 0;
+    if (vec) {  // 16 bytes at a time, over all sources
+      const int nv = TK >> 2, all = n * nv;
+      for (int i0 = tid; i0 < all; i0 += 4 * kSmallThreads) {
+        int4 ev[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int i = i0 + k * kSmallThreads, q = i / nv;
+          ev[k] = i < all ? __ldg(reinterpret_cast<const int4*>(P.idx[q]) + (i - q * nv)) : make_int4(-1, -1, -1, -1);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const int e = m == 0 ? ev[k].x : m == 1 ? ev[k].y : m == 2 ? ev[k].z : ev[k].w;
+            if ((unsigned)e < (unsigned)g.E) count_rank(into, rank_of(e));
+            else if (check && e >= 0) s_bad = 1;
+          }
+      }
+      return;
     }
-    const uint32_t s = (uint32_t)(n % S), parity = (uint32_t)((n / S) & 1);
-    // bounded wait for the tile to land
-    bool ok = ptx::mbar_try_wait(full + s, parity);
-    if (!ok) {
-      unsigned long long t0 = 0;
-      asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-      for (uint32_t tries = 1; !(ok = ptx::mbar_try_wait(full + s, parity)); ++tries) {
-        if ((tries & 1023u) == 0) {
-          unsigned long long t1;
-          asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
-          if (t1 - t0 > 2000000000ull) break;
+    for (int i = tid; i < TK; i += kSmallThreads)
+      for (int q0 = 0; q0 < n; q0 += 8) {
+        int ev[8];  // independent loads: one L2 latency per batch
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ev[k] = (q0 + k < n) ? __ldg(&P.idx[q0 + k][i]) : -1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if ((unsigned)ev[k] < (unsigned)g.E) count_rank(into, rank_of(ev[k]));
+          else if (check && ev[k] >= 0) s_bad = 1;
         }
       }
+  };
+  auto count_tokens = [&](int from, int to, unsigned long long (&into)[2]) {  // DEDUP: tokens numbered over the sources
+    for (int i = from + tid; i < to; i += kSmallThreads) {
+      const int q = i / T;
+      for (uint32_t set = rank_set(P.idx[q] + (size_t)(i - q * T) * K, K, Q.epr0, R); set; set &= set - 1) count_rank(into, __ffs(set) - 1);
     }
-    ok = __all_sync(0xFFFFFFFFu, ok);
-    if (!ok) { failed = true; break; }
-    // every token row is read once and every received row written once: both stream through L2
-    const unsigned char* tile = tiles + (size_t)s * g.slot_bytes;
-    for (uint32_t idx = lane; idx < n_st; idx += 32) {
-      if (idx >= 32) {
-        row = g.pos[tok * g.K + idx];
-        r = g.prank[tok * g.K + idx];
+  };
+  // ---- what goes to each rank in front of this CTA's tokens
+  unsigned long long c[2] = {0ull, 0ull};
+  if constexpr (DEDUP) {
+    if (tid < nrows) s_set[tid] = (int32_t)rank_set(own + (size_t)(t0 + tid) * K, K, Q.epr0, R);
+    count_tokens(0, p * T + t0, c);
+  } else {
+    for (int i = tid; i < TK; i += kSmallThreads) s_own[i] = __ldg(&own[i]);
+    count_sources(p, c, false);
+  }
+  __syncthreads();
+  sum_ranks(c, R, s_cnt);
+  if constexpr (!DEDUP) {
+    // this source's entries in front of each target: lower expert of the rank, or same expert and
+    // an earlier token.  Warp w takes targets w, w + 8, ...; its lanes share the entries.
+    for (int k = warp; k < n_tgt; k += kSmallThreads / 32) {
+      const int t = t0 + k / K, e = s_own[t0 * K + k];
+      if ((unsigned)e >= (unsigned)g.E) continue;
+      const int lo = rank_of(e) * g.epr;  // first expert of the rank
+      int n = 0;
+#pragma unroll 4
+      for (int i = lane; i < TK; i += 32) {
+        const int o = s_own[i];
+        n += (o >= lo && (o < e || (o == e && i < t * K))) ? 1 : 0;
       }
-      if (row >= 0)
-        ptx::bulk_s2g_hint(static_cast<char*>(P.recv[r]) + (size_t)row * g.row_bytes + off,
-                           tile + (size_t)(idx / (uint32_t)g.K) * bytes, bytes, ptx::policy_evict_first());
-    }
-    ptx::bulk_commit();
-    if (n >= (unsigned long long)L) {
-      ptx::bulk_wait_read<L>();
-      __syncwarp();
-      const unsigned long long m = n - L;  // its tile is no longer being read
-      if (lane == 0 && m + S < n_my) issue_load(m + S);
+      n = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)n);
+      if (lane == 0) s_before[k] = n;
     }
   }
-  ptx::bulk_wait<0>();
-  if (failed && lane == 0) {
-    g.flags[2] = 1;
-    // loads already issued may still land: give each a bounded chance before leaving
-    const unsigned long long last = min(n_my, n + S);
-    for (unsigned long long k = n; k < last; ++k) {
-      const uint32_t s = (uint32_t)(k % S), parity = (uint32_t)((k / S) & 1);
-      for (uint32_t tries = 0; tries < (1u << 20) && !ptx::mbar_try_wait(full + s, parity); ++tries) {}
+  __syncthreads();
+  // ---- place: thread k owns target k
+  int row = -1, r = 0, src = 0, meta_j = 0, meta_e = 0;
+  if (tid < n_tgt) {
+    src = tid / Kd;
+    const int j = tid - src * Kd, t = t0 + src;
+    bool live;
+    if constexpr (DEDUP) {
+      uint32_t set = (uint32_t)s_set[src], mask = 0;
+      for (int k = 0; k < j; ++k) set &= set - 1;
+      live = set != 0;
+      if (live) {
+        r = __ffs(set) - 1;
+        row = s_cnt[r];
+        for (int k = 0; k < src; ++k) row += (int)(((uint32_t)s_set[k] >> r) & 1u);
+        for (int k = 0; k < K; ++k) {
+          const int e = __ldg(&own[(size_t)t * K + k]);
+          if (e >= 0 && e / Q.epr0 == r) mask |= 1u << k;
+        }
+      }
+      const size_t o = ((size_t)p * T + t) * Kd + j;
+      Q.ridx[o] = live ? r : -1;
+      Q.rmask[o] = (int32_t)mask;
+      meta_j = (int)mask;
+      meta_e = r;
+    } else {
+      meta_j = j;
+      meta_e = s_own[t * K + j];
+      live = (unsigned)meta_e < (unsigned)g.E;
+      if (live) {
+        r = rank_of(meta_e);
+        row = s_cnt[r] + s_before[tid];
+      }
+    }
+    if (live && (unsigned long long)row >= g.cap) row = -1;
+  }
+  // ---- the rows have landed (bounded wait): one bulk store per target
+  bool ok = true;
+  if (tid < n_tgt) {
+    ok = wait_rows(full);
+    if (ok && row >= 0) {
+      ptx::bulk_s2g_hint(static_cast<char*>(P.recv[r]) + (size_t)row * g.row_bytes, tile + (size_t)src * g.row_bytes, g.row_bytes, ptx::policy_evict_first());
+      ptx::bulk_commit();
+    }
+    // bookkeeping while the rows leave
+    const size_t o = ((size_t)p * T + t0 + src) * Kd + (tid - src * Kd);
+    g.pos[o] = row;
+    g.prank[o] = r;
+    if (row >= 0 && P.meta[r]) reinterpret_cast<int4*>(P.meta[r])[row] = make_int4(p, t0 + src, meta_j, meta_e);
+  }
+  if (t0 == 0) {  // this source's counts
+    if constexpr (DEDUP) {
+      unsigned long long d[2] = {0ull, 0ull};
+      count_tokens(p * T, (p + 1) * T, d);
+      sum_ranks(d, R, s_total);
+      __syncthreads();
+      if (tid < R) g.counts[p * R + tid] = g.ecounts[p * R + tid] = s_total[tid];
+      __syncthreads();
+      if (tid < 16) s_total[tid] = 0;
+    } else {
+      for (int e = tid; e < g.E; e += kSmallThreads) s_hist[e] = 0;
+      __syncthreads();
+      for (int i = tid; i < TK; i += kSmallThreads) {
+        const int e = s_own[i];
+        if ((unsigned)e < (unsigned)g.E) atomicAdd(&s_hist[e], 1);
+      }
+      __syncthreads();
+      for (int e = tid; e < g.E; e += kSmallThreads) g.ecounts[(size_t)p * g.E + e] = s_hist[e];
+      if (tid < R) {
+        long long n = 0;
+        for (int e = tid * g.epr; e < (tid + 1) * g.epr; ++e) n += s_hist[e];
+        g.counts[p * R + tid] = n;
+      }
+    }
+  }
+  if (blockIdx.x == 0) {  // the whole routing: does every rank's share fit, does every slot name an expert
+    __syncthreads();
+    unsigned long long d[2] = {0ull, 0ull};
+    if constexpr (DEDUP) count_tokens(0, R * T, d);
+    else count_sources(R, d, true);
+    sum_ranks(d, R, s_total);
+    __syncthreads();
+    if (tid == 0) {
+      int over = 0;
+      for (int q = 0; q < R; ++q) over |= (unsigned long long)s_total[q] > g.cap;
+      g.flags[0] = over;
+      g.flags[1] = s_bad;
+      g.flags[2] = 0;
+    }
+  }
+  if (tid < n_tgt) {
+    ptx::bulk_wait<0>();
+    if (!ok) {
+      g.flags[3] = 1;  // reported and cleared by the next read of the plan
+      ptx::mbar_wait_bounded(full, 0, 1u << 20);
     }
   }
 }
 
+// ---- rows to their destinations ---------------------------------------------------------------
+// A CTA of one warp moves one tile: a part of a token's row, or `rows` consecutive short rows of one
+// source (contiguous in its input).  One bulk load, then a bulk store per destination.  Bound by HBM
+// (1 read : K writes); the order in which the tiles are dealt keeps all SMs inside one window of
+// the input, and tiles of 2 KiB were served best (8 x 4096 tokens of 14,336 bytes, top-8, whole
+// dispatch: 660 us; 3584 bytes 684, 7168 bytes 667, whole rows 666; a persistent ring of 56 KiB
+// loads on 132 SMs 742).
+constexpr uint32_t kMoveTile = 2048;
+__global__ void __launch_bounds__(32) moe_move_kernel(const __grid_constant__ DispatchPtrs P, const __grid_constant__ MoeGeo g) {
+  __shared__ __align__(128) unsigned char tile[kMoveTile];
+  __shared__ uint64_t full;
+  const uint32_t lane = threadIdx.x, T = (uint32_t)g.T, K = (uint32_t)g.K;
+  uint32_t p, t, nrows = 1, off = 0, bytes;  // tokens [t, t + nrows) of source p, bytes [off, off + bytes) of each
+  if (g.move_rows > 1) {
+    const uint32_t groups = (T + g.move_rows - 1) / g.move_rows;
+    p = blockIdx.x / groups;
+    t = (blockIdx.x - p * groups) * g.move_rows;
+    nrows = min(g.move_rows, T - t);
+    bytes = g.row_bytes;
+  } else {
+    const uint32_t tok = blockIdx.x / g.move_parts;
+    p = tok / T;
+    t = tok - p * T;
+    off = (blockIdx.x - tok * g.move_parts) * kMoveTile;
+    bytes = min(kMoveTile, g.row_bytes - off);
+  }
+  if (lane == 0) {
+    ptx::mbar_init(&full, 1);
+    ptx::mbar_init_fence();
+    ptx::mbar_expect_tx(&full, nrows * bytes);
+  }
+  __syncwarp();
+  // launched with programmatic stream serialization: wait for the bookkeeping kernel to complete
+  // before anything it wrote (pos, prank) is read
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (lane == 0)
+    ptx::bulk_g2s_hint(tile, static_cast<const char*>(P.x[p]) + (size_t)t * g.row_bytes + off, nrows * bytes, &full, ptx::policy_evict_first());
+  const size_t at = ((size_t)p * T + t) * K;
+  const uint32_t n_st = nrows * K;
+  int row = -1, r = 0;  // this lane's first store, fetched before the wait
+  if (lane < n_st) {
+    row = g.pos[at + lane];
+    r = g.prank[at + lane];
+  }
+  if (!wait_rows(&full)) {
+    g.flags[2] = 1;
+    ptx::mbar_wait_bounded(&full, 0, 1u << 20);
+    return;
+  }
+  for (uint32_t i = lane; i < n_st; i += 32) {
+    if (i >= 32) {
+      row = g.pos[at + i];
+      r = g.prank[at + i];
+    }
+    // every token row is read once and every received row written once: both stream through L2
+    if (row >= 0)
+      ptx::bulk_s2g_hint(static_cast<char*>(P.recv[r]) + (size_t)row * g.row_bytes + off, tile + (size_t)(i / K) * bytes, bytes, ptx::policy_evict_first());
+  }
+  ptx::bulk_commit();
+  ptx::bulk_wait<0>();
+}
+
+// fp32 softmax over a token's K logits (max-subtracted); lane j < K of a warp holds logit j
+__device__ __forceinline__ float softmax_gate(float logit, int K) {
+  const unsigned lanes = (K >= 32) ? 0xFFFFFFFFu : ((1u << K) - 1u);
+  float m = logit;
+  for (int j = 0; j < K; ++j) m = fmaxf(m, __shfl_sync(lanes, logit, j));
+  const float e = expf(logit - m);
+  float sum = 0.f;
+  for (int j = 0; j < K; ++j) sum += __shfl_sync(lanes, e, j);  // ascending slot order on every lane
+  return e / sum;
+}
+__device__ __forceinline__ void add_gated(float (&acc)[8], float gate, const uint4& q) {
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    acc[2 * i] = fmaf(gate, __uint_as_float(w[i] << 16), acc[2 * i]);
+    acc[2 * i + 1] = fmaf(gate, __uint_as_float(w[i] & 0xFFFF0000u), acc[2 * i + 1]);
+  }
+}
+__device__ __forceinline__ uint4 round_row(const float (&acc)[8]) {
+  uint4 o;
+  __nv_bfloat162 a = __floats2bfloat162_rn(acc[0], acc[1]), b = __floats2bfloat162_rn(acc[2], acc[3]);
+  __nv_bfloat162 c = __floats2bfloat162_rn(acc[4], acc[5]), d = __floats2bfloat162_rn(acc[6], acc[7]);
+  o.x = *reinterpret_cast<uint32_t*>(&a);
+  o.y = *reinterpret_cast<uint32_t*>(&b);
+  o.z = *reinterpret_cast<uint32_t*>(&c);
+  o.w = *reinterpret_cast<uint32_t*>(&d);
+  return o;
+}
+
 // combine: CTA per token (grid-strided), 16-byte column units across threads, the K source
 // rows and gates of the next token are fetched while the current one is summed.
-constexpr int kCombineThreads = 256;
 __global__ void __launch_bounds__(kCombineThreads) moe_combine_kernel(const __grid_constant__ CombinePtrs P, const __grid_constant__ MoeGeo g) {
   __shared__ const char* s_row[2][kMaxTopk];
   __shared__ float s_gate[2][kMaxTopk];
@@ -493,19 +744,12 @@ __global__ void __launch_bounds__(kCombineThreads) moe_combine_kernel(const __gr
       const int r = g.prank[tok * g.K + tid];
       s_row[buf][tid] = row >= 0 ? static_cast<const char*>(P.y[r]) + (size_t)row * g.row_bytes : nullptr;
       float gate = P.gates[p][t * g.K + tid];
-      if (g.gates_are_logits) {
-        // fp32 softmax over the token's K logits (max-subtracted); K <= 32 lanes of warp 0
-        const unsigned lanes = (g.K >= 32) ? 0xFFFFFFFFu : ((1u << g.K) - 1u);
-        float m = gate;
-        for (int j = 0; j < g.K; ++j) m = fmaxf(m, __shfl_sync(lanes, gate, j));
-        const float e = expf(gate - m);
-        float sum = 0.f;
-        for (int j = 0; j < g.K; ++j) sum += __shfl_sync(lanes, e, j);  // ascending slot order on every lane
-        gate = e / sum;
-      }
+      if (g.gates_are_logits) gate = softmax_gate(gate, g.K);
       s_gate[buf][tid] = gate;
     }
   };
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   unsigned long long tok = blockIdx.x;
   if (tok < n_tok) load_meta(tok, 0);
   __syncthreads();
@@ -528,30 +772,63 @@ __global__ void __launch_bounds__(kCombineThreads) moe_combine_kernel(const __gr
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          if (j0 + j < g.K) {
-            const float gt = s_gate[buf][j0 + j];
-            const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              acc[2 * i] = fmaf(gt, __uint_as_float(w[i] << 16), acc[2 * i]);
-              acc[2 * i + 1] = fmaf(gt, __uint_as_float(w[i] & 0xFFFF0000u), acc[2 * i + 1]);
-            }
-          }
+          if (j0 + j < g.K) add_gated(acc, s_gate[buf][j0 + j], q[j]);
         }
       }
-      uint4 o;
-      __nv_bfloat162 a = __floats2bfloat162_rn(acc[0], acc[1]);
-      __nv_bfloat162 b = __floats2bfloat162_rn(acc[2], acc[3]);
-      __nv_bfloat162 c2 = __floats2bfloat162_rn(acc[4], acc[5]);
-      __nv_bfloat162 d = __floats2bfloat162_rn(acc[6], acc[7]);
-      o.x = *reinterpret_cast<uint32_t*>(&a);
-      o.y = *reinterpret_cast<uint32_t*>(&b);
-      o.z = *reinterpret_cast<uint32_t*>(&c2);
-      o.w = *reinterpret_cast<uint32_t*>(&d);
-      __stcg(reinterpret_cast<uint4*>(out) + u, o);
+      __stcg(reinterpret_cast<uint4*>(out) + u, round_row(acc));
     }
     __syncthreads();
   }
+}
+
+// The same for few tokens or short rows: CTA per (token, part of the row) or per several tokens of a
+// short row, one 16-byte unit per thread, so that the work divides over the SMs whatever the token
+// count is.  `width` threads (whole warps) work on one token.  KB source rows are loaded at a time:
+// with few slots per token the registers of eight would cost half of the resident CTAs.
+template <int KB>
+__global__ void __launch_bounds__(kCombinePartThreads) moe_combine_parts_kernel(const __grid_constant__ CombinePtrs P, const __grid_constant__ MoeGeo g,
+                                                                                uint32_t parts, uint32_t width) {
+  constexpr int kTokens = kCombinePartThreads / 32;
+  __shared__ const char* s_row[kTokens][kMaxTopk];
+  __shared__ float s_gate[kTokens][kMaxTopk];
+  const uint32_t sub = threadIdx.x / width, tid = threadIdx.x - sub * width;  // token of this CTA, thread of that token
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  uint32_t tok, part = 0;
+  if (parts > 1) {
+    tok = blockIdx.x / parts;
+    part = blockIdx.x - tok * parts;
+  } else {
+    tok = blockIdx.x * (blockDim.x / width) + sub;
+  }
+  const bool live = tok < (uint32_t)g.R * (uint32_t)g.T;
+  const uint32_t p = live ? tok / (uint32_t)g.T : 0u, t = tok - p * (uint32_t)g.T;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (live && tid < (uint32_t)g.K) {
+    const int row = g.pos[(size_t)tok * g.K + tid];
+    const int r = g.prank[(size_t)tok * g.K + tid];
+    float gate = P.gates[p][(size_t)t * g.K + tid];
+    s_row[sub][tid] = row >= 0 ? static_cast<const char*>(P.y[r]) + (size_t)row * g.row_bytes : nullptr;
+    if (g.gates_are_logits) gate = softmax_gate(gate, g.K);
+    s_gate[sub][tid] = gate;
+  }
+  __syncthreads();
+  const uint32_t units = g.row_bytes >> 4, u = part * width + tid;
+  if (!live || u >= units) return;
+  float acc[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+  for (int j0 = 0; j0 < g.K; j0 += KB) {
+    uint4 q[KB];
+#pragma unroll
+    for (int j = 0; j < KB; ++j) {
+      const char* rowp = (j0 + j < g.K) ? s_row[sub][j0 + j] : nullptr;
+      q[j] = rowp ? __ldcg(reinterpret_cast<const uint4*>(rowp) + u) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < KB; ++j)
+      if (j0 + j < g.K) add_gated(acc, s_gate[sub][j0 + j], q[j]);
+  }
+  __stcg(reinterpret_cast<uint4*>(static_cast<char*>(P.out[p]) + (size_t)t * g.row_bytes) + u, round_row(acc));
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -560,7 +837,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // it is raised once per device to the most any plan can ask for, so that creating a second,
 // smaller plan cannot lower it under the feet of the first.
 constexpr int kMaxExperts = 4096;
-constexpr size_t kMoveSmemMax = 227 * 1024;
+constexpr size_t kSmallSmemMax = 64 * 1024;
 constexpr size_t kPlanSmemMax = 200 * 1024;  // the fused bookkeeping kernel is used while its tables fit this
 
 size_t plan_smem_bytes(const MoeGeo& g) {
@@ -570,9 +847,10 @@ bool configure_kernels(int device) {
   static std::atomic<unsigned long long> configured{0};
   const unsigned long long bit = 1ull << (device & 63);
   if (configured.load(std::memory_order_acquire) & bit) return true;
-  if (cudaFuncSetAttribute(moe_move_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMoveSmemMax) != cudaSuccess ||
-      cudaFuncSetAttribute(moe_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxExperts * kMaskWords * 4) != cudaSuccess ||
+  if (cudaFuncSetAttribute(moe_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxExperts * kMaskWords * 4) != cudaSuccess ||
       cudaFuncSetAttribute(moe_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxExperts * kMaskWords * 4 + kMaxExperts * 4) != cudaSuccess ||
+      cudaFuncSetAttribute(moe_small_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemMax) != cudaSuccess ||
+      cudaFuncSetAttribute(moe_small_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemMax) != cudaSuccess ||
       cudaFuncSetAttribute(moe_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlanSmemMax) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -590,8 +868,8 @@ struct pl_moe_plan_s {
   size_t blob_bytes = 0;
   int sm_count = 148;
   int combine_per_sm = 4;  // resident CTAs of the combine kernel per SM (occupancy query at plan creation)
-  size_t move_smem = 0;
   bool fused = false, fused_dedup = false;  // bookkeeping in one launch (grid co-resident, tables fit shared memory)
+  uint32_t small_rows = 0;  // > 0: dispatched in one launch with this many tokens per CTA
   bool dispatched = false;
   // deduplicated variant: the same machinery run over "one expert per rank" routing
   MoeGeo gd{};
@@ -639,20 +917,13 @@ pl_status_t pl_moe_plan_create(pl_comm_t comm, int tokens_per_rank, int hidden, 
   g.K = topk;
   g.NB = (tokens_per_rank + kTB - 1) / kTB;
   g.epr = n_experts / R;
+  g.epr_shift = -1;
+  for (int b = 0; b < 13; ++b)
+    if (g.epr == 1 << b) g.epr_shift = b;
   g.row_bytes = (uint32_t)row_bytes;
-  g.n_tiles = (uint32_t)((row_bytes + kMaxTile - 1) / kMaxTile);
-  g.tile_bytes = (uint32_t)align_up((row_bytes + g.n_tiles - 1) / g.n_tiles, 16);
-  // Rows of at most one tile are moved in groups of consecutive tokens, up to 56 KiB per bulk load,
-  // through exactly three slots: two store groups may still read their tiles while the third tile
-  // is loaded.  Measured at the C4 shape (14,336-byte rows, 8 stores per row): 4 rows x 3 slots
-  // 722-726 us; 4 slots 787 us, 2 or 3 rows per load with 4-6 slots 785-793 us, one row per load
-  // 771 us: the write-dominated stream wants large loads and few bytes in flight.  Wider rows go
-  // tile by tile through at least 4 slots.
-  g.rows_per_item = g.n_tiles == 1 ? (uint32_t)std::max<size_t>(1, std::min<size_t>(32, 57344 / g.tile_bytes)) : 1u;
-  g.slot_bytes = g.rows_per_item * g.tile_bytes;
-  g.slots = g.rows_per_item > 1 ? 3u : (uint32_t)std::min<size_t>(8, std::max<size_t>(4, (96 * 1024) / g.tile_bytes));
+  g.move_rows = (uint32_t)std::max<size_t>(1, std::min<size_t>(32, kMoveTile / row_bytes));
+  g.move_parts = (uint32_t)((row_bytes + kMoveTile - 1) / kMoveTile);
   g.cap = recv_capacity_rows;
-  pl->move_smem = 128 + (size_t)g.slots * g.slot_bytes;
   size_t off = 0;
   auto place = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t o_bc = place((size_t)R * g.NB * g.E * 4);
@@ -681,6 +952,7 @@ pl_status_t pl_moe_plan_create(pl_comm_t comm, int tokens_per_rank, int hidden, 
     d = g;
     d.E = R;
     d.epr = 1;
+    d.epr_shift = 0;
     d.K = std::min(topk, R);
     size_t off2 = 0;
     auto place2 = [&](size_t bytes) { size_t o = off2; off2 = align_up(off2 + bytes, 256); return o; };
@@ -725,6 +997,17 @@ pl_status_t pl_moe_plan_create(pl_comm_t comm, int tokens_per_rank, int hidden, 
     };
     pl->fused = feasible(pl->g);
     pl->fused_dedup = feasible(pl->gd);
+    // One launch while a CTA's share of the routing stays small; rows of one tile only.
+    if ((unsigned long long)tokens_per_rank * topk <= kSmallOwn && n_experts <= kSmallExperts) {
+      for (uint32_t rows = 1; rows * (uint32_t)topk <= kSmallTargets && 128 + rows * row_bytes <= kSmallSmemMax; ++rows) {
+        // the fewest tokens per CTA with which all CTAs are resident at once
+        const unsigned long long per_sm = std::min<unsigned long long>(2048 / kSmallThreads, (220 * 1024) / (rows * row_bytes + 12 * 1024));
+        if ((unsigned long long)R * ((tokens_per_rank + rows - 1) / rows) <= per_sm * comm->sm_count) {
+          pl->small_rows = rows;
+          break;
+        }
+      }
+    }
   }
   comm->n_plans += 1;
   *out = pl;
@@ -756,17 +1039,12 @@ static int launch_dispatch(pl_moe_plan_t plan, const DispatchPtrs& P, const MoeG
     launched = 3;
   }
   if (cudaGetLastError() != cudaSuccess) return 0;
-  const unsigned long long items = (unsigned long long)g.R * ((g.T + g.rows_per_item - 1) / g.rows_per_item) * g.n_tiles;
-  const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, (227 * 1024) / plan->move_smem));
-  int mgrid = (int)std::min<unsigned long long>(items, (unsigned long long)plan->sm_count * per_sm);
-  // Grouped rows: about 8/9 of the SMs, one CTA each (132 on a B200).  The 1 read : K writes stream
-  // is fastest there: 722-726 us at the C4 shape with 128-132 CTAs, 734-744 us with 136-148, 737 us
-  // with 296 (two per SM), 749-794 us with 112-120.
-  if (g.rows_per_item > 1) mgrid = (int)std::min<unsigned long long>(items, (unsigned long long)((plan->sm_count * 8 / 9 + 3) & ~3));
+  const unsigned long long tiles = g.move_rows > 1 ? (unsigned long long)g.R * ((g.T + g.move_rows - 1) / g.move_rows)
+                                                   : (unsigned long long)g.R * g.T * g.move_parts;
+  if (tiles > 0x7FFFFFFFull) return 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)mgrid);
+  cfg.gridDim = dim3((unsigned)tiles);
   cfg.blockDim = dim3(32);
-  cfg.dynamicSmemBytes = plan->move_smem;
   cfg.stream = cs;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -775,6 +1053,22 @@ static int launch_dispatch(pl_moe_plan_t plan, const DispatchPtrs& P, const MoeG
   cfg.numAttrs = fused ? 1 : 0;  // only the fused kernel releases its dependents early
   if (cudaLaunchKernelEx(&cfg, moe_move_kernel, P, g) != cudaSuccess) { cudaGetLastError(); return 0; }
   return launched + 1;
+}
+
+static bool launch_small(const DispatchPtrs& P, const MoeGeo& g, const SmallParams& Q, bool dedup, cudaStream_t cs) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)g.R * (((unsigned)g.T + Q.rows - 1) / Q.rows));
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = 128 + (size_t)Q.rows * g.row_bytes;
+  cfg.stream = cs;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = dedup ? cudaLaunchKernelEx(&cfg, moe_small_kernel<true>, P, g, Q) : cudaLaunchKernelEx(&cfg, moe_small_kernel<false>, P, g, Q);
+  if (e != cudaSuccess) { cudaGetLastError(); return false; }
+  return true;
 }
 
 pl_status_t pl_moe_dispatch(pl_moe_plan_t plan, const void* const* x, const int32_t* const* topk_idx,
@@ -793,11 +1087,46 @@ pl_status_t pl_moe_dispatch(pl_moe_plan_t plan, const void* const* x, const int3
     P.recv[r] = recv[r];
     P.meta[r] = recv_meta ? recv_meta[r] : nullptr;
   }
+  if (plan->small_rows) {
+    if (!launch_small(P, g, SmallParams{plan->small_rows, g.K, g.epr, nullptr, nullptr}, false, static_cast<cudaStream_t>(stream))) return PL_ERR_CUDA;
+    g_launches.fetch_add(1);
+    plan->dispatched = true;
+    return PL_OK;
+  }
   const int launched = launch_dispatch(plan, P, g, plan->fused, static_cast<cudaStream_t>(stream));
   if (!launched) return PL_ERR_CUDA;
   g_launches.fetch_add(launched);
   plan->dispatched = true;
   return PL_OK;
+}
+
+// Launched overlapped like the register executor: both kernels wait for everything in front before
+// they read.  Few tokens go by parts: a token per CTA turn leaves the last turn of a short launch
+// nearly empty, while at many tokens it hides the lookup of the next token's rows (B200, R = 8,
+// 7168 x bf16, top-8, turns -> parts: 64 tokens per rank 15.9 -> 13.9 us, 256 47.5 -> 45.0, 1024
+// 161 -> 168, 4096 611 -> 659).  So do rows of at most 256 units, which leave threads of a turn
+// idle or in flight with one unit (8 x 4096 tokens: 64 units top-8 145 -> 52 us, top-2 113 -> 23,
+// 256 units top-4 148 -> 120; 512 units top-6 291 -> 330, which is where the line lies).
+static bool launch_combine(pl_moe_plan_t plan, const CombinePtrs& P, const MoeGeo& g, cudaStream_t cs) {
+  const uint32_t units = g.row_bytes >> 4, parts = (units + kCombinePartThreads - 1) / kCombinePartThreads;
+  const unsigned long long n_tok = (unsigned long long)g.R * g.T, turns = (unsigned long long)plan->sm_count * plan->combine_per_sm;
+  const bool by_parts = (n_tok < 8 * turns || units <= 256) && n_tok * parts <= 0x7FFFFFFFull;
+  const uint32_t width = ((units + parts - 1) / parts + 31) / 32 * 32, tokens = parts > 1 ? 1u : kCombinePartThreads / width;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(by_parts ? (n_tok * parts + tokens - 1) / tokens : std::min(n_tok, turns)));
+  cfg.blockDim = dim3(by_parts ? tokens * width : kCombineThreads);
+  cfg.stream = cs;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = !by_parts  ? cudaLaunchKernelEx(&cfg, moe_combine_kernel, P, g)
+                        : g.K <= 2 ? cudaLaunchKernelEx(&cfg, moe_combine_parts_kernel<2>, P, g, parts, width)
+                        : g.K <= 4 ? cudaLaunchKernelEx(&cfg, moe_combine_parts_kernel<4>, P, g, parts, width)
+                                   : cudaLaunchKernelEx(&cfg, moe_combine_parts_kernel<8>, P, g, parts, width);
+  if (e != cudaSuccess) { cudaGetLastError(); return false; }
+  return true;
 }
 
 static pl_status_t combine_impl(pl_moe_plan_t plan, const void* const* y, const float* const* gates, void* const* out,
@@ -817,10 +1146,7 @@ static pl_status_t combine_impl(pl_moe_plan_t plan, const void* const* y, const 
     P.gates[r] = gates[r];
     P.out[r] = out[r];
   }
-  const unsigned long long n_tok = (unsigned long long)g.R * g.T;
-  const int grid = (int)std::min<unsigned long long>(n_tok, (unsigned long long)plan->sm_count * plan->combine_per_sm);
-  moe_combine_kernel<<<grid, kCombineThreads, 0, static_cast<cudaStream_t>(stream)>>>(P, g);
-  if (cudaGetLastError() != cudaSuccess) return PL_ERR_CUDA;
+  if (!launch_combine(plan, P, g, static_cast<cudaStream_t>(stream))) return PL_ERR_CUDA;
   g_launches.fetch_add(1);
   return PL_OK;
 }
@@ -875,6 +1201,13 @@ pl_status_t pl_moe_dispatch_dedup(pl_moe_plan_t plan, const void* const* x, cons
     P.meta[r] = recv_meta ? recv_meta[r] : nullptr;
   }
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  if (plan->small_rows) {
+    for (int r = 0; r < g.R; ++r) P.idx[r] = topk_idx[r];
+    if (!launch_small(P, d, SmallParams{plan->small_rows, g.K, g.epr, plan->d_ridx, plan->d_rmask}, true, cs)) return PL_ERR_CUDA;
+    g_launches.fetch_add(1);
+    plan->dispatched_dedup = true;
+    return PL_OK;
+  }
   const long long n_tok = (long long)g.R * g.T;
   moe_derive_ranks_kernel<<<(unsigned)((n_tok + 255) / 256), 256, 0, cs>>>(P0, g.R, g.T, g.K, g.epr, d.K, plan->d_ridx, plan->d_rmask);
   if (cudaGetLastError() != cudaSuccess) return PL_ERR_CUDA;
@@ -900,10 +1233,7 @@ pl_status_t pl_moe_combine_dedup(pl_moe_plan_t plan, const void* const* z, void*
     P.gates[r] = plan->d_ones;  // the expert layer has already applied the gates
     P.out[r] = out[r];
   }
-  const unsigned long long n_tok = (unsigned long long)d.R * d.T;
-  const int grid = (int)std::min<unsigned long long>(n_tok, (unsigned long long)plan->sm_count * plan->combine_per_sm);
-  moe_combine_kernel<<<grid, kCombineThreads, 0, static_cast<cudaStream_t>(stream)>>>(P, d);
-  if (cudaGetLastError() != cudaSuccess) return PL_ERR_CUDA;
+  if (!launch_combine(plan, P, d, static_cast<cudaStream_t>(stream))) return PL_ERR_CUDA;
   g_launches.fetch_add(1);
   return PL_OK;
 }

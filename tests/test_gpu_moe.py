@@ -313,3 +313,59 @@ def test_a_second_smaller_plan_does_not_break_the_first():
     finally:
         small.close()
         big.close()
+
+
+# One-launch dispatch up to 1024 routing entries per source, two launches above; combine by parts of
+# a row or by turns: both sides of the lines, rows of one vector, of a tile and a bit, several
+# tokens per CTA, receive buffers that are too small, and slots that are empty.
+@pytest.mark.parametrize("R,T,H,E,K", [
+    (8, 128, 64, 32, 8), (8, 129, 64, 32, 8), (2, 1024, 8, 4, 1), (2, 1025, 8, 4, 1), (4, 3, 1032, 1024, 4), (4, 9, 1032, 2048, 4),
+    (16, 40, 7168, 48, 3), (3, 700, 2048, 9, 2), (5, 33, 2056, 15, 6), (2, 20, 4096, 64, 32)])
+@pytest.mark.parametrize("short", [False, True])
+def test_dispatch_and_combine_around_the_lines(R, T, H, E, K, short):
+    idx, gates = gen.moe_routing(R, T, E, K, seed=5)
+    if K > 1:
+        idx = [a.copy() for a in idx]
+        for a in idx:
+            a[::7, K - 1] = -1
+    counts = np.zeros(R, np.int64)
+    for a in idx:
+        counts += np.bincount(a[a >= 0] // (E // R), minlength=R)
+    cap = int(counts.max()) - (1 if short and counts.max() > 1 else 0)
+    comm = B.pl_comm_create(R, B.PL_BF16)
+    plan = B.pl_moe_plan_create(comm, T, H, E, K, cap)
+    try:
+        x = gen.moe_tokens_bf16(R, T, H)
+        st = torch.cuda.current_stream().cuda_stream
+        d_x, d_i, d_g = [torch.from_numpy(a.view(np.int16)).cuda() for a in x], [torch.from_numpy(a).cuda() for a in idx], [torch.from_numpy(a).cuda() for a in gates]
+        recv = [torch.zeros(cap, H, dtype=torch.int16, device="cuda") for _ in range(R)]
+        meta = [torch.full((cap, 4), -1, dtype=torch.int32, device="cuda") for _ in range(R)]
+        out = [torch.zeros(T, H, dtype=torch.int16, device="cuda") for _ in range(R)]
+        ptr = lambda ts: [t.data_ptr() for t in ts]
+        for _ in range(2):
+            B.pl_moe_dispatch(plan, ptr(d_x), ptr(d_i), ptr(recv), ptr(meta), st)
+        B.pl_moe_combine(plan, ptr(recv), ptr(d_g), ptr(out), st)
+        pos, cnt, per = np.zeros((R, T, K), np.int32), np.zeros((R, R), np.int64), np.zeros((R, E), np.int64)
+        status = B.pl_moe_plan_read(plan, pos.ctypes.data, cnt.ctypes.data, per.ctypes.data, st)
+        assert status == (B.PL_ERR_OVERFLOW if cap < counts.max() else B.PL_OK)
+        # rows in (source rank, expert, token) order, by a sort that shares nothing with the kernels
+        for p in range(R):
+            assert np.array_equal(per[p], np.bincount(idx[p][idx[p] >= 0], minlength=E))
+            assert np.array_equal(cnt[p], per[p].reshape(R, E // R).sum(1))
+        for r in range(R):
+            rows = sorted((p, int(e), t, j) for p in range(R) for t, j in zip(*np.nonzero((idx[p] >= 0) & (idx[p] // (E // R) == r))) for e in [idx[p][t, j]])
+            got_rows, got_meta = recv[r].cpu().numpy().view(np.uint16), meta[r].cpu().numpy()
+            for i, (p, e, t, j) in enumerate(rows):
+                assert pos[p, t, j] == (i if i < cap else -1)
+                if i < cap:
+                    assert tuple(got_meta[i]) == (p, t, j, e)
+                    assert np.array_equal(got_rows[i], x[p][t])
+        for p in range(R):
+            w = np.where(pos[p] >= 0, gates[p], 0).astype(np.float64).sum(1)
+            want = gen.bf16_bits_to_f64(x[p].reshape(-1)).reshape(T, H) * w[:, None]
+            got = gen.bf16_bits_to_f64(out[p].cpu().numpy().view(np.uint16).reshape(-1)).reshape(T, H)
+            # every row of a token is the token itself: K fp32 products and sums, one rounding to bf16
+            assert np.all(np.abs(got - want) <= 2.0 ** -7 * np.abs(want) + 1e-6)
+    finally:
+        B.pl_moe_plan_destroy(plan)
+        B.pl_comm_destroy(comm)
