@@ -450,7 +450,10 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   // 1 MiB 6.2 -> 3.4 us, 4 MiB 10.3 -> 8.4 us, 8 MiB 24.7 -> 22.7 us).  Bulk-copy schedules only
   // on request: which SMs a grid smaller than the GPU lands on then depends on the launch in front
   // (all-gather of 64 MiB +7 us, fused all-reduce of 16 MiB +0.4 us).
-  S->overlap_launch = (flags & PL_OPT_OVERLAP_LAUNCH) || pol.datapath == PL_DP_LDST;
+  // Nor the layer executor with flags: its CTAs run for all layers, and those of the next launch
+  // take the SMs as they become free, two on one SM and none on another (80 layers of 1 MiB
+  // 292 -> 385 us, of 512 KiB 210 -> 361 us; as one cluster, 16 KiB, 104 -> 98 us).
+  S->overlap_launch = (flags & PL_OPT_OVERLAP_LAUNCH) || (pol.datapath == PL_DP_LDST && (layers.ctas_per_rank == 0 || layers.cluster));
   S->stage_ahead = (flags & PL_OPT_STAGE_AHEAD) != 0;
   S->out_scale = out_scale;
   S->hook = hook;
