@@ -35,12 +35,12 @@ MIB = 1 << 20
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 # dram__bytes_read.sum + dram__bytes_write.sum of one reduce-scatter launch of this workload
-# (one ncu capture of that launch, caches flushed before it: 537.7 MB read, 18.1 MB written; three
-# quarters of the 64 MiB of results are still in L2 when the kernel ends)
-NCU_RS_TRAFFIC_BYTES = 555785728.0
+# (one ncu capture of that launch, caches flushed before it: 536.9 MB read, 22.1 MB written; two
+# thirds of the 64 MiB of results are still in L2 when the kernel ends)
+NCU_RS_TRAFFIC_BYTES = 559000000.0
 # the same sum for a reduce-scatter launch inside the step (one pass, caches left as the
-# all-gather before it left them): 537.1 MB read, 76.9 MB written
-NCU_RS_TRAFFIC_IN_SITU_BYTES = 614000000.0
+# all-gather before it left them): 536.9 MB read, 79.1 MB written
+NCU_RS_TRAFFIC_IN_SITU_BYTES = 616000000.0
 
 
 def measured_peak():
@@ -148,7 +148,9 @@ def run_purlin(args):
     step_flags = 0 if args.plain_options else B.PL_OPT_INPUTS_LAST_USE
     opts = B.make_opts(n_ctas=args.n_ctas, threads=args.threads, slice_bytes=args.slice_bytes,
                        datapath=args.datapath, stages=args.stages, stage_bytes=args.stage_bytes, flags=step_flags)
-    # The reduce-scatter is also launched overlapped: its CTAs are set up (barriers, first
+    # With nothing else about the launch asked for, both run without queues (one CTA per tile), are
+    # always launched overlapped and use no tuned grid.  On the bulk-copy executor (--datapath 2)
+    # the reduce-scatter is launched overlapped: its CTAs are set up (barriers, first
     # descriptor) while the all-gather in front of it drains, 2 us per step.  The all-gather is
     # not: CTAs of an overlapped launch take the SMs in the order in which they become free, and a
     # grid smaller than the SM count then ends up on other SMs than the ones it was tuned for (+7 us).
@@ -300,7 +302,7 @@ def run_purlin(args):
     ag_floor = iag.hbm_bytes                               # compulsory DRAM traffic (R+1) * M
     rs_gbs = rs_alg / (rs_ms.mean() * 1e-3) / 1e9
     ag_gbs = ag_floor / (ag_ms.mean() * 1e-3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "pl_exec_tma_kernel<bf16> (reduce-scatter launch)",
+    roofline = {"bound": "hbm", "kernel": ("pl_flat_bulk_reduce_kernel<bf16>" if irs.stages == 1 else "pl_exec_tma_kernel<bf16>") + " (reduce-scatter launch)",
                 "achieved": rs_gbs, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                 "frac": rs_gbs / peak, "frac_of_nominal_8TBps": rs_gbs / NOMINAL_HBM_GBS,
                 "algorithmic_bytes_per_launch": int(rs_alg), "avg_launch_us": float(rs_ms.mean() * 1e3),
@@ -353,7 +355,8 @@ def run_purlin(args):
             "config": {"workload": "C2: reduce-scatter (64 MiB/rank in) then all-gather (64 MiB/rank out), "
                                    "R=8 emulated ranks in one HBM, bf16 N(0,1) seed 0, direct schedules, 1 MiB chunks",
                        "options": "default" if args.plain_options else "PL_OPT_INPUTS_LAST_USE on both schedules (inputs loaded evict-first), "
-                                  "PL_OPT_OVERLAP_LAUNCH on the reduce-scatter; all-gather grid from pl_comm_tune",
+                                  "PL_OPT_OVERLAP_LAUNCH on the reduce-scatter" +
+                                  ("" if iag.stages == 1 else "; all-gather grid from pl_comm_tune"),
                        "l2": "inputs_larger_than_l2 (512 MiB of inputs per step; no flush)",
                        "replicas": world, "parallelism": "replicas only (no inter-GPU exchange on this path)"},
             "clocks": clocks, "e2e": e2e, "gpu_launches": int(launches), "roofline": roofline,
