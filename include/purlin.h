@@ -116,6 +116,10 @@ typedef enum {
  *                         into all R outputs (no gather step, fewest bytes).
  *   PL_ALGO_RING          textbook ring; partial sums of bf16 data travel in fp32, of fp32
  *                         data as compensated fp32 pairs (PL_F32X2), of int32 data in int32.
+ *                         With nothing about the launch asked for the hops go through the
+ *                         shared memory of thread-block clusters where that is faster: the
+ *                         info then has that launch, no scratch, and the bytes of inputs and
+ *                         outputs; the op list still states which rank adds what, in order.
  *   PL_ALGO_TREE          all-reduce only: binomial reduce to a root, binomial broadcast from it;
  *                         the root of chunk c is rank c mod R (rank 0 for a one-chunk message).
  * Ring and tree are not in the paper (its only pattern is the direct pull); they are the

@@ -54,6 +54,8 @@ struct pl_schedule_s {
   bool flat = false;              // no flags, everything left to the library: one CTA per tile (pl_datapath_flat.cu)
   FlatLaunch flat_launch{};
   std::vector<FlatSpan> flat_spans;  // uploaded in place of op list and flags
+  bool ring = false;              // ring with everything left to the library: a cluster per tile (pl_datapath_ring.cu)
+  RingLaunch ring_launch{};
   int packet_ctas_per_rank = 0;   // > 0: packet datapath (layered one-shot all-reduce), CTAs per rank
   long long packet_break_op = -1; // test hook (pl_schedule_debug_break_wait on a packet schedule)
   size_t off_trace = 0;
@@ -145,6 +147,16 @@ void fill_info(pl_schedule_s* S, int R) {
   I.stages = S->pol.stages;
   I.stage_bytes = S->pol.stage_bytes;
   I.slice_bytes = S->pol.slice_bytes;
+  if (S->ring) {  // what travels between ranks stays in shared memory
+    I.grid = S->ring_launch.grid;
+    I.threads = S->ring_launch.threads;
+    I.smem_bytes = (int32_t)S->ring_launch.smem_bytes;
+    I.stages = 1;
+    I.stage_bytes = S->ring_launch.tile * 16u;
+    I.scratch_bytes = 0;
+    I.hbm_bytes = 0;
+    for (int r = 0; r < R; ++r) I.hbm_bytes += I.in_bytes[r] + I.out_bytes[r];
+  }
   if (S->flat) {
     I.grid = (int32_t)S->flat_launch.blocks;
     I.threads = S->flat_launch.threads;
@@ -238,7 +250,7 @@ pl_status_t upload(pl_schedule_s* S, int R) {
   uint64_t total = 0;
   for (int r = 0; r < R; ++r) {
     S->scratch_off[r] = total;
-    total += align_up(S->L.scratch_per_rank[r], 256);
+    if (!S->ring) total += align_up(S->L.scratch_per_rank[r], 256);
   }
   if (S->stage_ahead) {  // second staging buffer of every rank, one half behind the first
     S->scratch_half = total;
@@ -499,11 +511,19 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   }
   for (const HostOp& op : S->L.ops)
     if (op.kind == PL_OP_COPY && op.bcast) S->bcast_copies = true;
+  const bool all_default = !opts || (opts->n_ctas == 0 && opts->threads == 0 && opts->datapath == PL_DP_AUTO && opts->stages == 0 &&
+                                     opts->stage_bytes == 0 && opts->slice_bytes == 0 && !idle_asked);
+  // A ring with nothing about the launch asked for: its hops inside clusters.  (A processing phase is
+  // the queue executors' business.)
+  if (!comm->planner && rq.algo == PL_ALGO_RING && !hook && !S->trace && all_default && rq.n_layers == 0) {
+    const bool reduce = rq.coll != PL_ALLGATHER;
+    const uint64_t part = rq.count_per_rank * (uint64_t)elem_size(comm->dtype) / (reduce ? (uint64_t)comm->R : 1ull) / 16;
+    S->ring = ring_shape(comm->R, comm->dtype, reduce, part, comm->sm_count, &S->ring_launch) &&
+              ring_prepare(comm->dtype, comm->R, S->ring_launch) > 0;
+  }
   // No flags and nothing about the launch asked for: no queues.  Planner communicators keep the
   // queues, which is what their schedules are inspected for.
-  if (!comm->planner && rq.n_layers <= 1 && S->L.n_flags == 0 && !rq.staged && !S->trace && !S->layer_kernel &&
-      (!opts || (opts->n_ctas == 0 && opts->threads == 0 && opts->datapath == PL_DP_AUTO && opts->stages == 0 && opts->stage_bytes == 0 &&
-                 opts->slice_bytes == 0 && !idle_asked))) {
+  if (!comm->planner && rq.n_layers <= 1 && S->L.n_flags == 0 && !rq.staged && !S->trace && !S->layer_kernel && !S->ring && all_default) {
     bool reduce = false, all = false;
     if (flat_plan(S->L, comm->R, comm->dtype, &S->flat_spans, &reduce, &all)) {
       uint64_t units = 0, blocks = 0;
@@ -1025,6 +1045,17 @@ pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index) {
     s->layer_break_queue = h.queue;
     return PL_OK;
   }
+  if (s->ring) {  // it reads no wait entries: from here on the op queues execute the schedule
+    uint64_t total = 0;
+    for (int r = 0; r < s->comm->R; ++r) {
+      s->scratch_off[r] = total;
+      total += align_up(s->L.scratch_per_rank[r], 256);
+    }
+    if (total && !s->d_scratch && cudaMalloc(&s->d_scratch, total) != cudaSuccess) { cudaGetLastError(); return PL_ERR_OOM; }
+    s->scratch_total = total;
+    s->ring = false;
+    fill_info(s, s->comm->R);
+  }
   const size_t pos = (size_t)s->topo_to_dev[op_index];
   DevWait& w = s->waits[pos * s->wait_stride];
   w.need += 1;  // one more signal than the schedule will ever produce
@@ -1133,6 +1164,26 @@ pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
     F.status = s->comm->d_status;
     F.timeout_ns = s->timeout_ns;
     if (launch_flat(s->comm->dtype, F, s->flat_launch, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
+      cudaGetLastError();
+      return PL_ERR_CUDA;
+    }
+    g_launches.fetch_add(1);
+    return PL_OK;
+  }
+  if (s->ring) {
+    RingHopParams K;
+    for (int r = 0; r < R; ++r) {
+      K.in[r] = bufs->in[r];
+      K.out[r] = bufs->out[r];
+    }
+    // in units: a partition is the input of an all-gather, the output of a reduce-scatter
+    K.reduce = s->info.in_bytes[0] >= s->info.out_bytes[0];
+    K.gather = s->info.out_bytes[0] >= s->info.in_bytes[0];
+    K.part_units = std::min(std::min(s->info.in_bytes[0], s->info.out_bytes[0]), std::max(s->info.in_bytes[0], s->info.out_bytes[0]) / (uint64_t)R) / 16;
+    K.n_ranks = R;
+    K.tile = s->ring_launch.tile;
+    K.out_scale = s->out_scale;
+    if (launch_ring(s->comm->dtype, K, s->ring_launch, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
       cudaGetLastError();
       return PL_ERR_CUDA;
     }

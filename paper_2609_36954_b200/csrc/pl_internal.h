@@ -137,6 +137,25 @@ struct FlatLaunch {  // host side: which kernel, how many CTAs
   int threads;
 };
 
+// ---- ring execution, a cluster of one CTA per rank for every tile (pl_datapath_ring.cu) --------
+constexpr int kRingThreads = 256;  // most threads of a CTA
+struct RingHopParams {
+  const void* in[PL_MAX_RANKS];
+  void* out[PL_MAX_RANKS];
+  uint64_t part_units;     // 16-byte units of a partition
+  int n_ranks;
+  uint32_t reduce, gather; // reduce-scatter, all-gather, or both (all-reduce)
+  uint32_t tile;           // units of a partition per cluster
+  float out_scale;
+};
+struct RingLaunch {
+  int units, threads, grid;  // units per thread
+  uint32_t tile;
+  size_t smem_bytes;
+};
+// False where the op queues execute the ring better (or it has more tiles than a grid).
+bool ring_shape(int R, int dtype, bool reduce, uint64_t part_units, int sm_count, RingLaunch* L);
+
 // What the layer executor needs on top of ExecParams (see pl_datapath_layers.cu): the distance from
 // a layer's operands to the next layer's, in bytes.
 struct LayerParams {

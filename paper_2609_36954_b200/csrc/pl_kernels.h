@@ -28,6 +28,10 @@ bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads);
 FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units);
 cudaError_t launch_flat(int dtype, const FlatParams& P, const FlatLaunch& F, cudaStream_t stream);
 
+// ring schedules, a cluster per tile.  ring_prepare: clusters that can be resident at once (0: none)
+int ring_prepare(int dtype, int R, const RingLaunch& L);
+cudaError_t launch_ring(int dtype, const RingHopParams& P, const RingLaunch& L, cudaStream_t stream);
+
 // packet executor (latency path): rank = cluster of ctas_per_rank CTAs
 cudaError_t launch_exec_packet(int dtype, const PacketParams& P, int threads, bool overlap, cudaStream_t stream);
 int exec_packet_max_groups(int dtype, int ctas_per_rank, int threads);

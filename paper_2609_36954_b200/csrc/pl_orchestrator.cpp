@@ -1227,6 +1227,36 @@ void assign_queues(Lowered* L, int R, int n_queues, bool by_level) {
   }
 }
 
+// A hop takes longer the more a CTA stores into its neighbour, so small messages get as few threads per
+// CTA as leave about 1024 CTAs (seven per SM), or one CTA per SM while that needs at most 128 threads.
+// All-reduce, us by threads per CTA: 4 x 1 MiB fp32 7.9 (64), 9.0 (128), 11.5 (256); 8 x 1 MiB bf16
+// 15.9 (64), 18.3, 22.9; 8 x 2 MiB 30.7, 20.8 (128), 25.4; 8 x 4 MiB 59.8, 40.0, 30.9 (256); 8 x 256 KiB
+// 14.1, 11.5 (128), 12.0; 8 x 64 KiB 9.4 (32), 9.8 (128).  At 256 threads more CTAs than fit only queue
+// up behind one another: 8 x 64 MiB reduce-scatter 237 us, with 128 threads 311, with 512 247.  One unit
+// per thread, since the barrier comes sooner (two: 275 us); with two ranks there is one hop, and
+// four units keep more loads in flight (2 x 64 MiB int32 32 us, one unit 38).
+// A large all-gather alone stays with the queues: its hops carry no partial sums, which is what the
+// neighbours' shared memory saves.  us, clusters / queues, by bytes per rank: 8 ranks 1 MiB 28.3 / 34.3,
+// 8 MiB 197 / 155; 4 ranks 1 MiB 11.0 / 15.0, 8 MiB 61 / 50; 2 ranks 1 MiB 3.5 / 6.5, 2 MiB 5.3 / 4.8;
+// 16 ranks 256 KiB 43 / 49, 1 MiB 121 / 116.
+bool ring_shape(int R, int dtype, bool reduce, uint64_t part_units, int sm_count, RingLaunch* L) {
+  const uint64_t total = part_units * (uint64_t)R, mib = (1u << 20) / 16;
+  if (!part_units || (!reduce && (part_units > mib || total > 8 * mib))) return false;
+  L->units = 1;
+  if (total <= 128ull * sm_count) {
+    L->threads = (int)((total + sm_count - 1) / sm_count + 31) / 32 * 32;
+  } else {
+    for (L->threads = 32; L->threads < kRingThreads && total > 1024ull * L->threads; L->threads *= 2) {}
+    if (R == 2 && L->threads == kRingThreads) L->units = 4;
+  }
+  L->tile = (uint32_t)(L->units * L->threads);
+  const uint64_t tiles = (part_units + L->tile - 1) / L->tile;
+  if (tiles * R > 0x7FFFFFFFull) return false;
+  L->grid = (int)(tiles * R);
+  L->smem_bytes = (size_t)L->tile * 16 * 2 * (dtype == PL_BF16 || dtype == PL_F32 ? 2 : 1);
+  return true;
+}
+
 bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all) {
   spans->clear();
   if (L.ops.empty() || L.n_flags != 0) return false;

@@ -1,0 +1,55 @@
+"""Ring schedules with everything left to the library (a cluster per tile, hops through shared memory)
+against the same schedule on the op queues: the same bits, at the edges of tiles and launch shapes."""
+import pytest
+import torch
+
+from gpu_harness import DT, stream_handle
+from paper_2609_36954_b200 import binding as B
+from test_gpu_flat import SIZE, same_bits
+
+pytestmark = pytest.mark.gpu
+
+
+def build(coll, n):
+    return lambda c, o: B.pl_schedule_build(c, coll, B.PL_ALGO_RING, n, 64 * 1024, o)
+
+
+# units (16 bytes) of a partition: a single one, around a warp and the tiles of 64, 128, 256 and 1024
+# units, and one large enough for the largest tile with a ragged end
+@pytest.mark.parametrize("R,dtype", [(2, "f32"), (2, "i32"), (3, "bf16"), (5, "f32"), (8, "bf16"), (8, "i32"), (16, "bf16"), (16, "f32")])
+@pytest.mark.parametrize("units", [1, 31, 33, 257, 4099, 9001, 65539, "large"])
+def test_reducing_rings(R, dtype, units):
+    units = units if units != "large" else 2 ** 20 // R + 1025
+    n = 16 * units // SIZE[dtype] * R
+    for coll in (B.PL_REDUCE_SCATTER, B.PL_ALLREDUCE):
+        info = same_bits(R, dtype, build(coll, n), **({"out_scale": 0.375} if dtype != "i32" else {}))
+        assert info.scratch_bytes == 0
+
+
+# up to 1 MiB per rank and 8 MiB in all in clusters, above that on the op queues
+@pytest.mark.parametrize("R,dtype", [(2, "f32"), (3, "bf16"), (8, "u8"), (16, "bf16")])
+@pytest.mark.parametrize("units", [1, 33, 4099, 32768, 65536, 65537])
+def test_gathering_rings(R, dtype, units):
+    same_bits(R, dtype, build(B.PL_ALLGATHER, 16 * units // SIZE[dtype]))
+
+
+def test_broken_wait_times_out():
+    """The fault hook moves the schedule to the op queues, whose waits it edits."""
+    R, n = 4, 4096
+    comm = B.pl_comm_create(R, DT["f32"])
+    s = build(B.PL_ALLREDUCE, n)(comm, B.make_opts(timeout_ns=20_000_000))
+    try:
+        t = [torch.ones(n, device="cuda") for _ in range(2 * R)]
+        size = [4 * n] * R
+        bufs = B.make_bufs([x.data_ptr() for x in t[:R]], [x.data_ptr() for x in t[R:]], size, size)
+        B.pl_execute(s, bufs, stream_handle())
+        torch.cuda.synchronize()
+        assert all(bool((x == R).all()) for x in t[R:])
+        B.pl_schedule_debug_break_wait(s, next(o.topo for o in B.pl_schedule_dump(s) if o.n_wait > 0))
+        assert B.pl_schedule_info(s).scratch_bytes > 0
+        B.pl_execute(s, bufs, stream_handle())
+        torch.cuda.synchronize()
+        assert B.pl_comm_status(comm).code == B.PL_ERR_TIMEOUT
+    finally:
+        B.pl_schedule_destroy(s)
+        B.pl_comm_destroy(comm)
