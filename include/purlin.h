@@ -447,8 +447,9 @@ pl_status_t pl_schedule_build_rooted(pl_comm_t comm, pl_collective_t coll, int r
  * (M = count_per_rank * elem_size).  Rank r's layer-(l+1) contribution counts as published
  * only when r's layer-l output is complete, and no consumer reads it earlier.  Algorithms:
  * PL_ALGO_ONESHOT, PL_ALGO_DIRECT, PL_ALGO_DIRECT_FUSED; PL_ALGO_AUTO picks direct-fused on the
- * register executor, and for messages of at most 4 KiB (with grid, datapath and hooks left to the
- * library) one-shot on the packet datapath with one CTA per rank, the fastest form there. */
+ * register executor, and for messages of at most 4 KiB that do not split into a 16-byte vector or
+ * more per rank (with grid, datapath and hooks left to the library) one-shot on the packet datapath
+ * with one CTA per rank.  Planner communicators plan packets for every message of at most 4 KiB. */
 pl_status_t pl_schedule_build_layers(pl_comm_t comm, pl_algo_t algo, size_t count_per_rank,
                                      int n_layers, const pl_sched_opts_t* opts,
                                      pl_schedule_t* out);

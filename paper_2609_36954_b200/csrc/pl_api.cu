@@ -946,11 +946,15 @@ pl_status_t pl_schedule_build_layers(pl_comm_t comm, pl_algo_t algo, size_t coun
   rq.coll = PL_ALLREDUCE;
   rq.algo = algo == PL_ALGO_AUTO ? PL_ALGO_DIRECT_FUSED : algo;  // the fastest layered form at 16 KiB - 1 MiB
   if (algo == PL_ALGO_AUTO && opts && opts->struct_size == sizeof(pl_sched_opts_t) && opts->datapath == PL_DP_PACKET) rq.algo = PL_ALGO_ONESHOT;
-  // Everything left to the library and a message of at most 4 KiB: the packet datapath with one
-  // CTA per rank is the fastest layered form there (1.8-2.05 us per layer against 2.0-2.2 us with flags).
+  // Everything left to the library and a message of at most 4 KiB: the packet datapath with one CTA
+  // per rank, unless the message has a whole vector for every rank and the layer executor's cluster can
+  // run it (us per layer, packets / cluster: 2 ranks 32 bytes 1.37 / 0.94, 4 ranks 1 KiB 1.53 / 1.05,
+  // 8 ranks 1 KiB 2.08 / 1.17, 4 KiB 2.37 / 1.18, fp32 2.67 / 1.42, 16 ranks 4 KiB 3.45 / 1.74; the
+  // register executor's flags take 2.0-2.2).  A planner communicator, which runs nothing, has packets.
   pl_sched_opts_t packet_opts;
-  if (algo == PL_ALGO_AUTO && comm && comm->dtype != PL_U8 && count_per_rank * (size_t)elem_size(comm->dtype) <= 4096 &&
-      (count_per_rank * (size_t)elem_size(comm->dtype)) % 16 == 0 &&
+  const size_t tiny = comm ? count_per_rank * (size_t)elem_size(comm->dtype) : 0;
+  if (algo == PL_ALGO_AUTO && comm && comm->dtype != PL_U8 && tiny <= 4096 && tiny % 16 == 0 &&
+      (comm->planner || n_layers == 1 || tiny % (16 * (size_t)comm->R)) &&
       (!opts || (opts->struct_size == sizeof(pl_sched_opts_t) && opts->datapath == PL_DP_AUTO && opts->n_ctas == 0 && opts->threads == 0 &&
                  opts->hook == 0 && !(opts->flags & PL_OPT_STAGED)))) {
     std::memset(&packet_opts, 0, sizeof(packet_opts));

@@ -92,3 +92,22 @@ def test_layers_trace_and_time_out(nbytes):
         ses.execute(s, x)
     finally:
         ses.close()
+
+
+# tiny messages with everything left to the library: the layer executor where the message has a vector for
+# every rank, packets where it has not; the same bits as packets asked for
+@pytest.mark.parametrize("R,dtype,nbytes,want", [
+    (8, "bf16", 128, B.PL_DP_LDST), (8, "bf16", 128 + 16, B.PL_DP_PACKET), (8, "f32", 4096, B.PL_DP_LDST), (3, "f32", 48, B.PL_DP_LDST),
+    (3, "bf16", 4096, B.PL_DP_PACKET), (16, "i32", 256, B.PL_DP_LDST), (16, "bf16", 240, B.PL_DP_PACKET), (2, "i32", 4096, B.PL_DP_LDST)])
+def test_tiny_layers_left_to_the_library(R, dtype, nbytes, want):
+    n, layers = nbytes // SIZE[dtype], 5
+    x = [np.concatenate([gen.rank_inputs(R, n, dtype, seed=l)[r] for l in range(layers)]) for r in range(R)]
+    ses = Session(R, dtype)
+    try:
+        auto = ses.build_layers(B.PL_ALGO_AUTO, n, layers)
+        assert B.pl_schedule_info(auto).datapath == want
+        a, _ = ses.execute(auto, x)
+        b, _ = ses.execute(ses.build_layers(B.PL_ALGO_ONESHOT, n, layers, datapath=B.PL_DP_PACKET), x)
+        assert all(np.array_equal(p, q) for p, q in zip(a, b))
+    finally:
+        ses.close()
