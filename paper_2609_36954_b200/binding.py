@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 from . import build as _build
 
@@ -154,15 +155,15 @@ def load():
         "pl_comm_tune": [vp, vp, P(C.c_int32), P(C.c_int32), P(C.c_int32)],
         "pl_moe_plan_create": [vp, i32, i32, i32, i32, sz, P(vp)],
         "pl_moe_plan_destroy": [vp],
-        "pl_moe_dispatch": [vp, P(vp), P(vp), P(vp), P(vp), vp],
-        "pl_moe_combine": [vp, P(vp), P(vp), P(vp), vp],
+        "pl_moe_dispatch": [vp, vp, vp, vp, vp, vp],
+        "pl_moe_combine": [vp, vp, vp, vp, vp],
         "pl_moe_plan_read": [vp, vp, vp, vp, vp],
-        "pl_moe_combine_logits": [vp, P(vp), P(vp), P(vp), vp],
-        "pl_moe_dispatch_dedup": [vp, P(vp), P(vp), P(vp), P(vp), vp],
-        "pl_moe_combine_dedup": [vp, P(vp), P(vp), vp],
+        "pl_moe_combine_logits": [vp, vp, vp, vp, vp],
+        "pl_moe_dispatch_dedup": [vp, vp, vp, vp, vp, vp],
+        "pl_moe_combine_dedup": [vp, vp, vp, vp],
         "pl_moe_plan_read_dedup": [vp, vp, vp, vp],
-        "pl_reduce_scatter_ring_static": [i32, i32, sz, P(vp), P(vp), vp, vp],
-        "pl_reduce_scatter_ring_static_debug_timeout": [i32, i32, sz, P(vp), P(vp), vp, vp, u64],
+        "pl_reduce_scatter_ring_static": [i32, i32, sz, vp, vp, vp, vp],
+        "pl_reduce_scatter_ring_static_debug_timeout": [i32, i32, sz, vp, vp, vp, vp, u64],
     }
     for name, args in sig.items():
         fn = getattr(L, name)
@@ -328,7 +329,11 @@ def pl_schedule_destroy(s):
 
 
 def pl_execute(s, bufs, stream=0):
-    _check(load().pl_execute(s, C.byref(bufs), stream), "pl_execute")
+    # the shortest way into the library: a call that the GPU finishes sooner is bound by it (the
+    # structure itself instead of byref() and no helper calls: 0.8 -> 0.5 us in front of the launch)
+    st = (_lib or load()).pl_execute(s, bufs, stream)
+    if st:
+        raise PurlinError(st, "pl_execute")
 
 
 def pl_execute_host(s, host_bufs, dev_bufs, stream=0):
@@ -362,15 +367,17 @@ def pl_comm_host_sync(comm):
     _check(load().pl_comm_host_sync(comm), "pl_comm_host_sync")
 
 
-_ptr_types = {n: C.c_void_p * n for n in range(1, PL_MAX_RANKS + 1)}  # building the type costs more than filling it
+# Device addresses of a call, one per rank, as the array the library reads: the bytes of packed
+# 64-bit words cost a fifth of a ctypes array, whose items are converted one by one (8 ranks: 0.25
+# against 1.3 us; a small dispatch has four of them).
+_ptr_packers = {n: struct.Struct(f"{n}Q").pack for n in range(1, PL_MAX_RANKS + 1)}
 
 
 def _ptr_array(addrs):
-    T = _ptr_types.get(len(addrs)) or C.c_void_p * len(addrs)
     try:
-        return T(*addrs)  # plain ints and None
-    except TypeError:
-        return T(*[int(a) if a else None for a in addrs])
+        return _ptr_packers[len(addrs)](*addrs)  # plain addresses
+    except (KeyError, TypeError, struct.error):
+        return (C.c_void_p * len(addrs))(*[int(a) if a else None for a in addrs])
 
 
 def pl_moe_plan_create(comm, tokens_per_rank, hidden, n_experts, topk, recv_capacity_rows):
