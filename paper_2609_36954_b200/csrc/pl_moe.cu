@@ -30,6 +30,11 @@ constexpr int kMaskWords = kTB / 32;
 constexpr int kMaxTopk = 32;
 constexpr int kCombineThreads = 256, kCombinePartThreads = 128;
 
+// Kernels here are launched while the one in front drains, and that one may be what writes their
+// routing (the caller's router, moe_derive_ranks_kernel).  So what a launch in front can write is
+// read with coherent loads behind griddepcontrol.wait, plain ones or __ldcg, never with __ldg: a
+// non-coherent load wants data that nobody writes while the kernel lives.
+
 struct DispatchPtrs {
   const void* x[PL_MAX_RANKS];
   const int32_t* idx[PL_MAX_RANKS];
@@ -186,7 +191,7 @@ __global__ void __launch_bounds__(kTB) moe_plan_kernel(const __grid_constant__ D
     for (int j0 = 0; j0 < g.K; j0 += 8) {
       int ev[8];  // eight slots at a time: the loads are independent of one another
 #pragma unroll
-      for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < g.K) ? __ldg(&idx[(size_t)t * g.K + j0 + k]) : -1;
+      for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < g.K) ? idx[(size_t)t * g.K + j0 + k] : -1;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int e = ev[k];
@@ -298,7 +303,7 @@ __global__ void __launch_bounds__(kTB) moe_plan_kernel(const __grid_constant__ D
       for (int j0 = 0; j0 < g.K; j0 += 8) {
         int ev[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < g.K) ? __ldg(&idx[(size_t)t * g.K + j0 + k]) : -1;
+        for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < g.K) ? idx[(size_t)t * g.K + j0 + k] : -1;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int j = j0 + k;
@@ -438,7 +443,7 @@ __device__ __forceinline__ uint32_t rank_set(const int32_t* idx, int K, int epr,
   for (int j0 = 0; j0 < K; j0 += 8) {
     int ev[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < K) ? __ldg(&idx[j0 + k]) : -1;
+    for (int k = 0; k < 8; ++k) ev[k] = (j0 + k < K) ? idx[j0 + k] : -1;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (ev[k] >= 0 && ev[k] < epr * R) set |= 1u << (ev[k] / epr);
@@ -494,7 +499,7 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int i = i0 + k * kSmallThreads, q = i / nv;
-          ev[k] = i < all ? __ldg(reinterpret_cast<const int4*>(P.idx[q]) + (i - q * nv)) : make_int4(-1, -1, -1, -1);
+          ev[k] = i < all ? reinterpret_cast<const int4*>(P.idx[q])[i - q * nv] : make_int4(-1, -1, -1, -1);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -511,7 +516,7 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
       for (int q0 = 0; q0 < n; q0 += 8) {
         int ev[8];  // independent loads: one L2 latency per batch
 #pragma unroll
-        for (int k = 0; k < 8; ++k) ev[k] = (q0 + k < n) ? __ldg(&P.idx[q0 + k][i]) : -1;
+        for (int k = 0; k < 8; ++k) ev[k] = (q0 + k < n) ? P.idx[q0 + k][i] : -1;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           if ((unsigned)ev[k] < (unsigned)g.E) count_rank(into, rank_of(ev[k]));
@@ -538,7 +543,7 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
         for (int e = tid; e < g.E; e += kSmallThreads) s_hist[e] = 0;
         __syncthreads();
         for (int i = tid; i < TK; i += kSmallThreads) {
-          const int e = __ldg(&own[i]);
+          const int e = own[i];
           if ((unsigned)e < (unsigned)g.E) atomicAdd(&s_hist[e], 1);
         }
         __syncthreads();
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
     if (tid < nrows) s_set[tid] = (int32_t)rank_set(own + (size_t)(t0 + tid) * K, K, Q.epr0, R);
     count_tokens(0, p * T + t0, c);
   } else {
-    for (int i = tid; i < TK; i += kSmallThreads) s_own[i] = __ldg(&own[i]);
+    for (int i = tid; i < TK; i += kSmallThreads) s_own[i] = own[i];
     count_sources(p, c, false);
   }
   __syncthreads();
@@ -607,7 +612,7 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
         row = s_cnt[r];
         for (int k = 0; k < src; ++k) row += (int)(((uint32_t)s_set[k] >> r) & 1u);
         for (int k = 0; k < K; ++k) {
-          const int e = __ldg(&own[(size_t)t * K + k]);
+          const int e = own[(size_t)t * K + k];
           if (e >= 0 && e / Q.epr0 == r) mask |= 1u << k;
         }
       }

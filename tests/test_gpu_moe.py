@@ -369,3 +369,54 @@ def test_dispatch_and_combine_around_the_lines(R, T, H, E, K, short):
     finally:
         B.pl_moe_plan_destroy(plan)
         B.pl_comm_destroy(comm)
+
+
+# Dispatches are launched while the launch in front drains.  Here that launch makes their routing, another
+# one every time, in the same buffers: a reduce-scatter of int32 (flat executor, lets its followers start
+# at once) whose sum is the indices.  One-launch dispatch, bookkeeping + rows, and both deduplicated.
+@pytest.mark.parametrize("T", [64, 400])
+@pytest.mark.parametrize("dedup", [False, True])
+@pytest.mark.parametrize("graph", [False, True])
+def test_routing_written_by_the_launch_in_front(T, dedup, graph):
+    R, H, E, K, turns = 4, 256, 32, 4, 6
+    routes = [gen.moe_routing(R, T, E, K, seed=20 + i)[0] for i in range(turns)]
+    x = gen.moe_tokens_bf16(R, T, H, seed=9)
+    cap = R * T * K
+    run, ids = MoeRun(R, T, H, E, K, cap), B.pl_comm_create(R, B.PL_I32)
+    sched = B.pl_schedule_build(ids, B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, R * T * K, 1 << 20)
+    ptr = lambda ts: [t.data_ptr() for t in ts]
+    try:
+        nb = T * K * 4
+        noise = [np.random.default_rng(p).integers(-999, 999, R * T * K).astype(np.int32) for p in range(R - 1)]
+        made = []  # what the ranks hold, so that the sum over ranks of partition r is the routing of rank r
+        for route in routes:
+            last = np.concatenate([a.reshape(-1) for a in route]) - sum(noise)
+            made.append([to_dev(a) for a in noise + [last.astype(np.int32)]])
+        d_x, d_idx = [to_dev(a) for a in x], [poison(nb) for _ in range(R)]
+        recv = [[poison(cap * H * 2) for _ in range(R)] for _ in range(turns)]
+        meta = [[poison(cap * 16) for _ in range(R)] for _ in range(turns)]
+        bufs = [B.make_bufs(ptr(m), ptr(d_idx), [R * nb] * R, [nb] * R) for m in made]
+
+        def work(h):
+            for i in range(turns):
+                B.pl_execute(sched, bufs[i], h)
+                (B.pl_moe_dispatch_dedup if dedup else B.pl_moe_dispatch)(run.plan, ptr(d_x), ptr(d_idx), ptr(recv[i]), ptr(meta[i]), h)
+
+        if graph:
+            g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            with torch.cuda.graph(g, stream=side):
+                work(stream_handle())
+            g.replay()
+        else:
+            work(stream_handle())
+        torch.cuda.synchronize()
+        for i, route in enumerate(routes):
+            ref = (oracle.moe_dispatch_dedup if dedup else oracle.moe_dispatch)(x, route, E, recv_capacity_rows=cap)
+            for r in range(R):
+                n = int(ref["counts"][:, r].sum())
+                assert np.array_equal(meta[i][r].cpu().numpy().view(np.int32).reshape(cap, 4)[:n], ref["meta"][r][:n]), (i, r)
+                assert np.array_equal(recv[i][r].cpu().numpy().view(np.uint16).reshape(cap, H)[:n], ref["recv"][r][:n]), (i, r)
+    finally:
+        B.pl_schedule_destroy(sched)
+        B.pl_comm_destroy(ids)
+        run.close()
