@@ -526,13 +526,8 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   if (!comm->planner && rq.n_layers <= 1 && S->L.n_flags == 0 && !rq.staged && !S->trace && !S->layer_kernel && !S->ring && all_default) {
     bool reduce = false, all = false;
     const bool plan = flat_plan(S->L, comm->R, comm->dtype, &S->flat_spans, &reduce, &all);
-    // A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a short
-    // one (8 x 1 MiB 7.0 us, flat 7.5, with residual 7.1 / 8.0; 4 x 1 MiB 4.7 / 6.4; at 4 x 4 MiB flat is ahead,
-    // 11.3 / 12.8), and a streaming one without residual (8 x 64 MiB 267 us, flat 286; 4 x 64 MiB 139 / 148; 16 x
-    // 64 MiB 549 / 570; with residual flat is ahead, 325 / 505).
-    const bool wide = plan && reduce && all && comm->dtype == PL_BF16 && (hook & PL_HOOK_F32_OUT) &&
-                      (S->L.message_bytes * (uint64_t)comm->R <= (8u << 20) || (pol.datapath == PL_DP_TMA && !(hook & PL_HOOK_RESIDUAL)));
-    if (plan && !wide) {
+    const bool queues = plan && queues_faster(comm->R, comm->dtype, hook, rq.algo, reduce, all, pol.datapath == PL_DP_TMA, S->L.message_bytes);
+    if (plan && !queues) {
       uint64_t units = 0, blocks = 0;
       for (const FlatSpan& f : S->flat_spans) units += f.units;
       S->flat_launch = flat_launch(comm->R, reduce, all, pol.datapath == PL_DP_TMA, hook, units);

@@ -242,6 +242,9 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
 // The ops of a schedule without flags as spans; false if they are not of the forms a span describes.
 // `reduce` / `all` receive the one kind of op the schedule holds.  first_block is left to the caller.
 bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all);
+// True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
+// tma: the policy picked the bulk-copy datapath (the working set streams from HBM).
+bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes);
 LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster);
 Policy default_policy(const BuildRequest& rq, int max_resident_ctas);
 

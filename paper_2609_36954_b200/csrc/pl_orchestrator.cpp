@@ -1293,6 +1293,31 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
   return !spans->empty();
 }
 
+// A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a short
+// one (8 x 1 MiB 7.0 us, flat 7.5, with residual 7.1 / 8.0; 4 x 1 MiB 4.7 / 6.4; at 4 x 4 MiB flat is ahead,
+// 11.3 / 12.8), and a streaming one without residual (8 x 64 MiB 267 us, flat 286; 4 x 64 MiB 139 / 148; 16 x
+// 64 MiB 549 / 570; with residual flat is ahead, 325 / 505).
+// A one-shot all-reduce reads every input once per rank.  Flat, the tiles go out destination by
+// destination, so every sweep passes over all inputs; the op list has the destinations of a chunk next
+// to one another, which lets all reads but the first hit L2 when the inputs do not fit it.  us, queues /
+// flat, by MiB of all inputs: bf16 8 x 8 MiB (64) 68 / 51, 12 x 6 (72) 92 / 113, 16 x 5 (80) 142 / 158, 8 x 12 (96)
+// 100 / 124, 8 x 16 124 / 170, 8 x 256 1866 / 2664, 4 x 64 145 / 188, 2 x 256 191 / 231; int32, whose adds are
+// cheaper, 16 x 5 (80) 137 / 111, 13 x 7 (91) 141 / 161.  With a processing phase the register queues take
+// twice as long, and the line is where the queues use bulk copies (8 x 12 MiB residual 175 / 141, 8 x 16 MiB
+// 156 / 189).  Float sums of 12 and 16 ranks leave half of flat's registers idle while 144 queues
+// divide evenly among them: 12 x 768 KiB bf16 10 / 14, 12 x 3 MiB 47 / 52, 16 x 512 KiB 12.3 / 14.1, while 13 ranks
+// take 16.4 / 15.1 and 73 / 58.
+bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes) {
+  if (!reduce) return false;
+  const uint64_t inputs = message_bytes * (uint64_t)R, mib = 1u << 20;
+  if (all) return dtype == PL_BF16 && (hook & PL_HOOK_F32_OUT) && (inputs <= 8 * mib || (tma && !(hook & PL_HOOK_RESIDUAL)));
+  if (algo != PL_ALGO_ONESHOT) return false;
+  if (hook) return tma;
+  if (tma || inputs >= (dtype == PL_I32 ? 88 : 72) * mib) return true;
+  if (dtype == PL_I32 || (R != 12 && R != 16)) return false;
+  return (inputs >= 6 * mib && inputs <= 10 * mib) || (R == 12 && inputs >= 18 * mib);
+}
+
 int level_width(const Lowered& L, int R) {
   // level of an op = length of the longest chain of flag edges that ends in it
   std::vector<int> flag_level(L.n_flags, 0);

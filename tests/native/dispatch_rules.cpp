@@ -1,0 +1,48 @@
+// The host-only rules that pick an executor and its launch, callable from a test without a GPU.
+#include <vector>
+
+#include "pl_internal.h"
+
+using namespace pl;
+
+extern "C" {
+
+// Lowers a collective, lays its ops out for the flat executor and returns the number of spans (at most `cap`
+// written as src_off, dst_off, units, source rank, destination rank; 255 = every rank), -1 if the ops are not of that
+// form, -2 if the request is refused.
+int t_flat_plan(int R, int dtype, int coll, int algo, uint64_t count, uint64_t chunk, const uint64_t* counts_v, int root, uint32_t hook,
+                uint64_t* spans, int cap, int* reduce, int* all) {
+  BuildRequest rq{};
+  rq.R = R;
+  rq.dtype = dtype;
+  rq.coll = coll;
+  rq.algo = algo;
+  rq.count_per_rank = count;
+  rq.chunk_bytes = chunk;
+  rq.counts_v = counts_v;
+  rq.root = root;
+  rq.hook = hook;
+  rq.sm_count = 148;
+  rq.pol = default_policy(rq, 148);
+  Lowered L;
+  std::string err;
+  if (lower(rq, &L, &err) != PL_OK) return -2;
+  bool r = false, a = false;
+  std::vector<FlatSpan> f;
+  if (!flat_plan(L, R, dtype, &f, &r, &a)) return -1;
+  *reduce = r;
+  *all = a;
+  for (int i = 0; i < (int)f.size() && i < cap; ++i) {
+    spans[5 * i] = f[i].src_off;
+    spans[5 * i + 1] = f[i].dst_off;
+    spans[5 * i + 2] = f[i].units;
+    spans[5 * i + 3] = f[i].ranks & 0xFFu;
+    spans[5 * i + 4] = (f[i].ranks >> 8) & 0xFFu;
+  }
+  return (int)f.size();
+}
+
+int t_queues_faster(int R, int dtype, uint32_t hook, int algo, int reduce, int all, int tma, uint64_t message_bytes) {
+  return queues_faster(R, dtype, hook, algo, reduce, all, tma, message_bytes);
+}
+}

@@ -1,0 +1,39 @@
+"""The rules that pick an executor, on the CPU: the host-only part of the library compiled with g++."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2609_36954_b200 import binding as B
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+MIB = 1 << 20
+
+
+@pytest.fixture(scope="session")
+def rules(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("rules") / "rules.so")
+    csrc = os.path.join(ROOT, "paper_2609_36954_b200", "csrc")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", csrc, "-o", out,
+                    os.path.join(csrc, "pl_orchestrator.cpp"), os.path.join(ROOT, "tests", "native", "dispatch_rules.cpp")], check=True)
+    L = C.CDLL(out)
+    u64, i, u32, p = C.c_uint64, C.c_int, C.c_uint32, C.c_void_p
+    L.t_flat_plan.argtypes = [i, i, i, i, u64, u64, p, i, u32, p, i, p, p]
+    L.t_queues_faster.argtypes = [i, i, u32, i, i, i, i, u64]
+    return L
+
+
+# MiB of a message, R: a one-shot all-reduce whose inputs do not fit L2 is left to the queues, which read them
+# once; one that fits is not.
+@pytest.mark.parametrize("R,mib,dtype,hook,queues", [
+    (8, 256, "bf16", 0, 1), (8, 16, "bf16", 0, 1), (8, 12, "f32", 0, 1), (8, 8, "bf16", 0, 0), (8, 1, "bf16", 0, 0), (4, 64, "i32", 0, 1),
+    (2, 16, "bf16", 0, 0), (16, 5, "bf16", 0, 1), (16, 5, "i32", 0, 0), (16, 6, "i32", 0, 1), (8, 16, "bf16", B.PL_HOOK_RESIDUAL, 1),
+    (8, 12, "bf16", B.PL_HOOK_RESIDUAL, 0), (12, 0.75, "bf16", 0, 1), (13, 0.75, "bf16", 0, 0), (16, 0.5, "f32", 0, 1), (16, 1, "bf16", 0, 0)])
+def test_one_shot_all_reduce_stays_on_the_queues_where_they_are_faster(rules, R, mib, dtype, hook, queues):
+    dt = {"bf16": B.PL_BF16, "f32": B.PL_F32, "i32": B.PL_I32}[dtype]
+    tma = 2 * R * mib * MIB >= 256 * MIB
+    assert rules.t_queues_faster(R, dt, hook, B.PL_ALGO_ONESHOT, 1, 0, tma, int(mib * MIB)) == queues
+    # the same sizes without a second reading of the inputs
+    assert rules.t_queues_faster(R, dt, hook, B.PL_ALGO_DIRECT_FUSED, 1, 1, tma, int(mib * MIB)) == 0
