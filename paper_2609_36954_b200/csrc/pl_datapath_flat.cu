@@ -18,7 +18,10 @@
 //   bulk copy  streaming from HBM: one bulk asynchronous load per operand and tile into shared
 //              memory; reduce ops add from there and store from registers, copies leave by bulk
 //              stores.  Several CTAs per SM take the place of a ring of slots.
-// Copies store evict-first, which keeps what the next launch reads in L2.
+// Bulk copies store evict-first, which keeps in L2 what the next launch reads of a stream's inputs.  The
+// register form stores plainly: its results fit L2, and whoever reads them next finds them there (8 x 8 MiB
+// all-gather and a reader of the results 44.9 us evict-first, 39.7 plain; 8 x 4 MiB 28.7 / 25.4; back to back without a
+// reader evict-first is ahead, 12.5 / 13.0 and 6.6 / 7.3).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -72,10 +75,6 @@ __device__ __forceinline__ uint4 ld16_hint(const void* p, uint64_t policy) {
   asm volatile("ld.global.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
   return v;
 }
-__device__ __forceinline__ void st16_hint(void* p, const uint4& v, uint64_t policy) {
-  asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "l"(policy) : "memory");
-}
-
 template <int DT>
 __device__ __forceinline__ void add_unit(Acc<DT>& acc, const uint4& q) {
   if constexpr (DT == PL_BF16) acc.add_bf16(q);
@@ -174,7 +173,7 @@ template <int U, bool ALL>
 __global__ void __launch_bounds__(kFlatThreads) pl_flat_copy_kernel(const __grid_constant__ FlatParams P) {
   pdl_launch_dependents();
   const Tile t = my_tile(P);
-  const uint64_t policy = ptx::policy_evict_first();
+  const uint64_t policy = (P.hints & 1u) ? ptx::policy_evict_first() : 0ull;
   pdl_wait();
   const char* src = static_cast<const char*>(P.in[src_rank(t.span)]) + (t.span.src_off + t.first) * 16ull;
   const uint64_t at = (t.span.dst_off + t.first) * 16ull;
@@ -189,10 +188,7 @@ __global__ void __launch_bounds__(kFlatThreads) pl_flat_copy_kernel(const __grid
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       const uint32_t u = threadIdx.x + (uint32_t)(j * kFlatThreads);
-      if (u < t.units) {
-        if (P.hints & 2u) st16_hint(dst + u * 16ull, q[j], policy);
-        else st16(dst + u * 16ull, q[j]);
-      }
+      if (u < t.units) st16(dst + u * 16ull, q[j]);
     }
   };
   if constexpr (ALL) {

@@ -85,3 +85,38 @@ def test_variable_sizes_and_rooted(scale):
     # 256 spans, those between different ranks a single vector
     one = [[8 if p != r else 8 * 50 * scale for r in range(16)] for p in range(16)]
     same_bits(16, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, one, 4096, o))
+
+
+def test_results_that_fit_l2_stay_there():
+    """What a caller reads next must not be the first to leave L2: an all-gather of 8 x 8 MiB and a reader of its
+    results take as long as with PL_OPT_NO_L2_HINTS (stored evict-first they took 12 % longer)."""
+    R, n = 8, 4 * MIB
+    comm = B.pl_comm_create(R, DT["bf16"])
+    scheds = [B.pl_schedule_build(comm, B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n // R, MIB, B.make_opts(flags=f)) for f in (0, B.PL_OPT_NO_L2_HINTS)]
+    try:
+        info = B.pl_schedule_info(scheds[0])
+        assert info.datapath == B.PL_DP_LDST and info.grid != info.n_queues
+        sets = []
+        for _ in range(3):
+            x, y = [torch.randn(n // R, device="cuda").bfloat16() for _ in range(R)], torch.empty(R * n, dtype=torch.bfloat16, device="cuda")
+            sets.append((x, y, B.make_bufs([t.data_ptr() for t in x], [y[r * n:].data_ptr() for r in range(R)], [2 * n // R] * R, [2 * n] * R)))
+        top = torch.empty(64, dtype=torch.bfloat16, device="cuda")
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        times = ([], [])
+        for rep in range(12):  # both in turn
+            for k, s in enumerate(scheds):
+                t0.record()
+                for _ in range(20):
+                    for _, y, bufs in sets:
+                        B.pl_execute(s, bufs, stream_handle())
+                        torch.amax(y.view(64, -1), 1, out=top)
+                t1.record()
+                torch.cuda.synchronize()
+                if rep >= 2:
+                    times[k].append(t0.elapsed_time(t1))
+        default, plain = (sorted(t)[len(t) // 2] for t in times)
+        assert default <= 1.06 * plain, (default, plain)
+    finally:
+        for s in scheds:
+            B.pl_schedule_destroy(s)
+        B.pl_comm_destroy(comm)
