@@ -1307,9 +1307,13 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
 // 156 / 189).  Float sums of 12 and 16 ranks leave half of flat's registers idle while 144 queues
 // divide evenly among them: 12 x 768 KiB bf16 10 / 14, 12 x 3 MiB 47 / 52, 16 x 512 KiB 12.3 / 14.1, while 13 ranks
 // take 16.4 / 15.1 and 73 / 58.
+// An all-gather of more than 8 ranks stores every unit more than 8 times; between 10 and 36 MiB written the
+// queues, which keep 144 CTAs at it, are ahead (us, queues / flat: 16 x 768 KiB 3.7 / 8.5, 1 MiB 4.3 / 9.4, 2 MiB 7.8 /
+// 11.1, 3 MiB 10.0 / 11.4, 4 MiB 13.2 / 14.0; 14 x 1 MiB 4.1 / 8.5; 12 x 1 MiB 3.7 / 7.1, 4 MiB 10.3 / 10.9); below both
+// are bound by the launch, above by HBM (16 x 8 MiB 26.7 / 23.5).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes) {
-  if (!reduce) return false;
   const uint64_t inputs = message_bytes * (uint64_t)R, mib = 1u << 20;
+  if (!reduce) return all && !tma && R > 8 && inputs >= 10 * mib && inputs <= 36 * mib;  // a gathered message: bytes written
   if (all) return dtype == PL_BF16 && (hook & PL_HOOK_F32_OUT) && (inputs <= 8 * mib || (tma && !(hook & PL_HOOK_RESIDUAL)));
   if (algo != PL_ALGO_ONESHOT) return false;
   if (hook) return tma;

@@ -37,3 +37,11 @@ def test_one_shot_all_reduce_stays_on_the_queues_where_they_are_faster(rules, R,
     assert rules.t_queues_faster(R, dt, hook, B.PL_ALGO_ONESHOT, 1, 0, tma, int(mib * MIB)) == queues
     # the same sizes without a second reading of the inputs
     assert rules.t_queues_faster(R, dt, hook, B.PL_ALGO_DIRECT_FUSED, 1, 1, tma, int(mib * MIB)) == 0
+
+
+# KiB gathered, R: between 10 and 36 MiB written in all, more than 8 ranks gather on the queues
+@pytest.mark.parametrize("R,kib,queues", [(16, 1024, 1), (16, 2048, 1), (16, 512, 0), (16, 8192, 0), (14, 1024, 1), (12, 1024, 1), (8, 2048, 0), (4, 4096, 0)])
+def test_all_gather_of_many_ranks_stays_on_the_queues_where_they_are_faster(rules, R, kib, queues):
+    for tma in (0, 1):
+        assert rules.t_queues_faster(R, B.PL_BF16, 0, B.PL_ALGO_DIRECT, 0, 1, tma, kib << 10) == (queues and not tma)
+        assert rules.t_queues_faster(R, B.PL_BF16, 0, B.PL_ALGO_DIRECT, 0, 0, tma, kib << 10) == 0  # all-to-all
