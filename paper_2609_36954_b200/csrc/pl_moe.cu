@@ -746,6 +746,12 @@ __device__ __forceinline__ uint4 round_row(const float (&acc)[8]) {
   return o;
 }
 
+// Neither combine kernel releases its dependents: the launch behind it is set up as its CTAs exit.  Released
+// earlier, the few CTAs of the next dispatch's bookkeeping all crowd on the first SM that has room and share
+// it (dispatch and combine, 256 experts, top-8, released at the start / at the end: 8 x 256 tokens of 14 KiB 120 / 103 us,
+// of 1 KiB 38 / 20, 8 x 1024 of 4 KiB 132 / 115, 16 x 256 of 14 KiB 203 / 187; one-launch dispatch 8 x 8 of 14 KiB 13.3 / 7.9;
+// nothing is slower).
+//
 // combine: CTA per token (grid-strided), 16-byte column units across threads, the K source
 // rows and gates of the next token are fetched while the current one is summed.
 __global__ void __launch_bounds__(kCombineThreads) moe_combine_kernel(const __grid_constant__ CombinePtrs P, const __grid_constant__ MoeGeo g) {
@@ -773,9 +779,6 @@ __global__ void __launch_bounds__(kCombineThreads) moe_combine_kernel(const __gr
   for (int it = 0; tok < n_tok; tok += gridDim.x, ++it) {
     const int buf = it & 1;
     if (tok + gridDim.x < n_tok) load_meta(tok + gridDim.x, buf ^ 1);
-    // Last token of this CTA.  Released at the start instead, the next dispatch's bookkeeping sits on a few
-    // SMs for the whole launch (8 x 1024 tokens, dispatch and combine: 361 us, 344 with the release here).
-    else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int p = (int)(tok / g.T);
     char* out = static_cast<char*>(P.out[p]) + (tok % g.T) * g.row_bytes;
     for (uint32_t u = tid; u < units; u += kCombineThreads) {
@@ -811,7 +814,6 @@ __global__ void __launch_bounds__(kCombinePartThreads) moe_combine_parts_kernel(
   __shared__ const char* s_row[kTokens][kMaxTopk];
   __shared__ float s_gate[kTokens][kMaxTopk];
   const uint32_t sub = threadIdx.x / width, tid = threadIdx.x - sub * width;  // token of this CTA, thread of that token
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   uint32_t tok, part = 0;
   if (parts > 1) {
     tok = blockIdx.x / parts;
