@@ -245,6 +245,9 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
 // True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
 // tma: the policy picked the bulk-copy datapath (the working set streams from HBM).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes);
+// MoE combine: CTAs work on parts of a row (else a CTA takes whole token rows in turn).  units: 16-byte units of
+// a row; turns: CTAs of the other kernel that are resident at once.
+bool combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns);
 LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster);
 Policy default_policy(const BuildRequest& rq, int max_resident_ctas);
 

@@ -1121,17 +1121,11 @@ pl_status_t pl_moe_dispatch(pl_moe_plan_t plan, const void* const* x, const int3
   return PL_OK;
 }
 
-// Launched overlapped like the register executor: both kernels wait for everything in front before
-// they read.  Few tokens go by parts: a token per CTA turn leaves the last turn of a short launch
-// nearly empty, while at many tokens it hides the lookup of the next token's rows (B200, R = 8,
-// 7168 x bf16, top-8, turns -> parts: 64 tokens per rank 15.9 -> 13.9 us, 256 47.5 -> 45.0, 1024
-// 161 -> 168, 4096 611 -> 659).  So do rows of at most 256 units, which leave threads of a turn
-// idle or in flight with one unit (8 x 4096 tokens: 64 units top-8 145 -> 52 us, top-2 113 -> 23,
-// 256 units top-4 148 -> 120; 512 units top-6 291 -> 330, which is where the line lies).
+// Launched overlapped like the register executor: both kernels wait for everything in front before they read.
 static bool launch_combine(pl_moe_plan_t plan, const CombinePtrs& P, const MoeGeo& g, cudaStream_t cs) {
   const uint32_t units = g.row_bytes >> 4, parts = (units + kCombinePartThreads - 1) / kCombinePartThreads;
   const unsigned long long n_tok = (unsigned long long)g.R * g.T, turns = (unsigned long long)plan->sm_count * plan->combine_per_sm;
-  const bool by_parts = (n_tok < 8 * turns || units <= 256) && n_tok * parts <= 0x7FFFFFFFull;
+  const bool by_parts = combine_by_parts(n_tok, units, g.K, turns) && n_tok * parts <= 0x7FFFFFFFull;
   const uint32_t width = ((units + parts - 1) / parts + 31) / 32 * 32, tokens = parts > 1 ? 1u : kCombinePartThreads / width;
   if (!by_parts) return launch_after(true, moe_combine_kernel, dim3((unsigned)std::min(n_tok, turns)), kCombineThreads, 0, cs, P, g);
   return launch_after(true, g.K <= 2 ? moe_combine_parts_kernel<2> : g.K <= 4 ? moe_combine_parts_kernel<4> : moe_combine_parts_kernel<8>,

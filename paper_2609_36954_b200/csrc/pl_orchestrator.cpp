@@ -1322,6 +1322,20 @@ bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool 
   return (inputs >= 6 * mib && inputs <= 10 * mib) || (R == 12 && inputs >= 18 * mib);
 }
 
+// Few tokens go by parts: a token per CTA turn leaves the last turn of a short launch nearly empty, while at
+// many tokens it hides the lookup of the next token's rows.  us, turns / parts, 8 ranks, top-8, by tokens per rank: rows
+// of 14 KiB 128 24.5 / 24.9, 256 45.6 / 45.6, 512 83 / 87, 1024 160 / 171; of 24 KiB 64 20.4 / 22.1, 128 37.6 / 40.2,
+// 512 135 / 148; of 32 KiB 256 94 / 100, deduplicated 71 / 82; top-4, 4 ranks, 24 KiB 1024 82 / 92; top-2 14 KiB 1024 80 / 87: the line
+// lies at about 200 MB of rows read, where the launch is bound by HBM and not by its turns.  A second turn that is
+// less than half full is the exception (768 tokens, 592 turns: 32 KiB 41.5 / 39.8).  Rows of at most 256 units go by
+// parts whatever their number: they leave threads of a turn idle or in flight with one unit (8 x 4096 tokens: 64 units
+// top-8 145 -> 52 us, top-2 113 -> 23, 256 units top-4 148 -> 120; 512 units top-6 291 -> 330).
+bool combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns) {
+  if (units <= 256) return true;
+  if (n_tok >= 8 * turns) return false;
+  return n_tok * units * (uint64_t)topk < 12500000ull || (n_tok > turns && 2 * n_tok < 3 * turns);
+}
+
 int level_width(const Lowered& L, int R) {
   // level of an op = length of the longest chain of flag edges that ends in it
   std::vector<int> flag_level(L.n_flags, 0);

@@ -45,4 +45,6 @@ int t_flat_plan(int R, int dtype, int coll, int algo, uint64_t count, uint64_t c
 int t_queues_faster(int R, int dtype, uint32_t hook, int algo, int reduce, int all, int tma, uint64_t message_bytes) {
   return queues_faster(R, dtype, hook, algo, reduce, all, tma, message_bytes);
 }
+
+int t_combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns) { return combine_by_parts(n_tok, units, topk, turns); }
 }

@@ -22,6 +22,7 @@ def rules(tmp_path_factory):
     u64, i, u32, p = C.c_uint64, C.c_int, C.c_uint32, C.c_void_p
     L.t_flat_plan.argtypes = [i, i, i, i, u64, u64, p, i, u32, p, i, p, p]
     L.t_queues_faster.argtypes = [i, i, u32, i, i, i, i, u64]
+    L.t_combine_by_parts.argtypes = [u64, u32, i, u64]
     return L
 
 
@@ -45,3 +46,11 @@ def test_all_gather_of_many_ranks_stays_on_the_queues_where_they_are_faster(rule
     for tma in (0, 1):
         assert rules.t_queues_faster(R, B.PL_BF16, 0, B.PL_ALGO_DIRECT, 0, 1, tma, kib << 10) == (queues and not tma)
         assert rules.t_queues_faster(R, B.PL_BF16, 0, B.PL_ALGO_DIRECT, 0, 0, tma, kib << 10) == 0  # all-to-all
+
+
+# tokens of all ranks, KiB of a row, slots: a combine that reads about 200 MB or more takes whole rows in turn
+@pytest.mark.parametrize("tokens,kib,topk,parts", [
+    (1024, 32, 8, 0), (4096, 32, 8, 0), (4096, 24, 4, 0), (4096, 14, 8, 0), (1024, 24, 8, 0), (768, 32, 8, 1), (512, 14, 8, 1), (1024, 14, 8, 1),
+    (8, 32, 8, 1), (1024, 32, 2, 1), (32768, 4, 8, 1), (32768, 14, 8, 0)])
+def test_combine_of_wide_rows_takes_turns(rules, tokens, kib, topk, parts):
+    assert rules.t_combine_by_parts(tokens, kib * 64, topk, 592) == parts
