@@ -245,6 +245,13 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
 // True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
 // tma: the policy picked the bulk-copy datapath (the working set streams from HBM).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes);
+// ---- MoE dispatch in one launch (moe_small_kernel): its limits, and the tokens per CTA (0: not used) ----
+constexpr int kSmallThreads = 256;
+constexpr int kSmallOwn = 1024;       // most entries (T x K) of a source in a plan dispatched this way
+constexpr int kSmallExperts = 1024;
+constexpr int kSmallTargets = 64;     // most (token, slot) pairs of one CTA
+constexpr size_t kSmallSmemMax = 64 * 1024;
+uint32_t small_dispatch_rows(bool dedup, int R, int tokens, int topk, int experts, size_t row_bytes, int sm_count);
 // MoE combine: CTAs work on parts of a row (else a CTA takes whole token rows in turn).  units: 16-byte units of
 // a row; turns: CTAs of the other kernel that are resident at once.
 bool combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns);

@@ -382,18 +382,11 @@ __global__ void __launch_bounds__(256) moe_derive_ranks_kernel(const __grid_cons
 // Each CTA reads all routing in front of its own (16 KiB of indices at 8 x 64 tokens x 8 slots),
 // so nothing is counted, published and read back between launches or across a grid barrier.  A
 // dispatch of this size is bound by its chain (indices from DRAM, counting, rows out) and by the
-// launches (B200, R = 8, 7168 x bf16, top-8, two launches -> one: 1 token per rank 15.6 -> 6.4 us,
-// 64 tokens 25.4 -> 18 us; deduplicated 31 -> 16 us).  The line lies where a CTA's share of the
-// routing costs more than the grid barrier (256 tokens: 57 us in two launches, 70 us in one).
+// launches; small_dispatch_rows() says where it is used.
 // The row of (p, t, j) at rank r = entries of sources before p that go to r, plus entries of p that
 // go to r with a lower expert, or with the same expert and an earlier token.
 // DEDUP: an entry is (token, destination rank); the row is the number of earlier tokens, over
 // sources and then tokens, with a slot on r.
-constexpr int kSmallThreads = 256;
-constexpr int kSmallOwn = 1024;       // most entries (T x K) of a source in a plan dispatched this way
-constexpr int kSmallExperts = 1024;
-constexpr int kSmallTargets = 64;     // most (token, slot) pairs of one CTA
-
 struct SmallParams {
   uint32_t rows;            // tokens per CTA
   int K0, epr0;             // DEDUP: slots per token and experts per rank of the routing
@@ -879,7 +872,6 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // it is raised once per device to the most any plan can ask for, so that creating a second,
 // smaller plan cannot lower it under the feet of the first.
 constexpr int kMaxExperts = 4096;
-constexpr size_t kSmallSmemMax = 64 * 1024;
 constexpr size_t kPlanSmemMax = 200 * 1024;  // the fused bookkeeping kernel is used while its tables fit this
 
 size_t plan_smem_bytes(const MoeGeo& g) {
@@ -911,7 +903,7 @@ struct pl_moe_plan_s {
   int sm_count = 148;
   int combine_per_sm = 4;  // resident CTAs of the combine kernel per SM (occupancy query at plan creation)
   bool fused = false, fused_dedup = false;  // bookkeeping in one launch (grid co-resident, tables fit shared memory)
-  uint32_t small_rows = 0;  // > 0: dispatched in one launch with this many tokens per CTA
+  uint32_t small_rows = 0, small_rows_dedup = 0;  // > 0: dispatched in one launch with this many tokens per CTA
   bool dispatched = false;
   // deduplicated variant: the same machinery run over "one expert per rank" routing
   MoeGeo gd{};
@@ -1039,17 +1031,8 @@ pl_status_t pl_moe_plan_create(pl_comm_t comm, int tokens_per_rank, int hidden, 
     };
     pl->fused = feasible(pl->g);
     pl->fused_dedup = feasible(pl->gd);
-    // One launch while a CTA's share of the routing stays small; rows of one tile only.
-    if ((unsigned long long)tokens_per_rank * topk <= kSmallOwn && n_experts <= kSmallExperts) {
-      for (uint32_t rows = 1; rows * (uint32_t)topk <= kSmallTargets && 128 + rows * row_bytes <= kSmallSmemMax; ++rows) {
-        // the fewest tokens per CTA with which all CTAs are resident at once
-        const unsigned long long per_sm = std::min<unsigned long long>(2048 / kSmallThreads, (220 * 1024) / (rows * row_bytes + 12 * 1024));
-        if ((unsigned long long)R * ((tokens_per_rank + rows - 1) / rows) + R + 1 <= per_sm * comm->sm_count) {
-          pl->small_rows = rows;
-          break;
-        }
-      }
-    }
+    pl->small_rows = small_dispatch_rows(false, R, tokens_per_rank, topk, n_experts, row_bytes, comm->sm_count);
+    pl->small_rows_dedup = small_dispatch_rows(true, R, tokens_per_rank, topk, n_experts, row_bytes, comm->sm_count);
   }
   comm->n_plans += 1;
   *out = pl;
@@ -1206,9 +1189,9 @@ pl_status_t pl_moe_dispatch_dedup(pl_moe_plan_t plan, const void* const* x, cons
     P.meta[r] = recv_meta ? recv_meta[r] : nullptr;
   }
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  if (plan->small_rows) {
+  if (plan->small_rows_dedup) {
     for (int r = 0; r < g.R; ++r) P.idx[r] = topk_idx[r];
-    if (!launch_small(P, d, SmallParams{plan->small_rows, g.K, g.epr, plan->d_ridx, plan->d_rmask}, true, cs)) return PL_ERR_CUDA;
+    if (!launch_small(P, d, SmallParams{plan->small_rows_dedup, g.K, g.epr, plan->d_ridx, plan->d_rmask}, true, cs)) return PL_ERR_CUDA;
     g_launches.fetch_add(1);
     plan->dispatched_dedup = true;
     return PL_OK;

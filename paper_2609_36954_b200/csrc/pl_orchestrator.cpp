@@ -1322,6 +1322,24 @@ bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool 
   return (inputs >= 6 * mib && inputs <= 10 * mib) || (R == 12 && inputs >= 18 * mib);
 }
 
+// One launch while a CTA's share of the routing stays small, rows of one tile only (R = 8, 7168 x bf16, top-8, two
+// launches -> one: 1 token per rank 15.6 -> 6.4 us, 64 tokens 25.4 -> 18 us; deduplicated 31 -> 16 us).  The line lies
+// where a CTA's share of the routing costs more than the grid barrier (256 tokens: 57 us in two launches, 70
+// us in one); deduplicated, where the entries in front of a token are found token by token, at 2048 tokens of all ranks
+// (8 ranks, top-2, 384 tokens 16.5 / 22.0 us, 512 tokens 19.0 / 27.7).
+// Rows of 24 and 32 KiB stay with it: 8 x 16 tokens of 32 KiB dispatched over and over take 23.4 us in one launch and 15.2
+// in two, but dispatch and combine in turn, which is how they are called, 20.0 and 25.6 (8 x 32 of 24 KiB 25.6 / 32.0).
+uint32_t small_dispatch_rows(bool dedup, int R, int tokens, int topk, int experts, size_t row_bytes, int sm_count) {
+  if ((uint64_t)tokens * topk > kSmallOwn || experts > kSmallExperts) return 0;
+  if (dedup && (int64_t)R * tokens > 2048) return 0;
+  for (uint32_t rows = 1; rows * (uint32_t)topk <= kSmallTargets && 128 + rows * row_bytes <= kSmallSmemMax; ++rows) {
+    // the fewest tokens per CTA with which all CTAs are resident at once
+    const uint64_t per_sm = std::min<uint64_t>(2048 / kSmallThreads, (220 * 1024) / (rows * row_bytes + 12 * 1024));
+    if ((uint64_t)R * ((tokens + rows - 1) / rows) + R + 1 <= per_sm * sm_count) return rows;
+  }
+  return 0;
+}
+
 // Few tokens go by parts: a token per CTA turn leaves the last turn of a short launch nearly empty, while at
 // many tokens it hides the lookup of the next token's rows.  us, turns / parts, 8 ranks, top-8, by tokens per rank: rows
 // of 14 KiB 128 24.5 / 24.9, 256 45.6 / 45.6, 512 83 / 87, 1024 160 / 171; of 24 KiB 64 20.4 / 22.1, 128 37.6 / 40.2,

@@ -47,4 +47,8 @@ int t_queues_faster(int R, int dtype, uint32_t hook, int algo, int reduce, int a
 }
 
 int t_combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns) { return combine_by_parts(n_tok, units, topk, turns); }
+
+int t_small_dispatch_rows(int dedup, int R, int tokens, int topk, int experts, uint64_t row_bytes) {
+  return (int)small_dispatch_rows(dedup, R, tokens, topk, experts, row_bytes, 148);
+}
 }

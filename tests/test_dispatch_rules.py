@@ -23,6 +23,7 @@ def rules(tmp_path_factory):
     L.t_flat_plan.argtypes = [i, i, i, i, u64, u64, p, i, u32, p, i, p, p]
     L.t_queues_faster.argtypes = [i, i, u32, i, i, i, i, u64]
     L.t_combine_by_parts.argtypes = [u64, u32, i, u64]
+    L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
     return L
 
 
@@ -54,3 +55,15 @@ def test_all_gather_of_many_ranks_stays_on_the_queues_where_they_are_faster(rule
     (8, 32, 8, 1), (1024, 32, 2, 1), (32768, 4, 8, 1), (32768, 14, 8, 0)])
 def test_combine_of_wide_rows_takes_turns(rules, tokens, kib, topk, parts):
     assert rules.t_combine_by_parts(tokens, kib * 64, topk, 592) == parts
+
+
+# ranks, tokens per rank, slots, KiB of a row -> one launch, plain and deduplicated
+@pytest.mark.parametrize("R,T,K,kib,one,one_dedup", [
+    (8, 16, 8, 32, 1, 1), (8, 4, 8, 32, 1, 1), (8, 64, 8, 32, 1, 1),
+    (8, 64, 8, 14, 1, 1), (8, 16, 8, 14, 1, 1), (8, 128, 8, 14, 1, 1), (8, 129, 8, 14, 0, 0), (8, 256, 2, 4, 1, 1), (8, 384, 2, 4, 1, 0), (2, 1024, 1, 1, 1, 1),
+    (8, 8, 8, 80, 0, 0)])
+def test_one_launch_dispatch_where_it_is_faster(rules, R, T, K, kib, one, one_dedup):
+    rows = rules.t_small_dispatch_rows(0, R, T, K, 256, kib << 10), rules.t_small_dispatch_rows(1, R, T, K, 256, kib << 10)
+    assert (rows[0] > 0, rows[1] > 0) == (one, one_dedup)
+    assert all(r * K <= 64 and r * (kib << 10) <= 64 << 10 for r in rows)
+    assert rules.t_small_dispatch_rows(0, R, T, K, 2048, kib << 10) == 0
