@@ -436,7 +436,8 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   LayerShape layers{0, 0, false};
   const uint64_t layer_bytes = rq.count_per_rank * (uint64_t)elem_size(comm->dtype);
   if (rq.n_layers > 1 && rq.algo == PL_ALGO_DIRECT_FUSED && pol.datapath == PL_DP_LDST && requested == 0 && !rq.staged && comm->dtype != PL_U8 &&
-      (!opts || (opts->threads == 0 && opts->slice_bytes == 0)) && layer_bytes > 0 && layer_bytes % (16 * (uint64_t)comm->R) == 0) {
+      (!opts || (opts->threads == 0 && opts->slice_bytes == 0)) && layer_bytes > 0 && layer_bytes % (16 * (uint64_t)comm->R) == 0 &&
+      layer_executor_faster(comm->R, layer_bytes, hook != 0)) {
     layers = layer_shape(comm->R, layer_bytes, capacity, true);
     if (layers.cluster && !comm->planner && !layers_cluster_fits(comm->dtype, comm->R, hook != 0, layers.ctas_per_rank * comm->R, layers.threads))
       layers = layer_shape(comm->R, layer_bytes, capacity, false);
@@ -1235,6 +1236,7 @@ pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
     Y.in_stride = s->L.message_bytes;
     Y.out_stride = s->info.out_bytes[0] / (uint64_t)s->L.n_layers;
     Y.n_layers = (uint32_t)s->L.n_layers;
+    Y.ask_ahead = layer_asks_ahead(R, s->L.message_bytes);
     Y.break_layer = s->layer_break_layer;
     Y.break_queue = s->layer_break_queue;
   }

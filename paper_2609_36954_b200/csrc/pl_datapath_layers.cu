@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
       if (l + 1 < Y.n_layers) {
         topo += nq;
         // while the flag travels (asking two layers ahead measured the same)
-        ask_for_layer<NR>(P, in_off + Y.in_stride, units, tid, blockDim.x);
+        if (Y.ask_ahead) ask_for_layer<NR>(P, in_off + Y.in_stride, units, tid, blockDim.x);
       }
     }
     __syncthreads();

@@ -161,6 +161,7 @@ bool ring_shape(int R, int dtype, bool reduce, uint64_t part_units, int sm_count
 struct LayerParams {
   uint64_t in_stride, out_stride;
   uint32_t n_layers;
+  uint32_t ask_ahead;                 // ask the next layer's lines into L2
   int32_t break_layer, break_queue;  // test hook of the cluster variant (no wait entries to break), -1 = none
 };
 
@@ -256,6 +257,8 @@ uint32_t small_dispatch_rows(bool dedup, int R, int tokens, int topk, int expert
 // a row; turns: CTAs of the other kernel that are resident at once.
 bool combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns);
 LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster);
+bool layer_executor_faster(int R, uint64_t message_bytes, bool hook);  // than the register executor
+bool layer_asks_ahead(int R, uint64_t message_bytes);
 Policy default_policy(const BuildRequest& rq, int max_resident_ctas);
 
 }  // namespace pl

@@ -797,6 +797,18 @@ void a2a_direct_staged(Emitter& em, const Geo& g, uint64_t capacity) {
 // (the two values are two B200s) against 1.95, 64 KiB 2.16-2.24 against 1.96.  With flags as many
 // CTAs as there are slices of at least 32 units: 16, 32, 64 or 128 made no difference at 64 KiB
 // and above as long as every SM has a slice at the large end (1 MiB: 128 CTAs 3.6 us, 64 CTAs 5 us).
+// Lines of the next layer's inputs are asked into L2 ahead while they and what this layer writes have room there.
+// us for 20 layers with / without, by MiB of a layer's inputs: bf16 8 x 4 MiB (32) 245 / 257, 8 x 6 (48) 363 / 369, 4 x 12
+// (48) 412 / 404, 8 x 8 (64) 478 / 473, 16 x 4 (64) 487 / 484, 12 x 6 (72) 544 / 541, 16 x 6 (96) 748 / 720, 8 x 24 (192)
+// 1522 / 1431.
+bool layer_asks_ahead(int R, uint64_t message_bytes) { return (uint64_t)R * message_bytes < (64u << 20); }
+// With 12 ranks and more, and layers whose inputs do not fit L2 (128 MiB), the register executor streams better: 20
+// layers bf16, layer executor (asking ahead / not) / register, 16 x 8 MiB 1035 / 971 / 918 us, 16 x 12 1666 / 1499 / 1366, 12 x
+// 12 1156 / 1118 / 1034, 12 x 16 1585 / 1517 / 1552, while 12 x 8 753 / 733 / 740, 10 x 16 1282 / 1178 / 1368, 8 x 16 1024 /
+// 978 / 1062.  With a residual it is slower at every size (16 x 8 MiB 2140 / 1865 / 2316).
+bool layer_executor_faster(int R, uint64_t message_bytes, bool hook) {
+  return hook || R < 12 || (uint64_t)R * message_bytes < (128u << 20);
+}
 LayerShape layer_shape(int R, uint64_t message_bytes, int capacity, bool allow_cluster) {
   LayerShape s;
   const uint64_t units = std::max<uint64_t>(1, message_bytes / (uint64_t)R / 16);  // vectors of a rank's partition

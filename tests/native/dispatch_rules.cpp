@@ -51,4 +51,9 @@ int t_combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns)
 int t_small_dispatch_rows(int dedup, int R, int tokens, int topk, int experts, uint64_t row_bytes) {
   return (int)small_dispatch_rows(dedup, R, tokens, topk, experts, row_bytes, 148);
 }
+
+// bit 0: the layer executor runs it, bit 1: and asks for the next layer's lines
+int t_layers(int R, uint64_t message_bytes, int hook) {
+  return (layer_executor_faster(R, message_bytes, hook) ? 1 : 0) | (layer_asks_ahead(R, message_bytes) ? 2 : 0);
+}
 }

@@ -24,6 +24,7 @@ def rules(tmp_path_factory):
     L.t_queues_faster.argtypes = [i, i, u32, i, i, i, i, u64]
     L.t_combine_by_parts.argtypes = [u64, u32, i, u64]
     L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
+    L.t_layers.argtypes = [i, u64, i]
     return L
 
 
@@ -67,3 +68,10 @@ def test_one_launch_dispatch_where_it_is_faster(rules, R, T, K, kib, one, one_de
     assert (rows[0] > 0, rows[1] > 0) == (one, one_dedup)
     assert all(r * K <= 64 and r * (kib << 10) <= 64 << 10 for r in rows)
     assert rules.t_small_dispatch_rows(0, R, T, K, 2048, kib << 10) == 0
+
+
+# layers whose inputs do not fit L2: nothing is asked ahead, and with many ranks the register executor runs them
+@pytest.mark.parametrize("R,mib,hook,executor,ahead", [
+    (8, 1, 0, 1, 1), (16, 3, 0, 1, 1), (8, 8, 0, 1, 0), (16, 6, 0, 1, 0), (16, 8, 0, 0, 0), (16, 8, 1, 1, 0), (12, 12, 0, 0, 0), (12, 8, 0, 1, 0), (8, 24, 0, 1, 0)])
+def test_layers_that_stream(rules, R, mib, hook, executor, ahead):
+    assert rules.t_layers(R, mib * MIB, hook) == executor + 2 * ahead

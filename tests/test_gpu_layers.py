@@ -19,11 +19,11 @@ def as_f64(raw, dtype):
 
 # bytes of a rank's message: one vector per partition, two, a line and a vector, an odd number of
 # lines, the last size that runs as one cluster (R * bytes = 256 KiB) and the first that does not,
-# more units per slice than threads
+# more units per slice than threads, the lines of the next layer asked for and (from 64 MiB of inputs) not
 @pytest.mark.parametrize("R,dtype,nbytes", [
     (8, "bf16", 128), (8, "bf16", 8 * 32), (8, "i32", 8 * 144), (3, "bf16", 3 * 16 * 37), (8, "bf16", 32768), (8, "bf16", 32768 + 128),
     (2, "f32", 131072), (2, "f32", 131072 + 32), (16, "bf16", 16384), (16, "i32", 16384 + 256), (5, "f32", 5 * 16 * 1001),
-    (4, "bf16", 4 << 20)])
+    (4, "bf16", 4 << 20), (4, "bf16", (16 << 20) + 64 * 5)])
 def test_layers_match_oracle(R, dtype, nbytes):
     n, layers = nbytes // SIZE[dtype], 3
     x = [np.concatenate([gen.rank_inputs(R, n, dtype, seed=l)[r] for l in range(layers)]) for r in range(R)]
@@ -109,5 +109,23 @@ def test_tiny_layers_left_to_the_library(R, dtype, nbytes, want):
         a, _ = ses.execute(auto, x)
         b, _ = ses.execute(ses.build_layers(B.PL_ALGO_ONESHOT, n, layers, datapath=B.PL_DP_PACKET), x)
         assert all(np.array_equal(p, q) for p, q in zip(a, b))
+    finally:
+        ses.close()
+
+
+def test_layers_of_many_ranks_that_stream_run_on_the_register_executor():
+    R, n, layers = 16, 4 << 20, 2  # 8 MiB of bf16 per rank: 128 MiB of inputs a layer
+    ses = Session(R, "bf16")
+    try:
+        s = ses.build_layers(B.PL_ALGO_AUTO, n, layers)
+        assert len(B.pl_schedule_dump(s)) > layers * B.pl_schedule_info(s).n_queues  # the layer executor has one op per queue and layer
+        x = [torch.randint(-8, 8, (layers * n,), device="cuda").bfloat16() for _ in range(R)]
+        y = [poison(2 * layers * n) for _ in range(R)]
+        size = [2 * layers * n] * R
+        B.pl_execute(s, B.make_bufs([t.data_ptr() for t in x], [t.data_ptr() for t in y], size, size), stream_handle())
+        torch.cuda.synchronize()
+        assert B.pl_comm_status(ses.comm).code == B.PL_OK
+        want = sum(t.float() for t in x).bfloat16()  # whole numbers: exact
+        assert all(torch.equal(t.view(torch.bfloat16), want) for t in y)
     finally:
         ses.close()
