@@ -519,7 +519,7 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
   if (!comm->planner && rq.algo == PL_ALGO_RING && !hook && !S->trace && all_default && rq.n_layers == 0) {
     const bool reduce = rq.coll != PL_ALLGATHER;
     const uint64_t part = rq.count_per_rank * (uint64_t)elem_size(comm->dtype) / (reduce ? (uint64_t)comm->R : 1ull) / 16;
-    S->ring = ring_shape(comm->R, comm->dtype, reduce, part, comm->sm_count, &S->ring_launch) &&
+    S->ring = ring_shape(comm->R, comm->dtype, reduce, rq.coll != PL_REDUCE_SCATTER, part, rq.chunk_bytes, comm->sm_count, &S->ring_launch) &&
               ring_prepare(comm->dtype, comm->R, S->ring_launch) > 0;
   }
   // No flags and nothing about the launch asked for: no queues.  Planner communicators keep the

@@ -154,7 +154,7 @@ struct RingLaunch {
   size_t smem_bytes;
 };
 // False where the op queues execute the ring better (or it has more tiles than a grid).
-bool ring_shape(int R, int dtype, bool reduce, uint64_t part_units, int sm_count, RingLaunch* L);
+bool ring_shape(int R, int dtype, bool reduce, bool gather, uint64_t part_units, uint64_t chunk_bytes, int sm_count, RingLaunch* L);
 
 // What the layer executor needs on top of ExecParams (see pl_datapath_layers.cu): the distance from
 // a layer's operands to the next layer's, in bytes.

@@ -1251,9 +1251,18 @@ void assign_queues(Lowered* L, int R, int n_queues, bool by_level) {
 // neighbours' shared memory saves.  us, clusters / queues, by bytes per rank: 8 ranks 1 MiB 28.3 / 34.3,
 // 8 MiB 197 / 155; 4 ranks 1 MiB 11.0 / 15.0, 8 MiB 61 / 50; 2 ranks 1 MiB 3.5 / 6.5, 2 MiB 5.3 / 4.8;
 // 16 ranks 256 KiB 43 / 49, 1 MiB 121 / 116.
-bool ring_shape(int R, int dtype, bool reduce, uint64_t part_units, int sm_count, RingLaunch* L) {
+// A streaming all-reduce of int32 on more than 8 ranks, or of fp32 on more than 10, whose op list has a few chunks per
+// partition stays with the queues too: 2 R - 2 cluster barriers a tile cost more than what the partial sums save, which is
+// most for bf16.  us, clusters / queues: int32 16 x 64 MiB in chunks of 256 KiB 792 / 683, 12 x 64 581 / 512, 9 x 64 396 / 374, 8 x 64
+// 337 / 329, 12 x 128 (42 chunks) 1142 / 1067, 16 x 32 413 / 417, in chunks of 64 KiB 16 x 64 792 / 840; fp32 16 x 64 in 256 KiB 1115 / 1025, 16 x 32 570 / 531,
+// 12 x 32 407 / 387, 9 x 32 277 / 286, 12 x 128 (42 chunks) 1549 / 1563, 16 x 16 in 256 KiB 297 / 361, in 64 KiB 298 / 279; bf16 16 x 64 916 / 1003.
+bool ring_shape(int R, int dtype, bool reduce, bool gather, uint64_t part_units, uint64_t chunk_bytes, int sm_count, RingLaunch* L) {
   const uint64_t total = part_units * (uint64_t)R, mib = (1u << 20) / 16;
   if (!part_units || (!reduce && (part_units > mib || total > 8 * mib))) return false;
+  const uint64_t chunks = chunk_bytes ? part_units * 16 / chunk_bytes : 0;
+  const bool i32 = dtype == PL_I32;
+  if ((i32 ? R > 8 : dtype == PL_F32 && R > 10) && reduce && gather && chunks >= 2 && chunks <= (i32 ? 48 : 32) && total >= (i32 ? 60 : 30) * mib)
+    return false;
   L->units = 1;
   if (total <= 128ull * sm_count) {
     L->threads = (int)((total + sm_count - 1) / sm_count + 31) / 32 * 32;

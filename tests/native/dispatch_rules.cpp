@@ -56,4 +56,15 @@ int t_small_dispatch_rows(int dedup, int R, int tokens, int topk, int experts, u
 int t_layers(int R, uint64_t message_bytes, int hook) {
   return (layer_executor_faster(R, message_bytes, hook) ? 1 : 0) | (layer_asks_ahead(R, message_bytes) ? 2 : 0);
 }
+
+// 0 if the queues run the ring, else its threads, units per thread, tile and grid
+int t_ring_shape(int R, int dtype, int reduce, int gather, uint64_t part_units, uint64_t chunk_bytes, int* shape) {
+  RingLaunch L{};
+  if (!ring_shape(R, dtype, reduce, gather, part_units, chunk_bytes, 148, &L)) return 0;
+  shape[0] = L.threads;
+  shape[1] = L.units;
+  shape[2] = (int)L.tile;
+  shape[3] = L.grid;
+  return (int)L.smem_bytes;
+}
 }

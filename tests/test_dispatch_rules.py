@@ -25,6 +25,7 @@ def rules(tmp_path_factory):
     L.t_combine_by_parts.argtypes = [u64, u32, i, u64]
     L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
     L.t_layers.argtypes = [i, u64, i]
+    L.t_ring_shape.argtypes = [i, i, i, i, u64, u64, p]
     return L
 
 
@@ -75,3 +76,31 @@ def test_one_launch_dispatch_where_it_is_faster(rules, R, T, K, kib, one, one_de
     (8, 1, 0, 1, 1), (16, 3, 0, 1, 1), (8, 8, 0, 1, 0), (16, 6, 0, 1, 0), (16, 8, 0, 0, 0), (16, 8, 1, 1, 0), (12, 12, 0, 0, 0), (12, 8, 0, 1, 0), (8, 24, 0, 1, 0)])
 def test_layers_that_stream(rules, R, mib, hook, executor, ahead):
     assert rules.t_layers(R, mib * MIB, hook) == executor + 2 * ahead
+
+
+def ring(rules, R, dtype, coll, nbytes, chunk=MIB):
+    reduce, gather = coll != "ag", coll != "rs"
+    shape = (C.c_int * 4)()
+    part = nbytes // 16 if coll == "ag" else nbytes // R // 16
+    smem = rules.t_ring_shape(R, {"bf16": B.PL_BF16, "f32": B.PL_F32, "i32": B.PL_I32, "u8": B.PL_U8}[dtype], reduce, gather, part, chunk, shape)
+    return part, smem, list(shape)
+
+
+# ranks, type, MiB, KiB of a chunk: where the queues run a ring
+@pytest.mark.parametrize("R,dtype,coll,mib,kib,clusters", [
+    (16, "i32", "ar", 64, 256, 0), (16, "i32", "ar", 64, 1024, 0), (16, "i32", "ar", 64, 64, 1), (16, "i32", "rs", 64, 256, 1), (16, "i32", "ar", 32, 256, 1),
+    (9, "i32", "ar", 64, 1024, 0), (8, "i32", "ar", 64, 1024, 1), (16, "f32", "ar", 32, 256, 0), (12, "f32", "ar", 64, 1024, 0), (9, "f32", "ar", 64, 1024, 1), (12, "i32", "ar", 128, 256, 0), (16, "f32", "ar", 16, 64, 1),
+    (16, "f32", "ar", 16, 256, 1), (16, "bf16", "ar", 64, 1024, 1), (8, "f32", "ar", 256, 1024, 1), (2, "u8", "ag", 1, 64, 1), (2, "u8", "ag", 2, 64, 0)])
+def test_rings_that_stay_on_the_queues(rules, R, dtype, coll, mib, kib, clusters):
+    assert (ring(rules, R, dtype, coll, mib * MIB, kib << 10)[1] > 0) == clusters
+
+
+@pytest.mark.parametrize("R", [2, 3, 5, 8, 12, 16])
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "i32"])
+@pytest.mark.parametrize("units", [1, 31, 33, 257, 4099, 65539, 300007])
+def test_ring_tiles_cover_the_partition(rules, R, dtype, units):
+    for coll in ("rs", "ar"):
+        part, smem, (threads, per_thread, tile, grid) = ring(rules, R, dtype, coll, 16 * units * R, 1 << 30)
+        assert smem == tile * 16 * 2 * (1 if dtype == "i32" else 2) and smem <= 4 * 256 * 64
+        assert threads % 32 == 0 and 32 <= threads <= 256 and tile == threads * per_thread
+        assert grid % R == 0 and (grid // R - 1) * tile < part <= grid // R * tile
