@@ -1542,6 +1542,17 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
     std::vector<int> readers;
   };
   std::map<Key, std::map<uint64_t, Seg>> mem;
+  // Outputs that no op reads need no map: their ranges are collected and looked over once sorted (what
+  // makes up most of a layered schedule: 80 layers on 128 queues and 8 ranks 35 -> 4 ms).
+  bool outputs_read = false;
+  for (const HostOp& op : L.ops)
+    for (const pl_ref_t& s : op.src) outputs_read = outputs_read || s.buf == PL_BUF_OUT;
+  struct Written {
+    uint64_t lo, hi;
+    int writer;
+  };
+  std::vector<std::vector<Written>> written(R);
+  std::vector<Written> written_everywhere;  // by ops with a destination in every output
   // split so that `at` is a segment boundary
   auto split = [](std::map<uint64_t, Seg>& m, uint64_t at) {
     auto it = m.upper_bound(at);
@@ -1576,6 +1587,13 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
       }
     }
     const uint64_t b = op.count * elem_size(op.dst.dtype);
+    if (op.dst.buf == PL_BUF_OUT && !outputs_read) {
+      const Written w{op.dst.offset, op.dst.offset + b, (int)i};
+      if (b == 0) continue;
+      if (op.bcast) written_everywhere.push_back(w);
+      else written[op.dst.rank].push_back(w);
+      continue;
+    }
     for (int r = 0; r < R; ++r) {
       if (!op.bcast && r != op.dst.rank) continue;
       auto& m = mem[{op.dst.buf, r}];
@@ -1602,10 +1620,29 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
       m[lo] = Seg{hi, (int)i, {}};
     }
   }
+  auto by_offset = [](const Written& a, const Written& b) { return a.lo != b.lo ? a.lo < b.lo : a.writer < b.writer; };
+  std::sort(written_everywhere.begin(), written_everywhere.end(), by_offset);
   for (int r = 0; r < R; ++r) {
     uint64_t covered = 0;
     auto mit = mem.find({PL_BUF_OUT, r});
-    if (mit != mem.end())
+    if (!outputs_read) {
+      std::vector<Written> all;
+      const std::vector<Written>* w = &written_everywhere;
+      if (!written[r].empty()) {
+        all = written_everywhere;
+        all.insert(all.end(), written[r].begin(), written[r].end());
+        std::sort(all.begin(), all.end(), by_offset);
+        w = &all;
+      }
+      for (size_t k = 0; k < w->size(); ++k) {
+        if (k && (*w)[k].lo < (*w)[k - 1].hi) {
+          std::snprintf(msg, sizeof msg, "ops %d and %d write overlapping bytes of the output of rank %d", std::min((*w)[k - 1].writer, (*w)[k].writer),
+                        std::max((*w)[k - 1].writer, (*w)[k].writer), r);
+          return fail(msg);
+        }
+        if ((*w)[k].lo == covered) covered = (*w)[k].hi;
+      }
+    } else if (mit != mem.end())
       for (const auto& kv : mit->second) {
         if (kv.first != covered) break;
         covered = kv.second.hi;

@@ -1,4 +1,5 @@
 // The host-only rules that pick an executor and its launch, callable from a test without a GPU.
+#include <cstdio>
 #include <vector>
 
 #include "pl_internal.h"
@@ -66,5 +67,33 @@ int t_ring_shape(int R, int dtype, int reduce, int gather, uint64_t part_units, 
   shape[2] = (int)L.tile;
   shape[3] = L.grid;
   return (int)L.smem_bytes;
+}
+
+// Validates a lowered schedule after a change to op `which`: 0 none, 1 another op with the same destination, 2 the op's
+// output shortened by 16 bytes, 3 the op's destination moved up by 16 bytes.
+int t_validate_changed(int R, int dtype, int coll, int algo, uint64_t count, uint64_t chunk, int n_layers, int which, int change, char* msg, int cap) {
+  BuildRequest rq{};
+  rq.R = R;
+  rq.dtype = dtype;
+  rq.coll = coll;
+  rq.algo = algo;
+  rq.count_per_rank = count;
+  rq.chunk_bytes = chunk;
+  rq.n_layers = n_layers;
+  rq.sm_count = 148;
+  rq.pol = default_policy(rq, 148);
+  Lowered L;
+  std::string err;
+  if (lower(rq, &L, &err) != PL_OK) return -2;
+  HostOp& op = L.ops[which];
+  const HostOp copy = op;
+  const int es = copy.kind == PL_OP_COPY ? 1 : elem_size(dtype);
+  if (change == 2) op.count -= 16 / es;
+  if (change == 3) op.dst.offset += 16, op.count -= 16 / es;
+  if (change == 1) L.ops.insert(L.ops.begin() + which + 1, copy);
+  assign_queues(&L, R, rq.pol.n_ctas);
+  const pl_status_t st = validate(L, R, &err, false);
+  std::snprintf(msg, (size_t)cap, "%s", err.c_str());
+  return st;
 }
 }
