@@ -167,13 +167,15 @@ void fill_info(pl_schedule_s* S, int R) {
 }
 
 // Flatten the lowered ops into the device arrays (host side): op i of queue q at index
-// i * n_queues + q, queues padded to the longest one, empty queues get one placeholder.
+// i * n_queues + q, queues padded to the longest one, empty queues get one placeholder.  The layer executor
+// reads layer 0 only (one op per queue), so it is all that is laid out for it.
 void flatten(pl_schedule_s* S, int dtype) {
   const Lowered& L = S->L;
   const int nq = S->pol.n_ctas;
   size_t max_src = 1, max_wait = 1;
   std::vector<uint32_t> qlen(nq, 0);
   for (const HostOp& op : L.ops) {
+    if (S->layer_kernel && op.layer > 0) continue;
     max_src = std::max(max_src, op.src.size());
     max_wait = std::max(max_wait, op.waits.size());
     qlen[op.queue]++;
@@ -192,6 +194,7 @@ void flatten(pl_schedule_s* S, int dtype) {
   S->topo_to_dev.assign(L.ops.size(), 0);
   std::vector<uint32_t> cursor(nq, 0);
   for (const HostOp& op : L.ops) {  // topological order => per-queue order is a subsequence
+    if (S->layer_kernel && op.layer > 0) continue;
     const uint32_t i = cursor[op.queue]++;
     const size_t pos = (size_t)i * nq + op.queue;
     S->topo_to_dev[op.topo] = (int)pos;
@@ -217,6 +220,7 @@ void flatten(pl_schedule_s* S, int dtype) {
 }
 
 pl_status_t upload(pl_schedule_s* S, int R) {
+  if (S->ring) return PL_OK;  // sizes and pointers are all it reads
   if (S->flat) {
     S->blob_bytes = S->flat_spans.size() * sizeof(FlatSpan);
     if (cudaMalloc(&S->d_blob, S->blob_bytes) != cudaSuccess) { cudaGetLastError(); return PL_ERR_OOM; }
@@ -250,7 +254,7 @@ pl_status_t upload(pl_schedule_s* S, int R) {
   uint64_t total = 0;
   for (int r = 0; r < R; ++r) {
     S->scratch_off[r] = total;
-    if (!S->ring) total += align_up(S->L.scratch_per_rank[r], 256);
+    total += align_up(S->L.scratch_per_rank[r], 256);
   }
   if (S->stage_ahead) {  // second staging buffer of every rank, one half behind the first
     S->scratch_half = total;
@@ -563,7 +567,7 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
       if (sm < S->pol.idle_first || sm >= S->pol.idle_first + S->pol.idle_count) S->sm_mask[sm >> 5] |= 1u << (sm & 31);
   }
   fill_info(S, comm->R);
-  if (!S->flat) flatten(S, comm->dtype);
+  if (!S->flat && !S->ring) flatten(S, comm->dtype);
   if (!comm->planner) {
     st = upload(S, comm->R);
     if (st != PL_OK) {
@@ -611,7 +615,7 @@ void host_pipeline_destroy(pl_comm_s* comm) {
 // Argument checks shared by the two host entry points.
 pl_status_t check_host_bufs(pl_schedule_s* s, const pl_bufs_t* host, const pl_bufs_t* dev) {
   if (!s || !host || !dev) return PL_ERR_INVALID_ARG;
-  if (s->comm->planner || !s->d_blob) return PL_ERR_UNSUPPORTED;
+  if (s->comm->planner) return PL_ERR_UNSUPPORTED;
   pl_status_t st = check_bufs(s, dev);
   if (st != PL_OK) return st;
   for (int r = 0; r < s->comm->R; ++r) {
@@ -1053,14 +1057,15 @@ pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index) {
     return PL_OK;
   }
   if (s->ring) {  // it reads no wait entries: from here on the op queues execute the schedule
-    uint64_t total = 0;
-    for (int r = 0; r < s->comm->R; ++r) {
-      s->scratch_off[r] = total;
-      total += align_up(s->L.scratch_per_rank[r], 256);
-    }
-    if (total && !s->d_scratch && cudaMalloc(&s->d_scratch, total) != cudaSuccess) { cudaGetLastError(); return PL_ERR_OOM; }
-    s->scratch_total = total;
     s->ring = false;
+    flatten(s, s->comm->dtype);
+    const pl_status_t st = upload(s, s->comm->R);
+    if (st != PL_OK) {
+      if (s->d_blob) cudaFree(s->d_blob);
+      s->d_blob = nullptr;
+      s->ring = true;
+      return st;
+    }
     fill_info(s, s->comm->R);
   }
   const size_t pos = (size_t)s->topo_to_dev[op_index];
@@ -1123,7 +1128,7 @@ static pl_status_t check_bufs(pl_schedule_t s, const pl_bufs_t* b) {
 
 pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
   if (!s || !bufs) return PL_ERR_INVALID_ARG;
-  if (s->comm->planner || !s->d_blob) return PL_ERR_UNSUPPORTED;
+  if (s->comm->planner) return PL_ERR_UNSUPPORTED;
   if (!on_comm_device(s->comm)) return PL_ERR_INVALID_ARG;
   pl_status_t st = check_bufs(s, bufs);
   if (st != PL_OK) return st;

@@ -53,3 +53,19 @@ def test_broken_wait_times_out():
     finally:
         B.pl_schedule_destroy(s)
         B.pl_comm_destroy(comm)
+
+
+def test_a_ring_in_clusters_uploads_no_op_list():
+    R, n = 16, 32 * 1024 * 1024  # 64 MiB of bf16 per rank in chunks of 64 KiB: 30,720 ops
+    comm = B.pl_comm_create(R, DT["bf16"])
+    scheds = [build(B.PL_ALLREDUCE, n)(comm, None)]
+    try:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        scheds += [build(B.PL_ALLREDUCE, n)(comm, None) for _ in range(6)]
+        assert len(B.pl_schedule_dump(scheds[0])) >= 30720 and B.pl_schedule_info(scheds[0]).scratch_bytes == 0
+        assert free - torch.cuda.mem_get_info()[0] < 4 << 20  # an op list takes 3 MiB
+    finally:
+        for s in scheds:
+            B.pl_schedule_destroy(s)
+        B.pl_comm_destroy(comm)
