@@ -161,8 +161,8 @@ bool ring_shape(int R, int dtype, bool reduce, bool gather, uint64_t part_units,
 struct LayerParams {
   uint64_t in_stride, out_stride;
   uint32_t n_layers;
-  uint32_t ask_ahead;                 // ask the next layer's lines into L2
   int32_t break_layer, break_queue;  // test hook of the cluster variant (no wait entries to break), -1 = none
+  uint32_t ask_ahead;                 // flags variant: ask the next layer's lines into L2
 };
 
 // Parameters of the packet executor (layered one-shot all-reduce, see pl_datapath_packet.cu).
