@@ -535,7 +535,7 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
     if (plan && !queues) {
       uint64_t units = 0, blocks = 0;
       for (const FlatSpan& f : S->flat_spans) units += f.units;
-      S->flat_launch = flat_launch(comm->R, reduce, all, pol.datapath == PL_DP_TMA, hook, units);
+      S->flat_launch = flat_launch(comm->R, reduce, all, pol.datapath == PL_DP_TMA, hook, units, comm->sm_count);
       for (FlatSpan& f : S->flat_spans) {
         f.first_block = (uint32_t)blocks;
         blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;

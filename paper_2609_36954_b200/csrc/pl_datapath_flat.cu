@@ -347,7 +347,7 @@ cudaError_t launch_dt(const FlatParams& P, const FlatLaunch& F, cudaStream_t str
 
 }  // namespace
 
-FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units) {
+FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units, int sm_count) {
   FlatLaunch F;
   F.reduce = reduce;
   F.all = all;
@@ -369,7 +369,7 @@ FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, u
   } else {
     // one unit per thread where it goes to every rank (all-gather of 4 MiB: 6.4 us, 4 units 12.9 us)
     // or where 4 units would leave SMs without two CTAs
-    F.units = (!all && total_units >= 4ull * kFlatThreads * 2 * 148) ? 4 : 1;
+    F.units = (!all && total_units >= 4ull * kFlatThreads * 2 * (uint64_t)sm_count) ? 4 : 1;
     F.tile = (uint32_t)(F.units * kFlatThreads);
   }
   return F;

@@ -206,16 +206,11 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
 }
 
 template <int DT, int NR, bool HOOK, bool CLUSTER>
-cudaError_t prepare_t(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int grid, int threads, bool overlap) {
+void configure(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int grid, int threads, bool overlap) {
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)(threads + (CLUSTER ? 32 : 0)));
   int na = 0;
   if (CLUSTER) {
-    // up to 16 CTAs: more than the portable 8 needs the opt-in (a per-device attribute of the function)
-    if (grid > 8) {
-      const cudaError_t e = cudaFuncSetAttribute(pl_layers_kernel<DT, NR, HOOK, CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-    }
     attr[na].id = cudaLaunchAttributeClusterDimension;
     attr[na].val.clusterDim.x = (unsigned)grid;
     attr[na].val.clusterDim.y = 1;
@@ -229,15 +224,13 @@ cudaError_t prepare_t(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int gr
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaSuccess;
 }
 
 template <int DT, int NR, bool HOOK, bool CLUSTER>
 cudaError_t launch_t(const ExecParams& P, const LayerParams& Y, int grid, int threads, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
-  const cudaError_t e = prepare_t<DT, NR, HOOK, CLUSTER>(cfg, attr, grid, threads, P.overlap_launch);
-  if (e != cudaSuccess) return e;
+  configure<DT, NR, HOOK, CLUSTER>(cfg, attr, grid, threads, P.overlap_launch);
   cfg.stream = stream;
   return cudaLaunchKernelEx(&cfg, pl_layers_kernel<DT, NR, HOOK, CLUSTER>, P, Y);
 }
@@ -247,7 +240,10 @@ bool cluster_fits_t(int grid, int threads) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   int n = 0;
-  if (prepare_t<DT, NR, HOOK, true>(cfg, attr, grid, threads, false) != cudaSuccess ||
+  configure<DT, NR, HOOK, true>(cfg, attr, grid, threads, false);
+  // up to 16 CTAs: more than the portable 8 needs the opt-in (a per-device attribute of the function, raised here, when
+  // the schedule is built, and kept)
+  if ((grid > 8 && cudaFuncSetAttribute(pl_layers_kernel<DT, NR, HOOK, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
       cudaOccupancyMaxActiveClusters(&n, pl_layers_kernel<DT, NR, HOOK, true>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;

@@ -218,7 +218,9 @@ auto pick(int dtype, int units, F f) {
     case PL_BF16: return by_units(std::integral_constant<int, PL_BF16>{});
     case PL_F32: return by_units(std::integral_constant<int, PL_F32>{});
     case PL_I32: return by_units(std::integral_constant<int, PL_I32>{});
-    default: return by_units(std::integral_constant<int, PL_U8>{});
+    // bytes are only gathered, in tiles of one unit per thread (ring_shape() gives four to two ranks and 256 threads,
+    // which an all-gather of two ranks is too small for)
+    default: return f(std::integral_constant<int, PL_U8>{}, std::integral_constant<int, 1>{});
   }
 }
 

@@ -22,10 +22,11 @@ size_t exec_tma_smem_bytes(int stages, uint32_t stage_bytes);
 // layered direct-fused all-reduces with one op per queue and layer (`cluster`: the grid is one
 // thread-block cluster and the cluster barrier takes the place of the flags)
 cudaError_t launch_layers(int dtype, const ExecParams& P, const LayerParams& Y, int grid, int threads, bool cluster, cudaStream_t stream);
+// whether such a cluster can be resident; raises the limit its launches need, so it goes before the first of them
 bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads);
 
 // schedules without flags, one CTA per tile
-FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units);
+FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units, int sm_count);
 cudaError_t launch_flat(int dtype, const FlatParams& P, const FlatLaunch& F, cudaStream_t stream);
 
 // ring schedules, a cluster per tile.  ring_prepare: clusters that can be resident at once (0: none)

@@ -141,3 +141,10 @@ def test_validating_a_layered_schedule_costs_little():
         assert build(0) < 4 * build(B.PL_OPT_SKIP_VALIDATE)
     finally:
         B.pl_comm_destroy(comm)
+
+
+@pytest.mark.parametrize("R", [2, 3, 4, 8, 16])
+def test_gathering_rings_have_one_unit_per_thread(rules, R):
+    for units in (1, 127, 4095, 32768, 65536):
+        _, smem, (threads, per_thread, tile, _) = ring(rules, R, "u8", "ag", 16 * units)
+        assert smem == 0 or (per_thread == 1 and tile == threads)
