@@ -33,11 +33,18 @@
  *     nothing and never synchronises.  A schedule may be executed any number of times
  *     (flags carry a device-resident epoch; nothing is reset between executes).
  *   - One stream at a time per schedule: two executes of the same schedule must not
- *     overlap on the GPU.  Executes of DIFFERENT schedules may overlap only if their grids
- *     together are co-resident (pl_schedule_info reports each grid): the CTAs of a launch
- *     wait on one another, so two launches that each hold part of the SMs could starve each
- *     other until the wait limit reports PL_ERR_TIMEOUT.  Issuing all executes on one stream
+ *     overlap on the GPU.  Executes of DIFFERENT schedules may overlap if the CTAs of at most
+ *     one of them wait on one another, or if the grids of all that do are co-resident together
+ *     (pl_schedule_info reports each grid): launches that each hold part of the SMs could
+ *     otherwise starve each other until the wait limit reports PL_ERR_TIMEOUT.  CTAs wait on one
+ *     another in schedules with flags (n_flags > 0) that run on queues or layer by layer.
+ *     Schedules without flags do not, nor do rings and layers that run in thread-block clusters
+ *     (waits inside a cluster only, whose CTAs are resident together): their grids may be larger
+ *     than the GPU and count nothing here.  A MoE dispatch of more than 1024 routing entries per
+ *     source waits too (one CTA per source and 256 tokens).  Issuing all executes on one stream
  *     is always safe.
+ *   - A launch may be set up while the one in front of it on the stream drains; it reads and
+ *     writes nothing before everything in front has completed (but for PL_OPT_STAGE_AHEAD).
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).
  *   - A communicator belongs to the CUDA device that was current when it was created; its
  *     schedules and plans live there.  Every later call on it must be made with that device
