@@ -457,3 +457,52 @@ def test_dispatch_behind_a_combine_does_not_wait_for_it_in_one_place():
         assert together <= 1.4 * apart, (together, apart)
     finally:
         run.close()
+
+
+# The deduplicated dispatch on both sides of its lines (1024 entries per source, 2048 tokens in all): more than 8 ranks,
+# several tokens per CTA, more slots than ranks, experts per rank that are no power of two, empty slots, tokens without
+# any, receive buffers that are too small.
+@pytest.mark.parametrize("R,T,H,E,K", [
+    (8, 128, 64, 32, 8), (8, 129, 64, 32, 8), (8, 256, 64, 32, 2), (8, 257, 64, 32, 2), (2, 1024, 8, 4, 1), (4, 3, 1032, 1024, 4), (4, 9, 1032, 2048, 4),
+    (16, 40, 7168, 48, 3), (3, 600, 2048, 9, 1), (5, 33, 2056, 15, 6), (2, 20, 4096, 64, 32), (16, 64, 512, 256, 8)])
+@pytest.mark.parametrize("short", [False, True])
+def test_dedup_around_the_lines(R, T, H, E, K, short):
+    idx, _ = gen.moe_routing(R, T, E, K, seed=6)
+    idx = [a.copy() for a in idx]
+    for a in idx:
+        a[::7, K - 1] = -1
+        a[5::11] = -1
+    epr = E // R
+    rows = [[(p, t) for p in range(R) for t in range(T) if ((idx[p][t] >= 0) & (idx[p][t] // epr == r)).any()] for r in range(R)]
+    most = max(map(len, rows))
+    cap = most - (1 if short and most > 1 else 0)
+    run = MoeRun(R, T, H, E, K, cap)
+    try:
+        x = gen.moe_tokens_bf16(R, T, H)
+        ptr = lambda ts: [t.data_ptr() for t in ts]
+        d_x, d_i = [to_dev(a) for a in x], [to_dev(a) for a in idx]
+        recv, meta, out = [poison(cap * H * 2) for _ in range(R)], [poison(cap * 16) for _ in range(R)], [poison(T * H * 2) for _ in range(R)]
+        for _ in range(2):
+            B.pl_moe_dispatch_dedup(run.plan, ptr(d_x), ptr(d_i), ptr(recv), ptr(meta), stream_handle())
+        B.pl_moe_combine_dedup(run.plan, ptr(recv), ptr(out), stream_handle())
+        pos, cnt = np.zeros((R, T, R), np.int32), np.zeros((R, R), np.int64)
+        status = B.pl_moe_plan_read_dedup(run.plan, pos.ctypes.data, cnt.ctypes.data, stream_handle())
+        assert status == (B.PL_ERR_OVERFLOW if cap < most else B.PL_OK)
+        want_pos = np.full((R, T, R), -1, np.int32)
+        for r in range(R):
+            got_rows, got_meta = recv[r].cpu().numpy().view(np.uint16).reshape(cap, H), meta[r].cpu().numpy().view(np.int32).reshape(cap, 4)
+            assert np.array_equal(cnt[:, r], np.bincount([p for p, _ in rows[r]], minlength=R))
+            for i, (p, t) in enumerate(rows[r][:cap]):
+                want_pos[p, t, r] = i
+                mask = sum(1 << j for j in range(K) if idx[p][t, j] >= 0 and idx[p][t, j] // epr == r)
+                assert tuple(got_meta[i]) == (p, t, np.uint32(mask).view(np.int32), r)
+                assert np.array_equal(got_rows[i], x[p][t])
+            assert (got_rows[len(rows[r]):] == 0xFFFF).all()
+        assert np.array_equal(pos, want_pos)
+        for p in range(R):
+            times = (want_pos[p] >= 0).sum(1)[:, None]  # every returned row is the token itself: an exact sum, one rounding to bf16
+            want = gen.bf16_bits_to_f64(x[p].reshape(-1)).reshape(T, H) * times
+            got = gen.bf16_bits_to_f64(out[p].cpu().numpy().view(np.uint16).reshape(-1)).reshape(T, H)
+            assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want))
+    finally:
+        run.close()
