@@ -148,3 +148,80 @@ def test_gathering_rings_have_one_unit_per_thread(rules, R):
     for units in (1, 127, 4095, 32768, 65536):
         _, smem, (threads, per_thread, tile, _) = ring(rules, R, "u8", "ag", 16 * units)
         assert smem == 0 or (per_thread == 1 and tile == threads)
+
+
+def landing(R, ops_or_spans, out_units):
+    """Where every 16-byte unit of every output comes from: (source rank or 255 for the sum of all, source unit); every unit once."""
+    out = [np.full((n, 2), -1, np.int64) for n in out_units]
+    for src_off, dst_off, units, src, dst in ops_or_spans:
+        for r in (range(R) if dst == 255 else (dst,)):
+            at = out[r][dst_off:dst_off + units]
+            assert at.shape[0] == units and (at == -1).all()
+            at[:, 0] = src
+            at[:, 1] = np.arange(src_off, src_off + units)
+    assert all((o >= 0).all() for o in out)
+    return out
+
+
+# collectives without flags, over types, odd sizes, empty parts and a processing phase: the spans say of every unit of
+# every output what the op list says
+@pytest.mark.parametrize("R", [2, 3, 5, 8, 16])
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "i32", "u8"])
+@pytest.mark.parametrize("units", [1, 7, 129, 1025])
+def test_spans_say_what_the_ops_say(rules, R, dtype, units):
+    dt, es = {"bf16": (B.PL_BF16, 2), "f32": (B.PL_F32, 4), "i32": (B.PL_I32, 4), "u8": (B.PL_U8, 1)}[dtype]
+    vec = 16 // es
+    part = units * vec
+    v1 = [vec * ((3 * p + units) % 11) for p in range(R)]
+    v2 = [[vec * ((5 * p + 7 * r + units) % 13) for r in range(R)] for p in range(R)]
+    requests = [(B.PL_ALLGATHER, B.PL_ALGO_DIRECT, part, None, 0), (B.PL_ALLTOALL, B.PL_ALGO_DIRECT, part * R, None, 0),
+                (B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, 0, v2, 0), (B.PL_ALLGATHERV, B.PL_ALGO_DIRECT, 0, v1, 0),
+                (B.PL_SCATTER, B.PL_ALGO_DIRECT, part, None, 0), (B.PL_GATHER, B.PL_ALGO_DIRECT, part, None, 0)]
+    if dtype != "u8":
+        requests += [(B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, part * R, None, 0), (B.PL_ALLREDUCE, B.PL_ALGO_ONESHOT, part, None, 0),
+                     (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, part * R, None, 0), (B.PL_REDUCE_SCATTERV, B.PL_ALGO_DIRECT, 0, v1, 0)]
+    if dtype == "bf16":
+        requests += [(B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, part * R, None, B.PL_HOOK_F32_OUT | B.PL_HOOK_RESIDUAL),
+                     (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, part * R, None, B.PL_HOOK_F32_OUT)]
+    for coll, algo, count, counts, hook in requests:
+        comm = B.pl_comm_create_planner(R, dt)
+        opts = B.make_opts(hook=hook) if hook else None
+        try:
+            if counts is not None:
+                if sum(np.ravel(counts)) == 0:
+                    continue
+                s = B.pl_schedule_build_v(comm, coll, algo, counts, 256, opts)
+            elif coll in (B.PL_SCATTER, B.PL_GATHER):
+                s = B.pl_schedule_build_rooted(comm, coll, R - 1, count, 256, opts)
+            else:
+                s = B.pl_schedule_build(comm, coll, algo, count, 256, opts)
+            info = B.pl_schedule_info(s)
+            assert info.n_flags == 0
+            out_b = 32 if hook & B.PL_HOOK_F32_OUT else 16  # bytes of an output unit
+            out_units = [int(info.out_bytes[r]) // out_b for r in range(R)]
+            ops = []
+            for o in B.pl_schedule_dump(s):
+                copy = o.kind == B.PL_OP_COPY
+                if not copy:
+                    assert o.n_src == R and all(o.src[k].rank == k and o.src[k].offset == o.src[0].offset for k in range(R))
+                nbytes = o.count * (1 if copy else es)
+                if nbytes:
+                    ops.append((o.src[0].offset // 16, o.dst.offset // out_b, nbytes // 16, o.src[0].rank if copy else 255, 255 if o.dst_bcast & 1 else o.dst.rank))
+            flat = np.ravel(counts).astype(np.uint64) if counts is not None else None
+            buf, red, every = np.zeros((4096, 5), np.uint64), C.c_int(), C.c_int()
+            n = rules.t_flat_plan(R, dt, coll, algo, count, 256, flat.ctypes.data if flat is not None else None, R - 1, hook, buf.ctypes.data, 4096,
+                                  C.addressof(red), C.addressof(every))
+            assert 0 < n <= 4096 and n <= len(ops)
+            spans = [tuple(int(x) for x in row) for row in buf[:n]]
+            assert {s_[4] == 255 for s_ in spans} == {bool(every.value)} and {s_[3] == 255 for s_ in spans} == {bool(red.value)}
+            for a, b in zip(landing(R, ops, out_units), landing(R, spans, out_units)):
+                assert np.array_equal(a, b)
+            B.pl_schedule_destroy(s)
+        finally:
+            B.pl_comm_destroy(comm)
+
+
+def test_ops_with_flags_or_scratch_are_not_laid_out(rules):
+    buf, red, every = np.zeros((64, 5), np.uint64), C.c_int(), C.c_int()
+    for coll, algo in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT), (B.PL_ALLREDUCE, B.PL_ALGO_TREE), (B.PL_REDUCE_SCATTER, B.PL_ALGO_RING), (B.PL_ALLREDUCE, B.PL_ALGO_RING)):
+        assert rules.t_flat_plan(4, B.PL_F32, coll, algo, 4096, 1024, None, 0, 0, buf.ctypes.data, 64, C.addressof(red), C.addressof(every)) == -1

@@ -17,12 +17,23 @@ def values(nbytes, dtype, gen):
     return torch.randint(0, 256, (nbytes,), generator=gen, device="cuda", dtype=torch.uint8)
 
 
-def same_bits(R, dtype, build, **both):
-    """`build` makes a schedule from (comm, opts); runs it flat and on the queues, compares all outputs."""
+def executor(info):
+    """What runs a schedule that is not asked for a datapath: "tiles" (one CTA, or one cluster of a ring, per tile) or "queues"."""
+    if info.stages == 1:
+        assert info.stage_bytes > 0 and info.slice_bytes == 0
+        return "tiles"
+    assert info.grid == info.n_queues
+    return "queues"
+
+
+def same_bits(R, dtype, build, want, **both):
+    """`build` makes a schedule from (comm, opts); runs it as the library picks (`want` says on what) and on the register
+    queues, compares all outputs."""
     comm = B.pl_comm_create(R, DT[dtype])
     flat, queues = build(comm, B.make_opts(**both)), build(comm, B.make_opts(datapath=B.PL_DP_LDST, **both))
     try:
         info = B.pl_schedule_info(flat)
+        assert executor(info) == want and executor(B.pl_schedule_info(queues)) == "queues"
         gen = torch.Generator(device="cuda").manual_seed(3)
         sizes = [[int(a[r]) for r in range(R)] for a in (info.in_bytes, info.out_bytes, info.aux_bytes)]
         ins = [values(max(16, n), dtype, gen) for n in sizes[0]]
@@ -56,8 +67,10 @@ def test_fixed_size_collectives(R, dtype, units):
     for coll, algo, count in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n * R), (B.PL_ALLREDUCE, B.PL_ALGO_ONESHOT, n),
                               (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, n * R), (B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n),
                               (B.PL_ALLTOALL, B.PL_ALGO_DIRECT, n * R)):
+        # one-shot: 72 MiB of inputs on 2 ranks, 9 MiB on 16 are the queues'
+        want = "queues" if algo == B.PL_ALGO_ONESHOT and units == "stream" and R in (2, 16) else "tiles"
         for flags in (0, B.PL_OPT_INPUTS_LAST_USE):
-            info = same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, count, 64 * 1024, o), flags=flags)
+            info = same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, count, 64 * 1024, o), want, flags=flags)
         if units == "stream" and algo == B.PL_ALGO_DIRECT_FUSED:
             assert info.datapath == B.PL_DP_TMA
 
@@ -70,21 +83,42 @@ def test_processing_phase(R, dtype, units):
     hooks = [B.PL_HOOK_RESIDUAL] + ([B.PL_HOOK_F32_OUT, B.PL_HOOK_RESIDUAL | B.PL_HOOK_F32_OUT] if dtype == "bf16" else [])
     for hook in hooks:
         for coll, algo in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED), (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT)):
-            same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, n, 64 * 1024, o), hook=hook, out_scale=0.375)
+            # fused with fp32 output: the queues' up to 8 MiB of inputs, and where it streams without a residual
+            f32_fused = algo == B.PL_ALGO_DIRECT_FUSED and hook & B.PL_HOOK_F32_OUT
+            want = "queues" if f32_fused and (units != "stream" or hook == B.PL_HOOK_F32_OUT) else "tiles"
+            same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, n, 64 * 1024, o), want, hook=hook, out_scale=0.375)
+
+
+# units of a partition: 4 x 4 MiB and a ragged end, 16 ranks on both sides of 8 MiB of inputs
+@pytest.mark.parametrize("R,units,want", [(4, 65536 + 37, "tiles"), (8, 8192 + 129, "tiles"), (16, 2049, "tiles"), (16, 2048, "queues")])
+@pytest.mark.parametrize("hook", [B.PL_HOOK_F32_OUT, B.PL_HOOK_RESIDUAL | B.PL_HOOK_F32_OUT])
+def test_fused_with_f32_output_between_its_lines(R, units, want, hook):
+    same_bits(R, "bf16", lambda c, o: B.pl_schedule_build(c, B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, 8 * units * R, 64 * 1024, o), want, hook=hook, out_scale=0.375)
+
+
+# MiB of a message above L2 with one-shot, KiB gathered by many ranks
+@pytest.mark.parametrize("R,coll,nbytes,want", [
+    (8, "oneshot", 16 * MIB, "queues"), (8, "oneshot", 8 * MIB, "tiles"), (16, "gather", MIB, "queues"), (16, "gather", MIB // 2, "tiles"), (12, "gather", 3 * 330 * 1024, "queues")])
+def test_sizes_that_stay_on_the_queues(R, coll, nbytes, want):
+    n = nbytes // 2
+    if coll == "oneshot":
+        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build(c, B.PL_ALLREDUCE, B.PL_ALGO_ONESHOT, n, MIB, o), want)
+    else:
+        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build(c, B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n // R // 8 * 8, MIB, o), want)
 
 
 @pytest.mark.parametrize("scale", [1, 3000])
 def test_variable_sizes_and_rooted(scale):
     R = 8
     counts = [[0 if (p + r) % 3 == 0 else 8 * (1 + (5 * p + 11 * r) % 67) * scale for r in range(R)] for p in range(R)]
-    same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, counts, 4096, o))
+    same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, counts, 4096, o), "tiles")
     for coll in (B.PL_ALLGATHERV, B.PL_REDUCE_SCATTERV):
-        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_v(c, coll, B.PL_ALGO_DIRECT, counts[2], 4096, o))
+        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_v(c, coll, B.PL_ALGO_DIRECT, counts[2], 4096, o), "tiles")
     for coll in (B.PL_BROADCAST, B.PL_REDUCE, B.PL_SCATTER, B.PL_GATHER):
-        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_rooted(c, coll, 5, 8 * R * 77 * scale, 4096, o))
+        same_bits(R, "bf16", lambda c, o: B.pl_schedule_build_rooted(c, coll, 5, 8 * R * 77 * scale, 4096, o), "tiles")
     # 256 spans, those between different ranks a single vector
     one = [[8 if p != r else 8 * 50 * scale for r in range(16)] for p in range(16)]
-    same_bits(16, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, one, 4096, o))
+    same_bits(16, "bf16", lambda c, o: B.pl_schedule_build_v(c, B.PL_ALLTOALLV, B.PL_ALGO_DIRECT, one, 4096, o), "tiles")
 
 
 def test_results_that_fit_l2_stay_there():
