@@ -281,9 +281,9 @@ def run_purlin(args):
         d2h = (copied1[1] - copied0[1]) // Ke
         e2e = {"value": replicas.aggregate_throughput(eff_bytes, e_ms / Ke, world) / 1e9, "unit": "GB/s", "steps": Ke,
                "ms_per_step": e_ms / Ke, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
-               "api": "pl_execute_host_async (pinned host buffers in and out; uploads, schedule and downloads of "
-                      "consecutive calls on three streams; an input that the previous call's download is still "
-                      "writing from the same device buffer is not uploaded again)"}
+               "api": "pl_execute_host_async, pinned host buffers in and out"}
+        # uploads, schedule and downloads of consecutive calls on three streams; an input that the previous
+        # call's download is still writing from the same device buffer is not uploaded again
         # parity spot check of the e2e result on sampled elements against the definition
         got = h_out[3].numpy().view(np.uint16)
         idx = np.linspace(0, n - 1, 64).astype(np.int64)
@@ -362,19 +362,39 @@ def run_purlin(args):
             "clocks": clocks, "e2e": e2e, "gpu_launches": int(launches), "roofline": roofline,
             "cpu_baseline": cpu, "small_allreduce": latency, "detail": detail,
         }
-        print(json.dumps(line))
+        emit(line, args.detail_out)
     B.pl_schedule_destroy(rs)
     B.pl_schedule_destroy(ag)
     B.pl_comm_destroy(comm)
     replicas.finalize()
 
 
+def short_line(line):
+    """The one line that is printed: everything but the detail, numbers to six digits, well under 3 KB (whoever reads the
+    end of a long output must find the whole line in it)."""
+    def digits(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: digits(w) for k, w in v.items()}
+        return [digits(w) for w in v] if isinstance(v, list) else v
+    out = {k: v for k, v in line.items() if k != "detail"}
+    if out.get("small_allreduce"):
+        out["small_allreduce"] = {k: v for k, v in out["small_allreduce"].items() if k != "all"}
+    return json.dumps(digits(out))
+
+
+def emit(line, detail_out):
+    if detail_out:
+        with open(detail_out, "w") as f:
+            f.write(json.dumps(line) + "\n")
+    print(short_line(line))
+
+
 def measure_step_variant(B, torch, comm, n, chunk, R, b_rs, b_ag, stream, plain_ms, flags):
     """The C2 step built with other schedule options and timed without events between the two
-    launches.  PL_OPT_OVERLAP_LAUNCH (the CTAs of a launch are set up while the one in front of it
-    drains) is made for the latency path; on these HBM-bound launches it does not pay (the CTAs of
-    a launch then take the SMs in the order in which they become free).  flags = 0 is the step
-    without PL_OPT_INPUTS_LAST_USE."""
+    launches: PL_OPT_OVERLAP_LAUNCH on both (no difference while they run without queues, which are
+    always launched overlapped), and flags = 0, the step without PL_OPT_INPUTS_LAST_USE."""
     opts = B.make_opts(flags=flags)
     rs = B.pl_schedule_build(comm, B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, n, chunk, opts)
     ag = B.pl_schedule_build(comm, B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n // R, chunk, opts)
@@ -682,6 +702,8 @@ def main():
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--no-latency", action="store_true")
     ap.add_argument("--no-detail", action="store_true", help="skip the other configurations (C1, C3, C4, C5, stream ceilings)")
+    ap.add_argument("--detail-out", default=os.path.join(ROOT, "bench_detail.json"),
+                    help="file that receives the line with every configuration in its detail section (read by bench_table.py); empty for none")
     ap.add_argument("--ag-grid", type=int, default=0, help="grid of the all-gather schedule (skips pl_comm_tune); for profiling runs")
     ap.add_argument("--ag-idle", default="", help="with --ag-grid: window of idle SMs of the all-gather launch as first:count")
     ap.add_argument("--no-tune", action="store_true", help="skip pl_comm_tune (the all-gather then runs with the untuned default grid)")

@@ -1,10 +1,10 @@
 #!/usr/bin/env python
-"""Turns the JSON line printed by ``bench.py`` into the markdown tables of the design notes.
+"""Turns the record that ``bench.py`` writes beside its line into the markdown tables of the design notes.
 
-  python bench.py > line.json
-  python bench_table.py line.json
+  python bench.py
+  python bench_table.py bench_detail.json
 
-Nothing is measured here: every number is read from the line (its ``detail`` section holds one
+Nothing is measured here: every number is read from the record (its ``detail`` section holds one
 entry per configuration, each with its algorithmic bytes and fractions).
 """
 from __future__ import annotations

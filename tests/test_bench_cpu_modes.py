@@ -31,3 +31,20 @@ def test_reference_arm_prints_the_contract_line():
     assert r["cpu_baseline"]["kind"] == "oracle" and r["cpu_baseline"]["cores"] >= 1 and r["cpu_baseline"]["value"] == r["value"]
     assert r["e2e"] == {"value": r["value"], "unit": "GB/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}
     assert "workload" in r["config"]
+
+
+def test_the_printed_line_is_short(tmp_path, capsys):
+    """Whoever keeps the last 3 KB of the output must find the whole line in them; every configuration goes to a file."""
+    sys.path.insert(0, ROOT)
+    import bench
+    text = "x" * 60
+    entry = {f"number_{i}": 1234.56789012345 + i for i in range(12)}
+    line = {"metric": "effective collective GB/s", "value": 714.123456789012, "unit": "GB/s", "config": {k: text * 3 for k in "abcd"},
+            "clocks": {"sm_mhz": 1965, "reasons": []}, "e2e": dict(entry, api=text), "roofline": dict(entry, kernel=text), "cpu_baseline": dict(list(entry.items())[:3], sample=text),
+            "small_allreduce": {"metric": text, "p50_us": 1.23456789, "all": {"oneshot": entry, "fused": entry}}, "detail": {str(i): entry for i in range(100)}}
+    bench.emit(line, str(tmp_path / "detail.json"))
+    out = capsys.readouterr().out
+    assert out.count("\n") == 1 and len(out) < 2800
+    short, full = json.loads(out), json.loads((tmp_path / "detail.json").read_text())
+    assert full == line and "detail" not in short and "all" not in short["small_allreduce"]
+    assert set(line) - set(short) == {"detail"} and abs(short["value"] / line["value"] - 1) < 1e-5
