@@ -9,7 +9,7 @@
 // over at the end.  Queues of a persistent grid drift apart (equal work, unequal service) and touch
 // 144 windows at once.  B200, R = 8, bf16, back to back over three sets of buffers, queue executor
 // -> this: reduce-scatter + all-gather 64 MiB per rank 189 -> 175 us, fused all-reduce 256 MiB
-// 667 -> 632 us, 16 MiB 50.9 -> 42.1 us, 4 MiB 15.6 -> 11.9 us, 16 MiB with residual 82.6 -> 60.6 us,
+// 657 -> 631 us, 16 MiB 50.9 -> 42.1 us, 4 MiB 15.6 -> 11.9 us, 16 MiB with residual 82.6 -> 60.6 us,
 // 4 MiB with residual 34.8 -> 18.0 us, all-to-all-v of 24 MiB 67.5 -> 61.0 us.
 //
 // Two forms, by the schedule's datapath:

@@ -20,8 +20,8 @@
 // flag 0.3-0.6 us, inputs from L2 0.4 us), at 1 MiB the chain plus 16 MiB of L2 traffic per layer
 // (2.6 us at DRAM rate, which the prefetch and the write-back overlap with the chain).
 // Measured on B200, R = 8, bf16, 80 layers in one launch, three sets of buffers in turn, us per
-// layer, register executor -> this kernel: 8 KiB 2.10 -> 1.32, 16 KiB 2.40 -> 1.32-1.51 (cluster);
-// 64 KiB 3.20 -> 1.96, 128 KiB 3.28 -> 2.00, 512 KiB 3.86 -> 2.63, 1 MiB 4.99 -> 3.64 (flags).
+// layer, register executor -> this kernel: 4 KiB 2.0 -> 1.17, 16 KiB 2.16 -> 1.22 (cluster); 64 KiB 3.20 -> 1.95,
+// 128 KiB 3.28 -> 2.00, 512 KiB 3.86 -> 2.63, 1 MiB 5.00 -> 3.64 (flags).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

@@ -793,7 +793,7 @@ void a2a_direct_staged(Emitter& em, const Geo& g, uint64_t capacity) {
 }  // namespace
 
 // One cluster while it has at most 256 KiB of inputs to read per layer (16 KiB per CTA): at
-// R = 8 a 16 KiB layer takes 1.32-1.45 us as a cluster and 1.66 us with flags, 32 KiB 1.59-2.03
+// R = 8 a 16 KiB layer takes 1.22 us as a cluster and 1.66 us with flags, 32 KiB 1.59-2.03
 // (the two values are two B200s) against 1.95, 64 KiB 2.16-2.24 against 1.96.  With flags as many
 // CTAs as there are slices of at least 32 units: 16, 32, 64 or 128 made no difference at 64 KiB
 // and above as long as every SM has a slice at the large end (1 MiB: 128 CTAs 3.6 us, 64 CTAs 5 us).
