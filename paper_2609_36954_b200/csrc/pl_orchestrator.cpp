@@ -1321,13 +1321,15 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
 // A one-shot all-reduce reads every input once per rank.  Flat, the tiles go out destination by
 // destination, so every sweep passes over all inputs; the op list has the destinations of a chunk next
 // to one another, which lets all reads but the first hit L2 when the inputs do not fit it.  us, queues /
-// flat, by MiB of all inputs: bf16 8 x 8 MiB (64) 68 / 51, 12 x 6 (72) 92 / 113, 16 x 5 (80) 142 / 158, 8 x 12 (96)
-// 100 / 124, 8 x 16 124 / 170, 8 x 256 1866 / 2664, 4 x 64 145 / 188, 2 x 256 191 / 231; int32, whose adds are
-// cheaper, 16 x 5 (80) 137 / 111, 13 x 7 (91) 141 / 161.  With a processing phase the register queues take
-// twice as long, and the line is where the queues use bulk copies (8 x 12 MiB residual 175 / 141, 8 x 16 MiB
-// 156 / 189).  Float sums of 12 and 16 ranks leave half of flat's registers idle while 144 queues
-// divide evenly among them: 12 x 768 KiB bf16 10 / 14, 12 x 3 MiB 47 / 52, 16 x 512 KiB 12.3 / 14.1, while 13 ranks
-// take 16.4 / 15.1 and 73 / 58.
+// flat, ranks x MiB: bf16 8 x 8 68 / 51, 12 x 6 92 / 113, 16 x 5 142 / 158, 8 x 12 100 / 124, 4 x 24 63 / 72, 6 x 16 93 / 99, 8 x 16
+// 124 / 170, 8 x 256 1866 / 2664, 2 x 256 191 / 231, but 6 x 12 64 / 56 and 3 x 32 83 / 58; int32, whose adds are cheaper, 16 x
+// 5 137 / 111, 13 x 7 141 / 161.  The compensated adds of fp32 are what the bulk-copy queues' few warps wait for (8 x 16 200 /
+// 171, 16 x 64 3233 / 2536, 3 x 64 150 / 115), so it goes to the register queues only (10 x 12 184 / 247, 12 x 6 116 / 142).
+// With a processing phase the register queues of bf16 take twice as long; the bulk-copy queues are ahead where
+// their ranks divide the SMs evenly (residual 8 x 16 156 / 189, 12 x 64 1365 / 1565, 14 x 64 2191 / 2088, 3 x 64 170 / 142; fp32
+// output 8 x 64 663 / 743, 16 x 64 2773 / 2661; both 8 x 64 633 / 818, 14 x 64 2212 / 2199).  Float sums of 12 and 16 ranks leave half
+// of flat's registers idle while 144 queues divide evenly among them: 12 x 768 KiB bf16 10 / 14, 12 x 3 MiB 47 / 52, 16 x
+// 512 KiB 12.3 / 14.1, while 13 ranks take 16.4 / 15.1 and 73 / 58.
 // An all-gather of more than 8 ranks stores every unit more than 8 times; between 10 and 36 MiB written the
 // queues, which keep 144 CTAs at it, are ahead (us, queues / flat: 16 x 768 KiB 3.7 / 8.5, 1 MiB 4.3 / 9.4, 2 MiB 7.8 /
 // 11.1, 3 MiB 10.0 / 11.4, 4 MiB 13.2 / 14.0; 14 x 1 MiB 4.1 / 8.5; 12 x 1 MiB 3.7 / 7.1, 4 MiB 10.3 / 10.9); below both
@@ -1337,9 +1339,16 @@ bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool 
   if (!reduce) return all && !tma && R > 8 && inputs >= 10 * mib && inputs <= 36 * mib;  // a gathered message: bytes written
   if (all) return dtype == PL_BF16 && (hook & PL_HOOK_F32_OUT) && (inputs <= 8 * mib || (tma && !(hook & PL_HOOK_RESIDUAL)));
   if (algo != PL_ALGO_ONESHOT) return false;
-  if (hook) return tma;
-  if (tma || inputs >= (dtype == PL_I32 ? 88 : 72) * mib) return true;
-  if (dtype == PL_I32 || (R != 12 && R != 16)) return false;
+  if (dtype == PL_F32) {
+    if (tma) return false;
+    if (R >= (hook ? 10 : 8) && inputs >= 72 * mib) return true;
+  } else if (hook) {
+    const bool even = R >= 4 && 148 / R * R >= 144;
+    return tma && (hook == PL_HOOK_RESIDUAL ? even : hook == PL_HOOK_F32_OUT ? even && R < 16 : R >= 3);
+  } else if (tma || (R >= 4 && inputs >= (R < 8 ? 95 : dtype == PL_I32 ? 88 : 72) * mib)) {
+    return true;
+  }
+  if (hook || dtype == PL_I32 || (R != 12 && R != 16)) return false;
   return (inputs >= 6 * mib && inputs <= 10 * mib) || (R == 12 && inputs >= 18 * mib);
 }
 

@@ -36,13 +36,16 @@ def rules(tmp_path_factory):
 @pytest.mark.parametrize("R,mib,dtype,hook,queues", [
     (8, 256, "bf16", 0, 1), (8, 16, "bf16", 0, 1), (8, 12, "f32", 0, 1), (8, 8, "bf16", 0, 0), (8, 1, "bf16", 0, 0), (4, 64, "i32", 0, 1),
     (2, 16, "bf16", 0, 0), (16, 5, "bf16", 0, 1), (16, 5, "i32", 0, 0), (16, 6, "i32", 0, 1), (8, 16, "bf16", B.PL_HOOK_RESIDUAL, 1),
-    (8, 12, "bf16", B.PL_HOOK_RESIDUAL, 0), (12, 0.75, "bf16", 0, 1), (13, 0.75, "bf16", 0, 0), (16, 0.5, "f32", 0, 1), (16, 1, "bf16", 0, 0)])
+    (8, 12, "bf16", B.PL_HOOK_RESIDUAL, 0), (12, 0.75, "bf16", 0, 1), (13, 0.75, "bf16", 0, 0), (16, 0.5, "f32", 0, 1), (16, 1, "bf16", 0, 0),
+    (8, 16, "f32", 0, 0), (16, 64, "f32", 0, 0), (12, 6, "f32", 0, 1), (12, 12, "f32", 0, 0), (3, 32, "bf16", 0, 0), (6, 12, "bf16", 0, 0), (6, 16, "bf16", 0, 1),
+    (2, 64, "bf16", B.PL_HOOK_RESIDUAL, 0), (14, 16, "bf16", B.PL_HOOK_RESIDUAL, 0), (16, 16, "bf16", B.PL_HOOK_F32_OUT, 0), (8, 16, "bf16", B.PL_HOOK_F32_OUT, 1),
+    (16, 16, "bf16", B.PL_HOOK_F32_OUT | B.PL_HOOK_RESIDUAL, 1), (8, 16, "f32", B.PL_HOOK_RESIDUAL, 0), (10, 12, "f32", B.PL_HOOK_RESIDUAL, 1)])
 def test_one_shot_all_reduce_stays_on_the_queues_where_they_are_faster(rules, R, mib, dtype, hook, queues):
     dt = {"bf16": B.PL_BF16, "f32": B.PL_F32, "i32": B.PL_I32}[dtype]
     tma = 2 * R * mib * MIB >= 256 * MIB
     assert rules.t_queues_faster(R, dt, hook, B.PL_ALGO_ONESHOT, 1, 0, tma, int(mib * MIB)) == queues
     # the same sizes without a second reading of the inputs
-    assert rules.t_queues_faster(R, dt, hook, B.PL_ALGO_DIRECT_FUSED, 1, 1, tma, int(mib * MIB)) == 0
+    assert rules.t_queues_faster(R, dt, 0, B.PL_ALGO_DIRECT_FUSED, 1, 1, tma, int(mib * MIB)) == 0
 
 
 # KiB gathered, R: between 10 and 36 MiB written in all, more than 8 ranks gather on the queues

@@ -67,8 +67,8 @@ def test_fixed_size_collectives(R, dtype, units):
     for coll, algo, count in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n * R), (B.PL_ALLREDUCE, B.PL_ALGO_ONESHOT, n),
                               (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, n * R), (B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n),
                               (B.PL_ALLTOALL, B.PL_ALGO_DIRECT, n * R)):
-        # one-shot: 72 MiB of inputs on 2 ranks, 9 MiB on 16 are the queues'
-        want = "queues" if algo == B.PL_ALGO_ONESHOT and units == "stream" and R in (2, 16) else "tiles"
+        # one-shot: 9 MiB of inputs on 16 ranks are the queues'
+        want = "queues" if algo == B.PL_ALGO_ONESHOT and units == "stream" and R == 16 else "tiles"
         for flags in (0, B.PL_OPT_INPUTS_LAST_USE):
             info = same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, count, 64 * 1024, o), want, flags=flags)
         if units == "stream" and algo == B.PL_ALGO_DIRECT_FUSED:
@@ -98,7 +98,7 @@ def test_fused_with_f32_output_between_its_lines(R, units, want, hook):
 
 # MiB of a message above L2 with one-shot, KiB gathered by many ranks
 @pytest.mark.parametrize("R,coll,nbytes,want", [
-    (8, "oneshot", 16 * MIB, "queues"), (8, "oneshot", 8 * MIB, "tiles"), (16, "gather", MIB, "queues"), (16, "gather", MIB // 2, "tiles"), (12, "gather", 3 * 330 * 1024, "queues")])
+    (8, "oneshot", 16 * MIB, "queues"), (8, "oneshot", 8 * MIB, "tiles"), (3, "oneshot", 32 * MIB // 48 * 48, "tiles"), (16, "gather", MIB, "queues"), (16, "gather", MIB // 2, "tiles"), (12, "gather", 3 * 330 * 1024, "queues")])
 def test_sizes_that_stay_on_the_queues(R, coll, nbytes, want):
     n = nbytes // 2
     if coll == "oneshot":
