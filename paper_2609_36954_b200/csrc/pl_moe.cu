@@ -63,7 +63,10 @@ struct MoeGeo {
   const int32_t* slotmask;  // optional [R][T][K]: written into the metadata instead of the slot index
   int epr_shift;            // log2(epr), -1 if it is no power of two
   int gates_are_logits;     // combine: the gate input holds the K selected logits; softmax them first
+  uint32_t parts, width;    // combine by parts: CTAs per row, threads per token
+  uint64_t pad[4];
 };
+static_assert(cheap_params(sizeof(MoeGeo)) && sizeof(DispatchPtrs) % 64 == 0 && sizeof(CombinePtrs) % 64 == 0, "launch cost");
 
 __device__ __forceinline__ void build_mask(const MoeGeo& g, const int32_t* idx, uint32_t* mask, int t, int tid) {
   for (int i = tid; i < g.E * kMaskWords; i += kTB) mask[i] = 0u;
@@ -343,8 +346,16 @@ __global__ void __launch_bounds__(kTB) moe_plan_kernel(const __grid_constant__ D
 
 // Deduplicated routing: for every token the distinct destination ranks in ascending order
 // (padded with -1) and, per destination, the mask of slots whose expert lives there.
-__global__ void __launch_bounds__(256) moe_derive_ranks_kernel(const __grid_constant__ DispatchPtrs P, int R, int T, int K,
-                                                               int epr, int KR, int32_t* ridx, int32_t* rmask) {
+struct DeriveParams {
+  const int32_t* idx[PL_MAX_RANKS];
+  int R, T, K, epr, KR;  // KR: destinations per token
+  int32_t *ridx, *rmask;
+  uint64_t pad[7];
+};
+static_assert(cheap_params(sizeof(DeriveParams)), "launch cost");
+__global__ void __launch_bounds__(256) moe_derive_ranks_kernel(const __grid_constant__ DeriveParams P) {
+  const int R = P.R, T = P.T, K = P.K, epr = P.epr, KR = P.KR;
+  int32_t *const ridx = P.ridx, *const rmask = P.rmask;
   const long long tok = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -392,7 +403,9 @@ struct SmallParams {
   int K0, epr0;             // DEDUP: slots per token and experts per rank of the routing
   int32_t* ridx;            // DEDUP: distinct destination ranks per token, padded with -1, and the slots on each
   int32_t* rmask;
+  uint64_t pad[4];
 };
+static_assert(sizeof(SmallParams) % 64 == 0, "launch cost");  // it goes with a MoeGeo
 
 // Bounded wait for the first phase of `bar` (a CTA's rows have landed).
 __device__ __forceinline__ bool wait_rows(uint64_t* bar) {
@@ -803,8 +816,8 @@ __global__ void __launch_bounds__(kCombineThreads) moe_combine_kernel(const __gr
 // count is.  `width` threads (whole warps) work on one token.  KB source rows are loaded at a time:
 // with few slots per token the registers of eight would cost half of the resident CTAs.
 template <int KB>
-__global__ void __launch_bounds__(kCombinePartThreads) moe_combine_parts_kernel(const __grid_constant__ CombinePtrs P, const __grid_constant__ MoeGeo g,
-                                                                                uint32_t parts, uint32_t width) {
+__global__ void __launch_bounds__(kCombinePartThreads) moe_combine_parts_kernel(const __grid_constant__ CombinePtrs P, const __grid_constant__ MoeGeo g) {
+  const uint32_t parts = g.parts, width = g.width;
   constexpr int kTokens = kCombinePartThreads / 32;
   __shared__ const char* s_row[kTokens][kMaxTopk];
   __shared__ float s_gate[kTokens][kMaxTopk];
@@ -1107,14 +1120,16 @@ pl_status_t pl_moe_dispatch(pl_moe_plan_t plan, const void* const* x, const int3
 }
 
 // Launched overlapped like the register executor: both kernels wait for everything in front before they read.
-static bool launch_combine(pl_moe_plan_t plan, const CombinePtrs& P, const MoeGeo& g, cudaStream_t cs) {
+static bool launch_combine(pl_moe_plan_t plan, const CombinePtrs& P, MoeGeo g, cudaStream_t cs) {
   const uint32_t units = g.row_bytes >> 4, parts = (units + kCombinePartThreads - 1) / kCombinePartThreads;
   const unsigned long long n_tok = (unsigned long long)g.R * g.T, turns = (unsigned long long)plan->sm_count * plan->combine_per_sm;
   const bool by_parts = combine_by_parts(n_tok, units, g.K, turns) && n_tok * parts <= 0x7FFFFFFFull;
   const uint32_t width = ((units + parts - 1) / parts + 31) / 32 * 32, tokens = parts > 1 ? 1u : kCombinePartThreads / width;
   if (!by_parts) return launch_after(true, moe_combine_kernel, dim3((unsigned)std::min(n_tok, turns)), kCombineThreads, 0, cs, P, g);
+  g.parts = parts;
+  g.width = width;
   return launch_after(true, g.K <= 2 ? moe_combine_parts_kernel<2> : g.K <= 4 ? moe_combine_parts_kernel<4> : moe_combine_parts_kernel<8>,
-                      dim3((unsigned)((n_tok * parts + tokens - 1) / tokens)), tokens * width, 0, cs, P, g, parts, width);
+                      dim3((unsigned)((n_tok * parts + tokens - 1) / tokens)), tokens * width, 0, cs, P, g);
 }
 
 static pl_status_t combine_impl(pl_moe_plan_t plan, const void* const* y, const float* const* gates, void* const* out,
@@ -1175,14 +1190,14 @@ pl_status_t pl_moe_dispatch_dedup(pl_moe_plan_t plan, const void* const* x, cons
   if (!on_comm_device(plan->comm)) return PL_ERR_INVALID_ARG;
   const MoeGeo& g = plan->g;
   const MoeGeo& d = plan->gd;
-  DispatchPtrs P0, P;
-  std::memset(&P0, 0, sizeof(P0));
+  DispatchPtrs P;
+  DeriveParams D{};
   std::memset(&P, 0, sizeof(P));
   for (int r = 0; r < g.R; ++r) {
     if (!x[r] || !topk_idx[r] || !recv[r]) return PL_ERR_INVALID_ARG;
     if (((uintptr_t)x[r] & 15) || ((uintptr_t)recv[r] & 15) || ((uintptr_t)topk_idx[r] & 3)) return PL_ERR_ALIGNMENT;
     if (recv_meta && recv_meta[r] && ((uintptr_t)recv_meta[r] & 15)) return PL_ERR_ALIGNMENT;
-    P0.idx[r] = topk_idx[r];
+    D.idx[r] = topk_idx[r];
     P.x[r] = x[r];
     P.idx[r] = plan->d_ridx + (size_t)r * g.T * d.K;  // the derived per-rank routing
     P.recv[r] = recv[r];
@@ -1197,7 +1212,14 @@ pl_status_t pl_moe_dispatch_dedup(pl_moe_plan_t plan, const void* const* x, cons
     return PL_OK;
   }
   const long long n_tok = (long long)g.R * g.T;
-  if (!launch_after(true, moe_derive_ranks_kernel, dim3((unsigned)((n_tok + 255) / 256)), 256, 0, cs, P0, g.R, g.T, g.K, g.epr, d.K, plan->d_ridx, plan->d_rmask))
+  D.R = g.R;
+  D.T = g.T;
+  D.K = g.K;
+  D.epr = g.epr;
+  D.KR = d.K;
+  D.ridx = plan->d_ridx;
+  D.rmask = plan->d_rmask;
+  if (!launch_after(true, moe_derive_ranks_kernel, dim3((unsigned)((n_tok + 255) / 256)), 256, 0, cs, D))
     return PL_ERR_CUDA;
   const int launched = launch_dispatch(plan, P, d, plan->fused_dedup, cs);
   if (!launched) return PL_ERR_CUDA;

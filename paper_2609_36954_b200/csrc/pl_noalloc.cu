@@ -54,7 +54,9 @@ struct RingParams {
   unsigned long long units;     // 16-byte units of the element type per partition
   unsigned long long timeout_ns;
   int R;
+  uint64_t pad[4];
 };
+static_assert(cheap_params(sizeof(RingParams)), "launch cost");
 
 // dst = a + b over `n` units starting at unit `first`; a and dst may hold partials.
 template <int DT>
