@@ -123,9 +123,12 @@ typedef enum {
  *                         into all R outputs (no gather step, fewest bytes).
  *   PL_ALGO_RING          textbook ring; partial sums of bf16 data travel in fp32, of fp32
  *                         data as compensated fp32 pairs (PL_F32X2), of int32 data in int32.
- *                         With nothing about the launch asked for the hops go through the
- *                         shared memory of thread-block clusters where that is faster: the
- *                         info then has that launch, no scratch, and the bytes of inputs and
+ *                         With nothing about the launch asked for, a reducing ring's hops are folded
+ *                         into one chain of additions per element, in ring order (same bits, but
+ *                         no partial sum leaves the thread); with PL_OPT_RING_HOPS, and for a
+ *                         gathering ring, they go through the shared memory of thread-block
+ *                         clusters where that is faster than the op queues.  In both cases
+ *                         the info has that launch, no scratch, and the bytes of inputs and
  *                         outputs; the op list still states which rank adds what, in order.
  *   PL_ALGO_TREE          all-reduce only: binomial reduce to a root, binomial broadcast from it;
  *                         the root of chunk c is rank c mod R (rank 0 for a one-chunk message).
@@ -269,6 +272,10 @@ typedef struct {
  * and together with PL_OPT_NO_L2_HINTS.  Nothing in the paper corresponds to this option (its
  * inputs live in other GPUs' memories). */
 #define PL_OPT_INPUTS_LAST_USE 64u
+/* Keep the hops of a ring reduce-scatter or all-reduce: every rank is a CTA of its own and partial sums
+ * travel from rank to rank, as they have to between GPUs.  For those who measure the algorithm; the results are
+ * the same bits.  No effect on other schedules, nor on a ring that the op queues execute (which hops in any case). */
+#define PL_OPT_RING_HOPS 128u
 
 /* A buffer reference inside an op: rank's in/out/scratch buffer, byte offset, and the
  * element type stored there (partials of a bf16 reduction are PL_F32). */

@@ -54,7 +54,8 @@ struct pl_schedule_s {
   bool flat = false;              // no flags, everything left to the library: one CTA per tile (pl_datapath_flat.cu)
   FlatLaunch flat_launch{};
   std::vector<FlatSpan> flat_spans;  // uploaded in place of op list and flags
-  bool ring = false;              // ring with everything left to the library: a cluster per tile (pl_datapath_ring.cu)
+  bool folded = false;            // flat is a reducing ring: the hops of a unit are one chain of additions in a thread
+  bool ring = false;              // gathering ring, or one whose hops are asked for: a cluster per tile (pl_datapath_ring.cu)
   RingLaunch ring_launch{};
   int packet_ctas_per_rank = 0;   // > 0: packet datapath (layered one-shot all-reduce), CTAs per rank
   long long packet_break_op = -1; // test hook (pl_schedule_debug_break_wait on a packet schedule)
@@ -147,12 +148,14 @@ void fill_info(pl_schedule_s* S, int R) {
   I.stages = S->pol.stages;
   I.stage_bytes = S->pol.stage_bytes;
   I.slice_bytes = S->pol.slice_bytes;
-  if (S->ring) {  // what travels between ranks stays in shared memory
+  if (S->ring) {
     I.grid = S->ring_launch.grid;
     I.threads = S->ring_launch.threads;
     I.smem_bytes = (int32_t)S->ring_launch.smem_bytes;
     I.stages = 1;
     I.stage_bytes = S->ring_launch.tile * 16u;
+  }
+  if (S->ring || S->folded) {  // what travels between ranks stays on the SMs
     I.scratch_bytes = 0;
     I.hbm_bytes = 0;
     for (int r = 0; r < R; ++r) I.hbm_bytes += I.in_bytes[r] + I.out_bytes[r];
@@ -518,32 +521,41 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
     if (op.kind == PL_OP_COPY && op.bcast) S->bcast_copies = true;
   const bool all_default = !opts || (opts->n_ctas == 0 && opts->threads == 0 && opts->datapath == PL_DP_AUTO && opts->stages == 0 &&
                                      opts->stage_bytes == 0 && opts->slice_bytes == 0 && !idle_asked);
-  // A ring with nothing about the launch asked for: its hops inside clusters.  (A processing phase is
-  // the queue executors' business.)
+  // One CTA per tile of the spans, if the grid can hold them.
+  auto lay_flat = [&](bool reduce, bool all) {
+    uint64_t units = 0, blocks = 0;
+    for (const FlatSpan& f : S->flat_spans) units += f.units;
+    S->flat_launch = flat_launch(comm->R, reduce, all, pol.datapath == PL_DP_TMA, hook, units, comm->sm_count);
+    for (FlatSpan& f : S->flat_spans) {
+      f.first_block = (uint32_t)blocks;
+      blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;
+    }
+    S->flat_launch.blocks = (uint32_t)blocks;
+    S->flat = units > 0 && blocks <= 0x7FFFFFFFull;
+    if (S->flat) S->pol.idle_count = 0;
+  };
+  // A ring with nothing about the launch asked for.  (A processing phase is the queue executors' business.)  With every
+  // rank's buffers in one memory a thread can make all hops of a unit: faster than hops through memory at every size
+  // measured, 2 to 16 ranks (2 x 64 KiB 2.5 us both, 8 x 64 MiB 237 / 87 us; the others in pl_datapath_flat.cu).  An
+  // all-gather has no partial sums to keep, and goes as the direct one if that is what is wanted.
   if (!comm->planner && rq.algo == PL_ALGO_RING && !hook && !S->trace && all_default && rq.n_layers == 0) {
     const bool reduce = rq.coll != PL_ALLGATHER;
     const uint64_t part = rq.count_per_rank * (uint64_t)elem_size(comm->dtype) / (reduce ? (uint64_t)comm->R : 1ull) / 16;
-    S->ring = ring_shape(comm->R, comm->dtype, reduce, rq.coll != PL_REDUCE_SCATTER, part, rq.chunk_bytes, comm->sm_count, &S->ring_launch) &&
+    if (reduce && !(flags & PL_OPT_RING_HOPS)) {
+      ring_plan(comm->R, rq.coll == PL_ALLREDUCE, part, &S->flat_spans);
+      lay_flat(true, rq.coll == PL_ALLREDUCE);
+      S->folded = S->flat;
+    }
+    S->ring = !S->folded && ring_shape(comm->R, comm->dtype, reduce, rq.coll != PL_REDUCE_SCATTER, part, rq.chunk_bytes, comm->sm_count, &S->ring_launch) &&
               ring_prepare(comm->dtype, comm->R, S->ring_launch) > 0;
   }
   // No flags and nothing about the launch asked for: no queues.  Planner communicators keep the
   // queues, which is what their schedules are inspected for.
-  if (!comm->planner && rq.n_layers <= 1 && S->L.n_flags == 0 && !rq.staged && !S->trace && !S->layer_kernel && !S->ring && all_default) {
+  if (!comm->planner && rq.n_layers <= 1 && S->L.n_flags == 0 && !rq.staged && !S->trace && !S->layer_kernel && !S->ring && !S->folded && all_default) {
     bool reduce = false, all = false;
     const bool plan = flat_plan(S->L, comm->R, comm->dtype, &S->flat_spans, &reduce, &all);
     const bool queues = plan && queues_faster(comm->R, comm->dtype, hook, rq.algo, reduce, all, pol.datapath == PL_DP_TMA, S->L.message_bytes);
-    if (plan && !queues) {
-      uint64_t units = 0, blocks = 0;
-      for (const FlatSpan& f : S->flat_spans) units += f.units;
-      S->flat_launch = flat_launch(comm->R, reduce, all, pol.datapath == PL_DP_TMA, hook, units, comm->sm_count);
-      for (FlatSpan& f : S->flat_spans) {
-        f.first_block = (uint32_t)blocks;
-        blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;
-      }
-      S->flat_launch.blocks = (uint32_t)blocks;
-      S->flat = blocks <= 0x7FFFFFFFull;
-      if (S->flat) S->pol.idle_count = 0;
-    }
+    if (plan && !queues) lay_flat(reduce, all);
   }
   // A window of idle SMs needs: the bulk-copy datapath with one CTA per SM, no flags (a queue
   // may be claimed late, so no queue may wait for another), one staging buffer, at most 160 SMs,
@@ -1056,16 +1068,22 @@ pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index) {
     s->layer_break_queue = h.queue;
     return PL_OK;
   }
-  if (s->ring) {  // it reads no wait entries: from here on the op queues execute the schedule
-    s->ring = false;
+  if (s->ring || s->folded) {  // they read no wait entries: from here on the op queues execute the schedule
+    const bool ring = s->ring, folded = s->folded;
+    char* const spans = s->d_blob;
+    s->d_blob = nullptr;
+    s->ring = s->folded = s->flat = false;
     flatten(s, s->comm->dtype);
     const pl_status_t st = upload(s, s->comm->R);
     if (st != PL_OK) {
       if (s->d_blob) cudaFree(s->d_blob);
-      s->d_blob = nullptr;
-      s->ring = true;
+      s->d_blob = spans;
+      s->sync_bytes = 0;
+      s->ring = ring;
+      s->folded = s->flat = folded;
       return st;
     }
+    if (spans) cudaFree(spans);
     fill_info(s, s->comm->R);
   }
   const size_t pos = (size_t)s->topo_to_dev[op_index];

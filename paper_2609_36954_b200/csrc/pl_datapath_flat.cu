@@ -12,6 +12,12 @@
 // 657 -> 631 us, 16 MiB 50.9 -> 42.1 us, 4 MiB 15.6 -> 11.9 us, 16 MiB with residual 82.6 -> 60.6 us,
 // 4 MiB with residual 34.8 -> 18.0 us, all-to-all-v of 24 MiB 67.5 -> 61.0 us.
 //
+// A reducing ring comes here too, folded: the hops of a unit are a chain of additions in ring order, which one
+// thread makes with the same rounding (its span names the rank to start with).  A ring's bytes are mostly partial
+// sums in a wider type than the data; folded it reads inputs and writes outputs, like a direct reduction.  Through
+// neighbours' shared memory -> folded: reduce-scatter 8 x 64 MiB bf16 237 -> 87 us, fp32 277 -> 90, all-reduce
+// 8 x 64 MiB bf16 392 -> 160, 4 x 1 MiB fp32 7.55 -> 2.6, 8 x 64 KiB bf16 9.3 -> 2.7, 16 x 48 MiB fp32 814 -> 242.
+//
 // Two forms, by the schedule's datapath:
 //   register   the working set sits in L2 or nearly: one unit (16 bytes per operand) or a few per
 //              thread, all loads of a thread before its first add or store;
@@ -69,6 +75,7 @@ __device__ __forceinline__ Tile my_tile(const FlatParams& P) {
 }
 __device__ __forceinline__ uint32_t src_rank(const FlatSpan& s) { return s.ranks & 0xFFu; }
 __device__ __forceinline__ uint32_t dst_rank(const FlatSpan& s) { return (s.ranks >> 8) & 0xFFu; }
+__device__ __forceinline__ uint32_t first_rank(const FlatSpan& s) { return s.ranks >> 16; }
 
 __device__ __forceinline__ uint4 ld16_hint(const void* p, uint64_t policy) {
   uint4 v;
@@ -123,12 +130,14 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
     in_off[j] = (t.span.src_off + t.first + u) * 16ull;
   }
   uint4 q[U][NR];
+  const uint32_t first = first_rank(t.span);
 #pragma unroll
   for (int j = 0; j < U; ++j)
 #pragma unroll
     for (int s = 0; s < NR; ++s)
       if (live[j] && s < (int)R) {
-        const char* src = static_cast<const char*>(P.in[s]) + in_off[j];
+        const uint32_t rank = first + s < R ? first + s : first + s - R;
+        const char* src = static_cast<const char*>(P.in[rank]) + in_off[j];
         q[j][s] = (P.hints & 1u) ? ld16_hint(src, policy) : ld16(src);
       }
   // second operands: of 8 ranks at a time when the results go to every rank (16 of them and 16
@@ -235,8 +244,9 @@ __global__ void __launch_bounds__(kFlatBulkThreads) pl_flat_bulk_reduce_kernel(c
   if (tid < 32) {
     if (tid == 0) ptx::mbar_expect_tx(bar, bytes * (R + n_aux));
     __syncwarp();
-    if (tid < R + n_aux) {  // lane s: source s; lane R + k: second operand of rank k (or of the destination)
-      const char* from = tid < R ? static_cast<const char*>(P.in[tid]) + (t.span.src_off + t.first) * 16ull
+    if (tid < R + n_aux) {  // lane s: source s in order of addition; lane R + k: second operand of rank k (or of the destination)
+      const uint32_t s = first_rank(t.span) + tid, rank = s < R ? s : s - R;
+      const char* from = tid < R ? static_cast<const char*>(P.in[rank]) + (t.span.src_off + t.first) * 16ull
                                  : static_cast<const char*>(P.aux[ALL ? tid - R : to]) + at * 16ull;
       if ((P.hints & 1u) && tid < R) ptx::bulk_g2s_hint(tiles + tid * stride, from, bytes, bar, ptx::policy_evict_first());
       else ptx::bulk_g2s(tiles + tid * stride, from, bytes, bar);

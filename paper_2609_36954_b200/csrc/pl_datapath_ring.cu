@@ -1,5 +1,6 @@
-// Datapath for ring schedules whose grid is left to the library: a thread-block cluster per tile,
-// one CTA per rank, the hops through distributed shared memory.
+// Datapath for gathering rings, and for reducing rings whose hops are asked for (PL_OPT_RING_HOPS; else they are
+// folded, see pl_datapath_flat.cu), with the grid left to the library: a thread-block cluster per tile, one CTA per
+// rank, the hops through distributed shared memory.
 //
 // A ring moves the partial sums of a partition from rank to rank, in a wider type than the data, so
 // most of its bytes are partial sums: written by one rank, read once by the next.  On the op

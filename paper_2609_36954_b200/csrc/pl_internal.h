@@ -121,12 +121,13 @@ static_assert(cheap_params(sizeof(ExecParams)), "launch cost");
 // ---- flat execution of a schedule without flags (pl_datapath_flat.cu) ------------------------
 constexpr int kFlatThreads = 256, kFlatBulkThreads = 128;
 // A run of units (16 bytes of every operand): a copy from one rank's input, or the sum of every
-// rank's input at one offset in ascending rank order, to one rank's output or to all of them.
+// rank's input at one offset, to one rank's output or to all of them.  A sum adds rank f first, then f + 1, ...
+// (mod R): f = 0 is ascending order, a ring's partition k starts with rank k + 1.
 struct alignas(16) FlatSpan {
   uint64_t src_off, dst_off;  // units into the input(s) / into the output(s)
   uint64_t units;
   uint32_t first_block;       // CTAs of the spans in front
-  uint32_t ranks;             // source rank | destination rank << 8, 255 = every rank
+  uint32_t ranks;             // source rank | destination rank << 8 (255 = every rank) | first rank of a sum << 16
 };
 static_assert(sizeof(FlatSpan) == 32, "FlatSpan layout");
 struct FlatParams {
@@ -261,6 +262,8 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
 // The ops of a schedule without flags as spans; false if they are not of the forms a span describes.
 // `reduce` / `all` receive the one kind of op the schedule holds.  first_block is left to the caller.
 bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all);
+// The same for a reducing ring (a partition's chain of hops is one sum per unit); empty without units.
+void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* spans);
 // True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
 // tma: the policy picked the bulk-copy datapath (the working set streams from HBM).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes);

@@ -1314,6 +1314,13 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
   return !spans->empty();
 }
 
+void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* spans) {
+  spans->clear();
+  if (!part_units) return;
+  for (uint32_t k = 0; k < (uint32_t)R; ++k)
+    spans->push_back(FlatSpan{k * part_units, gather ? k * part_units : 0, part_units, 0, 255u | (gather ? 255u : k) << 8 | (k + 1) % (uint32_t)R << 16});
+}
+
 // A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a short
 // one (8 x 1 MiB 7.0 us, flat 7.5, with residual 7.1 / 8.0; 4 x 1 MiB 4.7 / 6.4; at 4 x 4 MiB flat is ahead,
 // 11.3 / 12.8), and a streaming one without residual (8 x 64 MiB 267 us, flat 286; 4 x 64 MiB 139 / 148; 16 x

@@ -69,6 +69,17 @@ int t_ring_shape(int R, int dtype, int reduce, int gather, uint64_t part_units, 
   return (int)L.smem_bytes;
 }
 
+// Spans of a folded ring: src_off, dst_off, units, first rank of the sum, destination rank (255 = every rank).
+int t_ring_plan(int R, int gather, uint64_t part_units, uint64_t* spans) {
+  std::vector<FlatSpan> f;
+  ring_plan(R, gather, part_units, &f);
+  for (size_t i = 0; i < f.size(); ++i) {
+    const uint64_t row[5] = {f[i].src_off, f[i].dst_off, f[i].units, f[i].ranks >> 16, (f[i].ranks >> 8) & 0xFFu};
+    for (int k = 0; k < 5; ++k) spans[5 * i + k] = row[k];
+  }
+  return (int)f.size();
+}
+
 // Validates a lowered schedule after a change to op `which`: 0 none, 1 another op with the same destination, 2 the op's
 // output shortened by 16 bytes, 3 the op's destination moved up by 16 bytes.
 int t_validate_changed(int R, int dtype, int coll, int algo, uint64_t count, uint64_t chunk, int n_layers, int which, int change, char* msg, int cap) {

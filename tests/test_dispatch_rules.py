@@ -27,6 +27,7 @@ def rules(tmp_path_factory):
     L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
     L.t_layers.argtypes = [i, u64, i]
     L.t_ring_shape.argtypes = [i, i, i, i, u64, u64, p]
+    L.t_ring_plan.argtypes = [i, i, u64, p]
     L.t_validate_changed.argtypes = [i, i, i, i, u64, u64, i, i, i, C.c_char_p, i]
     return L
 
@@ -228,3 +229,40 @@ def test_ops_with_flags_or_scratch_are_not_laid_out(rules):
     buf, red, every = np.zeros((64, 5), np.uint64), C.c_int(), C.c_int()
     for coll, algo in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT), (B.PL_ALLREDUCE, B.PL_ALGO_TREE), (B.PL_REDUCE_SCATTER, B.PL_ALGO_RING), (B.PL_ALLREDUCE, B.PL_ALGO_RING)):
         assert rules.t_flat_plan(4, B.PL_F32, coll, algo, 4096, 1024, None, 0, 0, buf.ctypes.data, 64, C.addressof(red), C.addressof(every)) == -1
+
+
+# a unit's hops in the op list, followed from rank to rank, name the ranks in the order in which a folded ring adds them
+@pytest.mark.parametrize("R", [2, 3, 5, 8, 16])
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "i32"])
+@pytest.mark.parametrize("units,chunk", [(1, 1 << 20), (7, 32), (65, 256)])
+def test_folded_rings_add_in_the_order_of_the_hops(rules, R, dtype, units, chunk):
+    dt, es = {"bf16": (B.PL_BF16, 2), "f32": (B.PL_F32, 4), "i32": (B.PL_I32, 4)}[dtype]
+    for coll in (B.PL_REDUCE_SCATTER, B.PL_ALLREDUCE):
+        comm = B.pl_comm_create_planner(R, dt)
+        s = B.pl_schedule_build(comm, coll, B.PL_ALGO_RING, units * 16 // es * R, chunk, None)
+        try:
+            terms, at = {}, {}  # (rank, buffer, byte offset of an op's destination) -> ranks added so far, first input unit
+            for o in B.pl_schedule_dump(s):
+                src = [(o.src[k].rank, o.src[k].buf, int(o.src[k].offset)) for k in range(o.n_src)]
+                dst = (o.dst.rank, o.dst.buf, int(o.dst.offset))
+                terms[dst] = [r for x in src for r in ([x[0]] if x[1] == B.PL_BUF_IN else terms[x])]
+                at[dst] = next((x[2] // 16 for x in src if x[1] == B.PL_BUF_IN), None)
+                at[dst] = at[src[0]] if at[dst] is None else at[dst]
+                n = o.count * (1 if o.kind == B.PL_OP_COPY else es) // 16
+                terms[dst + ("units",)] = n
+            buf = np.zeros((16, 5), np.uint64)
+            assert rules.t_ring_plan(R, coll == B.PL_ALLREDUCE, units, buf.ctypes.data) == R
+            covered = [0] * R
+            for key, order in terms.items():
+                if len(key) != 3 or key[1] != B.PL_BUF_OUT:
+                    continue
+                rank, _, off = key
+                n = terms[key + ("units",)]
+                span = next(x for x in buf[:R].astype(np.int64) if x[1] <= off // 16 < x[1] + x[2] and x[4] in (255, rank))
+                assert off // 16 + n <= span[1] + span[2] and at[key] - span[0] == off // 16 - span[1]
+                assert order == [(span[3] + k) % R for k in range(R)]
+                covered[rank] += n
+            assert covered == [units * (R if coll == B.PL_ALLREDUCE else 1)] * R
+        finally:
+            B.pl_schedule_destroy(s)
+            B.pl_comm_destroy(comm)

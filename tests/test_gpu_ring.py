@@ -1,5 +1,5 @@
-"""Ring schedules with everything left to the library (a cluster per tile, hops through shared memory)
-against the same schedule on the op queues: the same bits, at the edges of tiles and launch shapes."""
+"""Ring schedules with everything left to the library (reductions folded into one chain of additions per
+unit, or with their hops in clusters, through shared memory) against the same schedule on the op queues: the same bits, at the edges of tiles and launch shapes."""
 import pytest
 import torch
 
@@ -24,6 +24,16 @@ def test_reducing_rings(R, dtype, units):
     for coll in (B.PL_REDUCE_SCATTER, B.PL_ALLREDUCE):
         info = same_bits(R, dtype, build(coll, n), "tiles", **({"out_scale": 0.375} if dtype != "i32" else {}))
         assert info.scratch_bytes == 0
+
+
+@pytest.mark.parametrize("R,dtype", [(2, "i32"), (3, "f32"), (8, "bf16"), (16, "bf16")])
+@pytest.mark.parametrize("units", [1, 33, 4099, 65539])
+def test_rings_that_keep_their_hops(R, dtype, units):
+    """A CTA per rank: the same bits as on the queues, which is what the folded form is compared with above."""
+    n = 16 * units // SIZE[dtype] * R
+    for coll in (B.PL_REDUCE_SCATTER, B.PL_ALLREDUCE):
+        info = same_bits(R, dtype, build(coll, n), "tiles", flags=B.PL_OPT_RING_HOPS)
+        assert info.scratch_bytes == 0 and info.grid % R == 0
 
 
 # up to 1 MiB per rank and 8 MiB in all in clusters, above that on the op queues (two ranks gather without flags: tiles)
