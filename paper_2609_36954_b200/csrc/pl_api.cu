@@ -53,7 +53,9 @@ struct pl_schedule_s {
   int layer_break_layer = -1, layer_break_queue = -1;  // test hook (pl_schedule_debug_break_wait without flag words)
   bool flat = false;              // no flags, everything left to the library: one CTA per tile (pl_datapath_flat.cu)
   FlatLaunch flat_launch{};
-  std::vector<FlatSpan> flat_spans;  // uploaded in place of op list and flags
+  std::vector<FlatSpan> flat_spans;  // uploaded in place of op list and flags, unless they are a run
+  bool flat_is_run = false;
+  FlatRun flat_run{};
   bool folded = false;            // flat is a reducing ring: the hops of a unit are one chain of additions in a thread
   bool ring = false;              // gathering ring, or one whose hops are asked for: a cluster per tile (pl_datapath_ring.cu)
   RingLaunch ring_launch{};
@@ -224,6 +226,7 @@ void flatten(pl_schedule_s* S, int dtype) {
 
 pl_status_t upload(pl_schedule_s* S, int R) {
   if (S->ring) return PL_OK;  // sizes and pointers are all it reads
+  if (S->flat && S->flat_is_run) return PL_OK;  // its parameters say where its tiles are
   if (S->flat) {
     S->blob_bytes = S->flat_spans.size() * sizeof(FlatSpan);
     if (cudaMalloc(&S->d_blob, S->blob_bytes) != cudaSuccess) { cudaGetLastError(); return PL_ERR_OOM; }
@@ -531,6 +534,8 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
       blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;
     }
     S->flat_launch.blocks = (uint32_t)blocks;
+    S->flat_is_run = units > 0 && flat_run(S->flat_spans, &S->flat_run);
+    if (S->flat_is_run) S->flat_run.blocks = (uint32_t)(blocks / S->flat_spans.size());
     S->flat = units > 0 && blocks <= 0x7FFFFFFFull;
     if (S->flat) S->pol.idle_count = 0;
   };
@@ -1193,6 +1198,7 @@ pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
     F.out_scale = s->out_scale;
     F.status = s->comm->d_status;
     F.timeout_ns = s->timeout_ns;
+    F.run = s->flat_run;
     if (launch_flat(s->comm->dtype, F, s->flat_launch, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
       cudaGetLastError();
       return PL_ERR_CUDA;

@@ -127,9 +127,16 @@ struct alignas(16) FlatSpan {
   uint64_t src_off, dst_off;  // units into the input(s) / into the output(s)
   uint64_t units;
   uint32_t first_block;       // CTAs of the spans in front
-  uint32_t ranks;             // source rank | destination rank << 8 (255 = every rank) | first rank of a sum << 16
+  uint32_t ranks;             // source rank | destination rank << 8 (255 = every rank) | first rank of a sum << 16 (R = 0)
 };
 static_assert(sizeof(FlatSpan) == 32, "FlatSpan layout");
+// Spans of equal length at equal distances, which the parameters of a launch can describe: span k starts k steps into
+// the inputs and outputs, and its `ranks` are k rank steps on from the first one's.
+struct FlatRun {
+  uint64_t units, src_step, dst_step;
+  uint32_t blocks;  // CTAs of a span
+  uint32_t ranks, rank_step, pad;
+};
 struct FlatParams {
   const void* in[PL_MAX_RANKS];
   void* out[PL_MAX_RANKS];
@@ -141,7 +148,8 @@ struct FlatParams {
   float out_scale;
   int* status;
   unsigned long long timeout_ns;
-  uint64_t pad[6];
+  FlatRun run;             // the spans, if `spans` is null
+  uint64_t pad;
 };
 static_assert(cheap_params(sizeof(FlatParams)), "launch cost");
 struct FlatLaunch {  // host side: which kernel, how many CTAs
@@ -262,7 +270,9 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
 // The ops of a schedule without flags as spans; false if they are not of the forms a span describes.
 // `reduce` / `all` receive the one kind of op the schedule holds.  first_block is left to the caller.
 bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all);
-// The same for a reducing ring (a partition's chain of hops is one sum per unit); empty without units.
+// True if the spans are a run; `blocks` of it is left to the caller.
+bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run);
+// flat_plan() for a reducing ring (a partition's chain of hops is one sum per unit); empty without units.
 void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* spans);
 // True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
 // tma: the policy picked the bulk-copy datapath (the working set streams from HBM).

@@ -1318,7 +1318,20 @@ void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* s
   spans->clear();
   if (!part_units) return;
   for (uint32_t k = 0; k < (uint32_t)R; ++k)
-    spans->push_back(FlatSpan{k * part_units, gather ? k * part_units : 0, part_units, 0, 255u | (gather ? 255u : k) << 8 | (k + 1) % (uint32_t)R << 16});
+    spans->push_back(FlatSpan{k * part_units, gather ? k * part_units : 0, part_units, 0, 255u | (gather ? 255u : k) << 8 | (k + 1) << 16});
+}
+
+bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run) {
+  const FlatSpan& a = spans[0];
+  const FlatSpan& b = spans.size() > 1 ? spans[1] : a;
+  *run = FlatRun{a.units, b.src_off, b.dst_off, 0, a.ranks, b.ranks - a.ranks, 0};
+  if (spans.size() == 1) run->src_step = run->dst_step = 0;
+  for (size_t k = 0; k < spans.size(); ++k) {
+    const FlatSpan& f = spans[k];
+    if (f.units != run->units || f.src_off != k * run->src_step || f.dst_off != k * run->dst_step || f.ranks != run->ranks + (uint32_t)k * run->rank_step)
+      return false;
+  }
+  return true;
 }
 
 // A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a short

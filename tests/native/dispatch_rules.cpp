@@ -80,6 +80,23 @@ int t_ring_plan(int R, int gather, uint64_t part_units, uint64_t* spans) {
   return (int)f.size();
 }
 
+// Whether spans (rows as t_flat_plan writes them) are a run, and the run's spans written over them.
+int t_flat_run(uint64_t* spans, int n) {
+  std::vector<FlatSpan> f;
+  for (int i = 0; i < n; ++i) {
+    const uint64_t* s = spans + 5 * i;
+    f.push_back(FlatSpan{s[0], s[1], s[2], 0, (uint32_t)(s[3] | s[4] << 8)});
+  }
+  FlatRun run;
+  if (!flat_run(f, &run)) return 0;
+  for (uint64_t k = 0; k < (uint64_t)n; ++k) {
+    const uint32_t ranks = run.ranks + (uint32_t)k * run.rank_step;
+    const uint64_t row[5] = {k * run.src_step, k * run.dst_step, run.units, ranks & 0xFFu, ranks >> 8 & 0xFFu};
+    for (int i = 0; i < 5; ++i) spans[5 * k + i] = row[i];
+  }
+  return 1;
+}
+
 // Validates a lowered schedule after a change to op `which`: 0 none, 1 another op with the same destination, 2 the op's
 // output shortened by 16 bytes, 3 the op's destination moved up by 16 bytes.
 int t_validate_changed(int R, int dtype, int coll, int algo, uint64_t count, uint64_t chunk, int n_layers, int which, int change, char* msg, int cap) {

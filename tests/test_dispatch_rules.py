@@ -27,6 +27,7 @@ def rules(tmp_path_factory):
     L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
     L.t_layers.argtypes = [i, u64, i]
     L.t_ring_shape.argtypes = [i, i, i, i, u64, u64, p]
+    L.t_flat_run.argtypes = [p, i]
     L.t_ring_plan.argtypes = [i, i, u64, p]
     L.t_validate_changed.argtypes = [i, i, i, i, u64, u64, i, i, i, C.c_char_p, i]
     return L
@@ -220,6 +221,10 @@ def test_spans_say_what_the_ops_say(rules, R, dtype, units):
             assert {s_[4] == 255 for s_ in spans} == {bool(every.value)} and {s_[3] == 255 for s_ in spans} == {bool(red.value)}
             for a, b in zip(landing(R, ops, out_units), landing(R, spans, out_units)):
                 assert np.array_equal(a, b)
+            # a run says the same: what is of equal parts in one row, and nothing with two steps
+            run = rules.t_flat_run(buf.ctypes.data, n)
+            assert run or coll not in (B.PL_REDUCE_SCATTER, B.PL_ALLGATHER, B.PL_ALLREDUCE, B.PL_SCATTER, B.PL_GATHER)
+            assert not run or [tuple(int(x) for x in row) for row in buf[:n]] == spans
             B.pl_schedule_destroy(s)
         finally:
             B.pl_comm_destroy(comm)
