@@ -385,7 +385,10 @@ FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, u
     const uint32_t n_aux = (hook & PL_HOOK_RESIDUAL) ? (all ? (uint32_t)R : 1u) : 0u;
     F.smem_bytes = kBarBytes + ((uint32_t)R + n_aux) * F.tile * 16u;
   } else if (bulk) {
-    F.tile = all ? 128u : 256u;  // all-gather of 64 MiB: 93.2 us with 128 units, 95.1 with 256, 99.4 with 1024
+    // all-gather 8 x 64 MiB 93.2 us with 128 units, 95.1 with 256, 99.4 with 1024.  With two or three stores for a load a CTA
+    // of 128 is over too soon: reduce-scatter + all-gather 2 x 64 MiB 66.3 us, 256 units 52.9, 512 54.0; 2 x 128 MiB 129.0,
+    // 114.8, 115.2; 3 x 64 MiB 77.7, 74.7; 4 x 64 MiB 93.4, 93.5; 5 x 64 MiB 117.5, 117.7
+    F.tile = all && R > 3 ? 128u : 256u;
     F.smem_bytes = kBarBytes + F.tile * 16u;
   } else if (reduce) {
     const int U = hook ? (R <= 2 ? 2 : 1) : (R <= 2 ? 4 : R <= 4 ? 2 : 1);  // FlatUnits
