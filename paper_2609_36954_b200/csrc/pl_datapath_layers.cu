@@ -16,12 +16,13 @@
 //   - CLUSTER: when the whole schedule fits 16 CTAs, they form one thread-block cluster and the
 //     flag is the cluster barrier (release / acquire): one hop instead of an increment in L2 and a
 //     poll that has to see it.
-// What bounds it: at the small end the chain (outputs acknowledged by L2 about 0.6 us, barrier or
-// flag 0.3-0.6 us, inputs from L2 0.4 us), at 1 MiB the chain plus 16 MiB of L2 traffic per layer
+// What bounds it: at the small end the chain (outputs acknowledged by L2 about 0.6 us, barrier 0.1 or
+// flag 0.6 us, inputs from L2 0.3 us), at 1 MiB the chain plus 16 MiB of L2 traffic per layer
 // (2.6 us at DRAM rate, which the prefetch and the write-back overlap with the chain).
 // Measured on B200, R = 8, bf16, 80 layers in one launch, three sets of buffers in turn, us per
-// layer, register executor -> this kernel: 4 KiB 2.0 -> 1.17, 16 KiB 2.16 -> 1.22 (cluster); 64 KiB 3.20 -> 1.95,
-// 128 KiB 3.28 -> 2.00, 512 KiB 3.86 -> 2.63, 1 MiB 5.00 -> 3.64 (flags).
+// layer, register executor -> this kernel: 4 KiB 2.0 -> 1.01, 16 KiB 2.16 -> 1.12, 32 KiB 1.41 (cluster); 64 KiB 3.20 -> 1.74,
+// 128 KiB 3.28 -> 1.78, 512 KiB 3.86 -> 2.49, 1 MiB 5.00 -> 3.46 (flags).  Clock stamps of a 16 KiB layer, cycles: loads
+// issued 66, arrived 445, summed and stored 290, acknowledged (release) 1160, barrier 200.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -43,13 +44,23 @@ __device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // One unit (16 bytes of every source) of a layer: NR bounds the ranks, all loads before the adds.
-template <int DT, int NR, bool HOOK>
-__device__ __forceinline__ void layer_unit(const ExecParams& P, uint64_t in_off, uint64_t out_off) {
-  const int R = P.n_ranks;
+// EXACT: there are NR ranks, so the loads and stores follow one another without a test of the rank between them, which
+// costs a load 37 cycles (8 ranks, 16 KiB: the loads are issued in 66 cycles instead of 299).  The compiler may
+// then spread them over the additions, which waits for memory several times over (8 x 64 KiB 146 -> 212 us for 80
+// layers): one word of each goes through a shuffle to its own lane, and every lane of the warp waits there for all.
+// So all 32 lanes come here, and one with nothing to do (`live` false) loads what another loads and stores nothing.
+template <int DT, int NR, bool HOOK, bool EXACT>
+__device__ __forceinline__ void layer_unit(const ExecParams& P, uint64_t in_off, uint64_t out_off, bool live) {
+  const int R = EXACT ? NR : P.n_ranks;
   uint4 q[NR];
 #pragma unroll
   for (int s = 0; s < NR; ++s)
     if (s < R) q[s] = ld16(static_cast<const char*>(P.base[kSlotIn + s]) + in_off);
+  if constexpr (EXACT) {
+#pragma unroll
+    for (int s = 0; s < NR; ++s) q[s].w = __shfl_sync(0xFFFFFFFFu, q[s].w, (int)(threadIdx.x & 31u));
+    if (!live) return;
+  }
   uint4 second[HOOK ? NR : 1];
   if constexpr (HOOK) {
     if (P.hook & PL_HOOK_RESIDUAL) {
@@ -80,6 +91,17 @@ __device__ __forceinline__ void layer_unit(const ExecParams& P, uint64_t in_off,
   }
 }
 
+// The units of one layer that fall to this thread, `n` apart.  Not unrolled: there is one as a rule, and the shorter
+// code is fetched sooner (8 x 32 KiB 142 -> 125 us for 80 layers).
+template <int DT, int NR, bool HOOK, bool EXACT>
+__device__ __forceinline__ void layer_slice(const ExecParams& P, uint64_t in_off, uint64_t out_off, uint32_t out_unit, uint32_t units, uint32_t t, uint32_t n) {
+#pragma unroll 1
+  for (uint32_t u = t; EXACT ? (u & ~31u) < units : u < units; u += n) {  // EXACT: the same number of turns for a whole warp
+    const uint32_t at = EXACT ? min(u, units - 1u) : u;
+    layer_unit<DT, NR, HOOK, EXACT>(P, in_off + at * 16ull, out_off + (uint64_t)at * out_unit, u < units);
+  }
+}
+
 // Lines of one layer's operands for this CTA's slice into L2: line j of rank s by the thread with
 // number j * NR + s modulo n.  The slice starts on a 16-byte boundary, so it can touch one line
 // more than its bytes fill; that one is left to the load.
@@ -87,6 +109,7 @@ template <int NR>
 __device__ __forceinline__ void ask_for_layer(const ExecParams& P, uint64_t in_off, uint32_t units, uint32_t t, uint32_t n) {
   const uint32_t lines = (units + 7u) >> 3;
   const bool residual = P.hook & PL_HOOK_RESIDUAL;
+#pragma unroll 1
   for (uint32_t j = t; j < lines * NR; j += n) {
     const uint32_t line = j / NR, s = j % NR;
     if (s >= (uint32_t)P.n_ranks) continue;
@@ -96,7 +119,9 @@ __device__ __forceinline__ void ask_for_layer(const ExecParams& P, uint64_t in_o
   }
 }
 
-template <int DT, int NR, bool HOOK, bool CLUSTER>
+// FULL: with the stamps of a trace and the hook that breaks a wait.  They are a kernel of their own because the code in
+// the loop costs a layer time even if it is not run (80 layers of 4 KiB 86 -> 81 us without it).
+template <int DT, int NR, bool HOOK, bool CLUSTER, bool EXACT, bool FULL>
 __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThreads) pl_layers_kernel(const __grid_constant__ ExecParams P,
                                                                                   const __grid_constant__ LayerParams Y) {
   __shared__ int s_abort;
@@ -115,7 +140,7 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
   if constexpr (CLUSTER) {
     const uint32_t movers = blockDim.x - 32u;
     for (uint32_t l = 0; l < Y.n_layers; ++l) {
-      if ((int)l == Y.break_layer) {
+      if (FULL && (int)l == Y.break_layer) {
         // test hook: a wait that nothing satisfies.  Every CTA leaves here; the one whose op was
         // broken gives up after the time limit and says so.
         if ((int)q == Y.break_queue && tid == 0) {
@@ -126,21 +151,21 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
         break;
       }
       const uint64_t in_off = in_off0 + l * Y.in_stride, out_off = out_off0 + l * Y.out_stride;
-      if (P.trace && tid == 0) P.trace[2ull * topo] = globaltimer_ns();
+      if (FULL && P.trace && tid == 0) P.trace[2ull * topo] = globaltimer_ns();
       if (tid < movers) {
-        for (uint32_t u = tid; u < units; u += movers) layer_unit<DT, NR, HOOK>(P, in_off + u * 16ull, out_off + (uint64_t)u * out_unit);
+        layer_slice<DT, NR, HOOK, EXACT>(P, in_off, out_off, out_unit, units, tid, movers);
       } else if (l + 1 < Y.n_layers) {
         ask_for_layer<NR>(P, in_off + Y.in_stride, units, tid - movers, 32u);
       }
       if (l + 1 < Y.n_layers) {
-        if (P.trace) {
+        if (FULL && P.trace) {
           __syncthreads();
           if (tid == 0) P.trace[2ull * topo + 1] = globaltimer_ns();
         }
         __syncwarp();
         cluster_arrive_release();
         cluster_wait_acquire();
-      } else if (P.trace) {
+      } else if (FULL && P.trace) {
         __syncthreads();
         if (tid == 0) P.trace[2ull * topo + 1] = globaltimer_ns();
       }
@@ -154,7 +179,7 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
       if (l > 0) {
         if (tid == 0) {
           // every CTA signals once per layer; acquire, bounded by the time limit
-          const unsigned long long need = epoch * (gridDim.x + (((int)l == Y.break_layer && (int)q == Y.break_queue) ? 1ull : 0ull));
+          const unsigned long long need = epoch * (gridDim.x + ((FULL && (int)l == Y.break_layer && (int)q == Y.break_queue) ? 1ull : 0ull));
           unsigned long long seen = ld_acquire_u64(flag);
           if (seen < need) {
             const unsigned long long t0 = globaltimer_ns();
@@ -176,12 +201,12 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
         if (s_abort) { aborted = true; break; }
       }
       const uint64_t in_off = in_off0 + l * Y.in_stride, out_off = out_off0 + l * Y.out_stride;
-      if (P.trace && tid == 0) P.trace[2ull * topo] = globaltimer_ns();
-      for (uint32_t u = tid; u < units; u += blockDim.x) layer_unit<DT, NR, HOOK>(P, in_off + u * 16ull, out_off + (uint64_t)u * out_unit);
-      if (l + 1 < Y.n_layers || P.trace) {
+      if (FULL && P.trace && tid == 0) P.trace[2ull * topo] = globaltimer_ns();
+      layer_slice<DT, NR, HOOK, EXACT>(P, in_off, out_off, out_unit, units, tid, blockDim.x);
+      if (l + 1 < Y.n_layers || (FULL && P.trace)) {
         __syncthreads();  // every thread's writes are done
         if (tid == 0) {
-          if (P.trace) P.trace[2ull * topo + 1] = globaltimer_ns();
+          if (FULL && P.trace) P.trace[2ull * topo + 1] = globaltimer_ns();
           // cumulative: covers the other threads' stores, observed through the barrier
           if (l + 1 < Y.n_layers) red_release_add_u64(flag, 1ull);
         }
@@ -205,12 +230,11 @@ __global__ void __launch_bounds__(CLUSTER ? kMaxClusterThreads + 32 : kMaxThread
   }
 }
 
-template <int DT, int NR, bool HOOK, bool CLUSTER>
-void configure(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int grid, int threads, bool overlap) {
+void configure(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int grid, int threads, bool cluster, bool overlap) {
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)(threads + (CLUSTER ? 32 : 0)));
+  cfg.blockDim = dim3((unsigned)(threads + (cluster ? 32 : 0)));
   int na = 0;
-  if (CLUSTER) {
+  if (cluster) {
     attr[na].id = cudaLaunchAttributeClusterDimension;
     attr[na].val.clusterDim.x = (unsigned)grid;
     attr[na].val.clusterDim.y = 1;
@@ -226,25 +250,40 @@ void configure(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int grid, int
   cfg.numAttrs = na;
 }
 
+using LayerKernel = void (*)(ExecParams, LayerParams);
+
+// The kernel of a launch: a processing phase has one form, with everything in it, and so have traces and broken waits.
 template <int DT, int NR, bool HOOK, bool CLUSTER>
-cudaError_t launch_t(const ExecParams& P, const LayerParams& Y, int grid, int threads, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
-  configure<DT, NR, HOOK, CLUSTER>(cfg, attr, grid, threads, P.overlap_launch);
-  cfg.stream = stream;
-  return cudaLaunchKernelEx(&cfg, pl_layers_kernel<DT, NR, HOOK, CLUSTER>, P, Y);
+LayerKernel kernel_t(int R, bool full) {
+  if constexpr (HOOK) return pl_layers_kernel<DT, NR, true, CLUSTER, false, true>;
+  else if (full) return pl_layers_kernel<DT, NR, false, CLUSTER, false, true>;
+  else {
+    auto exact = [](auto n) -> LayerKernel { return pl_layers_kernel<DT, n(), false, CLUSTER, true, false>; };
+    switch (R) {
+      case 2: return exact(std::integral_constant<int, 2>{});
+      case 3: return exact(std::integral_constant<int, 3>{});
+      case 4: return exact(std::integral_constant<int, 4>{});
+      case 5: return exact(std::integral_constant<int, 5>{});
+      case 6: return exact(std::integral_constant<int, 6>{});
+      case 7: return exact(std::integral_constant<int, 7>{});
+      case 8: return exact(std::integral_constant<int, 8>{});
+      case 12: return exact(std::integral_constant<int, 12>{});
+      case 16: return exact(std::integral_constant<int, 16>{});
+      default: return pl_layers_kernel<DT, NR, false, CLUSTER, false, false>;
+    }
+  }
 }
 
-template <int DT, int NR, bool HOOK>
-bool cluster_fits_t(int grid, int threads) {
+// Up to 16 CTAs: more than the portable 8 needs the opt-in (a per-device attribute of the function, raised here, when
+// the schedule is built, and kept).
+bool cluster_fits(LayerKernel kernel, int grid, int threads) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   int n = 0;
-  configure<DT, NR, HOOK, true>(cfg, attr, grid, threads, false);
-  // up to 16 CTAs: more than the portable 8 needs the opt-in (a per-device attribute of the function, raised here, when
-  // the schedule is built, and kept)
-  if ((grid > 8 && cudaFuncSetAttribute(pl_layers_kernel<DT, NR, HOOK, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
-      cudaOccupancyMaxActiveClusters(&n, pl_layers_kernel<DT, NR, HOOK, true>, &cfg) != cudaSuccess) {
+  configure(cfg, attr, grid, threads, true, false);
+  const void* f = reinterpret_cast<const void*>(kernel);
+  if ((grid > 8 && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -268,13 +307,22 @@ auto pick(int dtype, int R, bool hook, F f) {
 
 cudaError_t launch_layers(int dtype, const ExecParams& P, const LayerParams& Y, int grid, int threads, bool cluster, cudaStream_t stream) {
   if (dtype == PL_U8 || (dtype == PL_I32 && P.hook)) return cudaErrorInvalidValue;
-  return pick(dtype, P.n_ranks, P.hook != 0, [&](auto dt, auto nr, auto hk) {
-    return cluster ? launch_t<dt(), nr(), hk(), true>(P, Y, grid, threads, stream) : launch_t<dt(), nr(), hk(), false>(P, Y, grid, threads, stream);
+  const bool full = P.trace || Y.break_layer >= 0;
+  const LayerKernel kernel = pick(dtype, P.n_ranks, P.hook != 0, [&](auto dt, auto nr, auto hk) {
+    return cluster ? kernel_t<dt(), nr(), hk(), true>(P.n_ranks, full) : kernel_t<dt(), nr(), hk(), false>(P.n_ranks, full);
   });
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  configure(cfg, attr, grid, threads, cluster, P.overlap_launch);
+  cfg.stream = stream;
+  return cudaLaunchKernelEx(&cfg, kernel, P, Y);
 }
 
+// Both kernels that a schedule may launch: the hook that breaks a wait can be set after the build.
 bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads) {
-  return pick(dtype, R, hook, [&](auto dt, auto nr, auto hk) { return cluster_fits_t<dt(), nr(), hk()>(grid, threads); });
+  return pick(dtype, R, hook, [&](auto dt, auto nr, auto hk) {
+    return cluster_fits(kernel_t<dt(), nr(), hk(), true>(R, false), grid, threads) && cluster_fits(kernel_t<dt(), nr(), hk(), true>(R, true), grid, threads);
+  });
 }
 
 }  // namespace pl
