@@ -117,19 +117,30 @@ __device__ __forceinline__ void store_sum(const FlatParams& P, const Acc<DT>& ac
 }
 
 // ---- register form ---------------------------------------------------------------------------
+// Sums, and copies to every rank, do not release the launch behind them: it is set up as their CTAs exit.  Released at
+// the start, its CTAs take the room that is left and then share SMs while others idle, as soon as the host enqueues
+// faster than the GPU finishes (all-reduce, us, released at the start / after the loads / not: 8 x 1 MiB 4.85 / 3.73 / 3.02,
+// 2 x 4 MiB 4.45 / 3.78 / 2.90, 8 x 2 MiB 6.4 / 6.0 / 5.2, 16 x 256 KiB 4.66 / 3.39 / 3.20, 16 x 1 MiB 6.8 / 6.6 / 6.1, 8 x 64 KiB 2.94 / 2.98 / 2.95;
+// reduce-scatter + all-gather 8 x 2 MiB, the all-gather released / not, 8.7 / 8.3).  Copies to one rank read their span from
+// memory first and do (all-to-all-v 8 x 2 MiB 5.0 / 5.4), and so do the bulk-copy forms (no difference, or 1 % slower without).
 // Units per thread of a reduce: about 8 operand vectors in flight (16 with a second operand per rank).
 template <int NR, bool HOOK>
 struct FlatUnits {
   static constexpr int value = HOOK ? (NR <= 2 ? 2 : 1) : (NR <= 2 ? 4 : NR <= 4 ? 2 : 1);
 };
 
-// NR bounds the ranks, so that the register of every operand is a compile-time constant.
-template <int DT, int NR, bool HOOK, bool ALL>
+// NR bounds the ranks, so that the register of every operand is a compile-time constant.  EXACT: there are NR ranks, and
+// the loads follow one another without a test between them; a word of each source goes through a shuffle to its own
+// lane, where the warp waits for all of them (see layer_unit() in pl_datapath_layers.cu).  A unit past the end of the
+// tile is then loaded from its last one and not stored.  With a processing phase that is faster at every size (residual,
+// bf16, us: 4 x 4 MiB 9.5 -> 8.9, 8 x 1.6 MiB 9.3 -> 9.0, 8 x 4 MiB 18.1 -> 17.2, 16 x 4 MiB 33.6 -> 31.9; fp32 8 x 2 MiB 11.1 -> 10.2);
+// without one the bursts are slower where inputs and outputs take 20 to 40 MB of L2 (8 x 2 MiB 6.4 / 8.2, 16 x 1 MiB
+// 6.9 / 8.3, while 16 x 2 MiB 13.0 / 12.2), so it goes with HOOK.
+template <int DT, int NR, bool HOOK, bool ALL, bool EXACT>
 __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const __grid_constant__ FlatParams P) {
   constexpr int U = FlatUnits<NR, HOOK>::value;
-  pdl_launch_dependents();
   const Tile t = my_tile(P);
-  const uint32_t R = (uint32_t)P.n_ranks, to = dst_rank(t.span);
+  const uint32_t R = EXACT ? (uint32_t)NR : (uint32_t)P.n_ranks, to = dst_rank(t.span);
   const bool residual = HOOK && (P.hook & PL_HOOK_RESIDUAL);
   const uint32_t out_b = (HOOK && DT == PL_BF16 && (P.hook & PL_HOOK_F32_OUT)) ? 32u : 16u;
   const uint64_t policy = (P.hints & 1u) ? ptx::policy_evict_first() : 0ull;
@@ -138,22 +149,27 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
   bool live[U];
 #pragma unroll
   for (int j = 0; j < U; ++j) {
-    const uint32_t u = threadIdx.x + (uint32_t)(j * kFlatThreads);
+    uint32_t u = threadIdx.x + (uint32_t)(j * kFlatThreads);
     live[j] = u < t.units;
+    if (EXACT) u = min(u, t.units - 1u);
     at[j] = t.span.dst_off + t.first + u;
     in_off[j] = (t.span.src_off + t.first + u) * 16ull;
   }
   uint4 q[U][NR];
   const uint32_t first = first_rank(t.span);
+  // one test of the hint for all loads (in front of each: 16 x 2 MiB 15.1 us, so 13.0; 8 x 2 MiB 7.4 / 6.4)
+  auto load = [&](auto ld) {
 #pragma unroll
-  for (int j = 0; j < U; ++j)
+    for (int j = 0; j < U; ++j)
 #pragma unroll
-    for (int s = 0; s < NR; ++s)
-      if (live[j] && s < (int)R) {
-        const uint32_t rank = first + s < R ? first + s : first + s - R;
-        const char* src = static_cast<const char*>(P.in[rank]) + in_off[j];
-        q[j][s] = (P.hints & 1u) ? ld16_hint(src, policy) : ld16(src);
-      }
+      for (int s = 0; s < NR; ++s)
+        if (EXACT || (live[j] && s < (int)R)) {
+          const uint32_t rank = first + s < R ? first + s : first + s - R;
+          q[j][s] = ld(static_cast<const char*>(P.in[rank]) + in_off[j]);
+        }
+  };
+  if (P.hints & 1u) load([&](const char* src) { return ld16_hint(src, policy); });
+  else load([](const char* src) { return ld16(src); });
   // second operands: of 8 ranks at a time when the results go to every rank (16 of them and 16
   // sources would not fit the registers), else the one of the destination
   constexpr int NS = !HOOK ? 1 : !ALL ? 1 : NR < 8 ? NR : 8;
@@ -163,7 +179,15 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
     for (int j = 0; j < U; ++j)
 #pragma unroll
       for (int k = 0; k < NS; ++k)
-        if (live[j] && (!ALL || k < (int)R)) second[j][k] = ld16(static_cast<const char*>(P.aux[ALL ? k : (int)to]) + at[j] * 16ull);
+        if (EXACT || (live[j] && (!ALL || k < (int)R))) second[j][k] = ld16(static_cast<const char*>(P.aux[ALL ? k : (int)to]) + at[j] * 16ull);
+  }
+  if constexpr (EXACT) {
+    const int lane = (int)(threadIdx.x & 31u);
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+#pragma unroll
+      for (int s = 0; s < NR; ++s) q[j][s].w = __shfl_sync(0xFFFFFFFFu, q[j][s].w, lane);
+    }
   }
 #pragma unroll
   for (int j = 0; j < U; ++j) {
@@ -194,7 +218,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
 
 template <int U, bool ALL>
 __global__ void __launch_bounds__(kFlatThreads) pl_flat_copy_kernel(const __grid_constant__ FlatParams P) {
-  pdl_launch_dependents();
+  if (!ALL) pdl_launch_dependents();
   const Tile t = my_tile(P);
   const uint64_t policy = (P.hints & 1u) ? ptx::policy_evict_first() : 0ull;
   pdl_wait();
@@ -356,9 +380,18 @@ cudaError_t launch(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream
   return cudaLaunchKernelEx(&cfg, kernel, P);
 }
 
+template <int DT, int NR, bool HOOK, bool EXACT>
+cudaError_t launch_all(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
+  return F.all ? launch<pl_flat_reduce_kernel<DT, NR, HOOK, true, EXACT>>(P, F, stream) : launch<pl_flat_reduce_kernel<DT, NR, HOOK, false, EXACT>>(P, F, stream);
+}
 template <int DT, int NR, bool HOOK>
 cudaError_t launch_reduce(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
-  return F.all ? launch<pl_flat_reduce_kernel<DT, NR, HOOK, true>>(P, F, stream) : launch<pl_flat_reduce_kernel<DT, NR, HOOK, false>>(P, F, stream);
+  if constexpr (HOOK) {
+    if (P.n_ranks == NR) return launch_all<DT, NR, true, true>(P, F, stream);
+    if (P.n_ranks == 3) return launch_all<DT, 3, true, true>(P, F, stream);
+    if (P.n_ranks == 6) return launch_all<DT, 6, true, true>(P, F, stream);
+  }
+  return launch_all<DT, NR, HOOK, false>(P, F, stream);
 }
 template <int DT, bool HOOK>
 cudaError_t launch_dt(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
