@@ -534,6 +534,7 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
       blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;
     }
     S->flat_launch.blocks = (uint32_t)blocks;
+    S->flat_launch.release = flat_release(reduce, all, S->flat_launch.bulk, blocks);
     S->flat_is_run = units > 0 && flat_run(S->flat_spans, &S->flat_run);
     if (S->flat_is_run) S->flat_run.blocks = (uint32_t)(blocks / S->flat_spans.size());
     S->flat = units > 0 && blocks <= 0x7FFFFFFFull;
@@ -1199,6 +1200,7 @@ pl_status_t pl_execute(pl_schedule_t s, const pl_bufs_t* bufs, void* stream) {
     F.status = s->comm->d_status;
     F.timeout_ns = s->timeout_ns;
     F.run = s->flat_run;
+    F.release = s->flat_launch.release;
     if (launch_flat(s->comm->dtype, F, s->flat_launch, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
       cudaGetLastError();
       return PL_ERR_CUDA;

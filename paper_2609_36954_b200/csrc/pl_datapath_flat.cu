@@ -117,12 +117,7 @@ __device__ __forceinline__ void store_sum(const FlatParams& P, const Acc<DT>& ac
 }
 
 // ---- register form ---------------------------------------------------------------------------
-// Sums, and copies to every rank, do not release the launch behind them: it is set up as their CTAs exit.  Released at
-// the start, its CTAs take the room that is left and then share SMs while others idle, as soon as the host enqueues
-// faster than the GPU finishes (all-reduce, us, released at the start / after the loads / not: 8 x 1 MiB 4.85 / 3.73 / 3.02,
-// 2 x 4 MiB 4.45 / 3.78 / 2.90, 8 x 2 MiB 6.4 / 6.0 / 5.2, 16 x 256 KiB 4.66 / 3.39 / 3.20, 16 x 1 MiB 6.8 / 6.6 / 6.1, 8 x 64 KiB 2.94 / 2.98 / 2.95;
-// reduce-scatter + all-gather 8 x 2 MiB, the all-gather released / not, 8.7 / 8.3).  Copies to one rank read their span from
-// memory first and do (all-to-all-v 8 x 2 MiB 5.0 / 5.4), and so do the bulk-copy forms (no difference, or 1 % slower without).
+// Which launches release the one behind them at their start is flat_release()'s.
 // Units per thread of a reduce: about 8 operand vectors in flight (16 with a second operand per rank).
 template <int NR, bool HOOK>
 struct FlatUnits {
@@ -139,6 +134,7 @@ struct FlatUnits {
 template <int DT, int NR, bool HOOK, bool ALL, bool EXACT>
 __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const __grid_constant__ FlatParams P) {
   constexpr int U = FlatUnits<NR, HOOK>::value;
+  if (P.release) pdl_launch_dependents();
   const Tile t = my_tile(P);
   const uint32_t R = EXACT ? (uint32_t)NR : (uint32_t)P.n_ranks, to = dst_rank(t.span);
   const bool residual = HOOK && (P.hook & PL_HOOK_RESIDUAL);
@@ -218,7 +214,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
 
 template <int U, bool ALL>
 __global__ void __launch_bounds__(kFlatThreads) pl_flat_copy_kernel(const __grid_constant__ FlatParams P) {
-  if (!ALL) pdl_launch_dependents();
+  if (P.release) pdl_launch_dependents();
   const Tile t = my_tile(P);
   const uint64_t policy = (P.hints & 1u) ? ptx::policy_evict_first() : 0ull;
   pdl_wait();
@@ -433,6 +429,21 @@ FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, u
     F.tile = (uint32_t)(F.units * kFlatThreads);
   }
   return F;
+}
+
+// Else the launch behind is set up as the CTAs exit.  Released at the start its CTAs take the room that is left, and in a
+// grid of middle size they then share SMs while others idle, once launches are enqueued faster than the GPU finishes
+// them.  us, released / not, back to back in a CUDA graph: sums to every rank 8 x 16 KiB (4 CTAs) 1.95 / 2.03, 2 x 128 KiB (8)
+// 1.79 / 1.85, 8 x 64 KiB (16) 2.09 / 2.02, 8 x 128 KiB (32) 2.31 / 2.05, 4 x 512 KiB (64) 2.52 / 1.90, 8 x 512 KiB (128) 3.56 / 2.15; launched one
+// by one 8 x 1 MiB (256) 4.85 / 3.02, 8 x 2 MiB (512) 6.4 / 5.2, 8 x 8 MiB (2048) 21.9 / 22.0.  Sums to one rank (one-shot) 4 x 16 KiB
+// (8) 1.38 / 1.61, 4 x 128 KiB (64) 1.48 / 1.63, 8 x 64 KiB (128) 1.94 / 1.81, 4 x 512 KiB (256) 2.30 / 2.02, 4 x 1 MiB (512) 2.35 / 2.75, 8 x 1
+// MiB (2048) 6.26 / 6.45.  Copies to every rank 8 x 4 KiB (8) 0.91 / 1.30, 4 x 128 KiB (32) 1.19 / 1.40, 8 x 256 KiB (64) 1.83 / 1.70, 8 x
+// 512 KiB (128) 3.53 / 1.73.  Copies to one rank read their span from memory first (all-to-all-v 8 x 2 MiB 5.0 / 5.4), the bulk-copy
+// forms are the same or 1 % slower without: they always release.
+bool flat_release(bool reduce, bool all, bool bulk, uint64_t blocks) {
+  if (bulk || (!reduce && !all)) return true;
+  if (all) return blocks <= (reduce ? 8 : 32);
+  return blocks <= 64 || blocks >= 512;
 }
 
 cudaError_t launch_flat(int dtype, const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {

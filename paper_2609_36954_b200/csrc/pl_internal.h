@@ -149,12 +149,13 @@ struct FlatParams {
   int* status;
   unsigned long long timeout_ns;
   FlatRun run;             // the spans, if `spans` is null
-  uint64_t pad;
+  uint32_t release, pad;   // register sums and copies: release the launch behind at the start
 };
 static_assert(cheap_params(sizeof(FlatParams)), "launch cost");
 struct FlatLaunch {  // host side: which kernel, how many CTAs
   bool reduce, all, bulk;  // all: every rank is a destination
   int units = 1;           // units per thread of a register copy
+  bool release = true;
   uint32_t tile, blocks = 0, smem_bytes;
   int threads;
 };
