@@ -154,3 +154,14 @@ def test_results_that_fit_l2_stay_there():
         for s in scheds:
             B.pl_schedule_destroy(s)
         B.pl_comm_destroy(comm)
+
+
+# sums with a second operand have a kernel for a fixed number of ranks: around the ends of warps and tiles, one unit
+@pytest.mark.parametrize("R", [2, 3, 4, 5, 6, 8, 12, 16])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("units", [1, 31, 255, 513])
+def test_residual_by_number_of_ranks(R, dtype, units):
+    n = 16 * units // SIZE[dtype] * R
+    for coll, algo in ((B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED), (B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT)):
+        for flags in (0, B.PL_OPT_INPUTS_LAST_USE):
+            same_bits(R, dtype, lambda c, o: B.pl_schedule_build(c, coll, algo, n, 64 * 1024, o), "tiles", hook=B.PL_HOOK_RESIDUAL, out_scale=0.375, flags=flags)

@@ -129,3 +129,25 @@ def test_layers_of_many_ranks_that_stream_run_on_the_register_executor():
         assert all(torch.equal(t.view(torch.bfloat16), want) for t in y)
     finally:
         ses.close()
+
+
+# kernels for a fixed number of ranks, and the one for any other: slices that do not fill a warp, end inside one, and take
+# several turns of a thread, as one cluster and with flags, against the register executor (a grid asked for): the same bits
+@pytest.mark.parametrize("R", [2, 3, 4, 5, 6, 7, 8, 9, 12, 16])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("units", [1, 33, 149, 2055])
+def test_layers_by_number_of_ranks(R, dtype, units):
+    layers, es = 3, {"bf16": 2, "f32": 4}[dtype]
+    n = 16 * units * R // es
+    ses = Session(R, dtype)
+    try:
+        x = [torch.randn(n * layers, device="cuda", generator=torch.Generator("cuda").manual_seed(r)).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+             for r in range(R)]
+        outs = []
+        for kw in ({}, {"n_ctas": R}):
+            s = ses.build_layers(B.PL_ALGO_DIRECT_FUSED, n, layers, **kw)
+            outs.append(ses.execute(s, None, repeats=2, d_ins=x)[0])
+        for a, b in zip(*outs):
+            assert np.array_equal(a, b)
+    finally:
+        ses.close()
