@@ -417,7 +417,7 @@ def measure_step_variant(B, torch, comm, n, chunk, R, b_rs, b_ag, stream, plain_
 
 
 def measure_all_configs(peak):
-    """C1, C3 (three sizes x five algorithms), C4 (both routings), C5 (three sizes, both latency
+    """C1, C3 (three sizes x five algorithms, the ring with its hops and folded), C4 (both routings), C5 (three sizes, both latency
     protocols) and the stream ceilings of the bulk-copy ring, each timed with CUDA events in this
     process.  Every entry carries its algorithmic bytes (pl_schedule_info), the fraction of the
     measured copy peak and of 8 TB/s, and the fraction of the matching stream ceiling."""
@@ -440,7 +440,7 @@ def measure_all_configs(peak):
         comp = rec["compulsory_bytes"]
         us = rec["us"] * max(1, rec["layers"])
         gbs = comp / us / 1e3
-        c = which_ceiling(comp - rec["bytes_written"], rec["bytes_written"])
+        c = which_ceiling(comp - rec["moved_written"], rec["moved_written"])
         e = {"us": round(rec["us"], 3), "us_p10": round(rec["us_p10"], 3), "us_p90": round(rec["us_p90"], 3),
              "message_bytes": rec["message_bytes"], "algorithmic_bytes": alg, "hbm_bytes": comp,
              "algbw_gbs": round(rec["eff_gbs"], 1), "hbm_gbs": round(gbs, 1),
@@ -454,14 +454,14 @@ def measure_all_configs(peak):
         return e
 
     l2 = "working set sits in L2: the HBM fractions do not apply"
-    # C1: all-reduce, R = 4, 1 MiB per rank, ring, 64 KiB chunks
-    out["C1"] = {name: entry(b.collective("C1", 4, dt, B.PL_ALLREDUCE, "ring", 262144, 65536, iters=50, graph=True), l2)
-                 for name, dt in (("f32", B.PL_F32), ("i32", B.PL_I32))}
+    # C1: all-reduce, R = 4, 1 MiB per rank, ring, 64 KiB chunks: with its hops, and folded as the library runs it if left alone
+    out["C1"] = {name + suffix: entry(b.collective("C1", 4, dt, B.PL_ALLREDUCE, "ring" + suffix, 262144, 65536, iters=50, graph=True), l2)
+                 for name, dt in (("f32", B.PL_F32), ("i32", B.PL_I32)) for suffix in ("", "_folded")}
     # C3: all-reduce sweep points
     out["C3"] = {}
     for label, size, graph, iters in (("64KiB", 64 << 10, True, 30), ("16MiB", 16 << 20, False, 20), ("256MiB", 256 << 20, False, 8)):
         out["C3"][label] = {}
-        for algo in ("ring", "tree", "oneshot", "direct", "fused"):
+        for algo in ("ring", "ring_folded", "tree", "oneshot", "direct", "fused"):
             chunk = max(16, min(MIB, size if (algo == "oneshot" or (algo == "tree" and size <= (128 << 10))) else size // 8))
             rec = b.collective("C3", 8, B.PL_BF16, B.PL_ALLREDUCE, algo, size // 2, chunk, iters=iters, graph=graph)
             out["C3"][label][algo] = entry(rec, l2 if size < (32 << 20) else None)
@@ -470,6 +470,7 @@ def measure_all_configs(peak):
         "reduce_scatter": entry(b.collective("C2-RS", 8, B.PL_BF16, B.PL_REDUCE_SCATTER, "direct", 32 * MIB, MIB)),
         "all_gather": entry(b.collective("C2-AG", 8, B.PL_BF16, B.PL_ALLGATHER, "direct", 4 * MIB, MIB)),
         "reduce_scatter_ring": entry(b.collective("C2-RS", 8, B.PL_BF16, B.PL_REDUCE_SCATTER, "ring", 32 * MIB, 256 << 10)),
+        "reduce_scatter_ring_folded": entry(b.collective("C2-RS", 8, B.PL_BF16, B.PL_REDUCE_SCATTER, "ring_folded", 32 * MIB, 256 << 10)),
         "all_gather_ring": entry(b.collective("C2-AG", 8, B.PL_BF16, B.PL_ALLGATHER, "ring", 4 * MIB, 256 << 10)),
         "all_to_all": entry(b.collective("A2A", 8, B.PL_BF16, B.PL_ALLTOALL, "direct", 32 * MIB, MIB)),
     }

@@ -19,7 +19,9 @@ from paper_2609_36954_b200 import binding as B
 from paper_2609_36954_b200 import inputs as gen
 
 MIB = 1 << 20
-ALGO = {"ring": B.PL_ALGO_RING, "tree": B.PL_ALGO_TREE, "direct": B.PL_ALGO_DIRECT,
+# "ring" keeps its hops (PL_OPT_RING_HOPS); "ring_folded" is a reducing ring as the library runs it when left alone:
+# one chain of additions per element, in ring order.
+ALGO = {"ring": B.PL_ALGO_RING, "ring_folded": B.PL_ALGO_RING, "tree": B.PL_ALGO_TREE, "direct": B.PL_ALGO_DIRECT,
         "oneshot": B.PL_ALGO_ONESHOT, "fused": B.PL_ALGO_DIRECT_FUSED}
 
 
@@ -29,6 +31,15 @@ def _peak():
         return float(json.load(open(os.path.join(root, "MEASURED_PEAKS.json")))["hbm_gbs"])
     except Exception:
         return 6650.0
+
+
+def moved_bytes(info, algo, R):
+    """(read, written) by one execute: the op list's bytes, but of a ring whose partial sums stay on the SMs
+    (folded, or with its hops in shared memory) the inputs and outputs alone."""
+    ins, outs = sum(int(info.in_bytes[r]) for r in range(R)), sum(int(info.out_bytes[r]) for r in range(R))
+    if ALGO[algo] == B.PL_ALGO_RING and int(info.hbm_bytes) == ins + outs:
+        return ins, outs
+    return int(info.bytes_read), int(info.bytes_written)
 
 
 def _fill(nbytes, stream_id):
@@ -109,6 +120,8 @@ class Bench:
         comm = B.pl_comm_create(R, dtype)
         okw = dict(self.opts_kw)
         okw.update(kw)
+        if algo == "ring":
+            okw["flags"] = okw.get("flags", 0) | B.PL_OPT_RING_HOPS
         opts = B.make_opts(**okw)
         try:
             if root is not None:
@@ -147,10 +160,12 @@ class Bench:
             in_kernel = {"p50_us": float(np.median(gaps)), "p10_us": float(np.percentile(gaps, 10)),
                          "p90_us": float(np.percentile(gaps, 90))}
         nl = max(1, layers)
-        sched_bytes = info.bytes_read + info.bytes_written
+        read, written = moved_bytes(info, algo, R)
+        sched_bytes = read + written
         # bytes that must cross the HBM interface when nothing is cached between launches
         # (pl_sched_info_t.hbm_bytes: input bytes once however often they are read, everything else as scheduled)
         rec = {"cfg": cfg, "bytes_read": int(info.bytes_read), "bytes_written": int(info.bytes_written),
+               "moved_read": read, "moved_written": written,
                "compulsory_bytes": int(info.hbm_bytes), "coll": int(coll), "algo": algo, "R": R, "dtype": int(dtype),
                "message_bytes": int(info.message_bytes), "chunk": int(min(chunk, 1 << 40)), "layers": layers,
                "us": p50 / nl, "us_p10": p10 / nl, "us_p90": p90 / nl, "us_graph128": graph_us, "layer_us_in_kernel": in_kernel,
@@ -274,13 +289,15 @@ def main(args=None):
         probe(b)
     if "c1" in which:
         for dt in (B.PL_F32, B.PL_I32):
-            b.collective("C1", 4, dt, B.PL_ALLREDUCE, "ring", 262144, 65536, iters=50, graph=True)
+            for algo in ("ring", "ring_folded"):
+                b.collective("C1", 4, dt, B.PL_ALLREDUCE, algo, 262144, 65536, iters=50, graph=True)
     if "c2" in which:
         n = 32 * MIB  # 64 MiB bf16 per rank
         for algo in ("direct", "ring"):
             for chunk in (256 * 1024, MIB):
                 b.collective("C2-RS", 8, B.PL_BF16, B.PL_REDUCE_SCATTER, algo, n, chunk)
                 b.collective("C2-AG", 8, B.PL_BF16, B.PL_ALLGATHER, algo, n // 8, chunk)
+        b.collective("C2-RS", 8, B.PL_BF16, B.PL_REDUCE_SCATTER, "ring_folded", n, MIB)
     if "c2big" in which:
         # the same two collectives at 256 MiB per rank: the sustained rate, launch edges amortised
         n = 128 * MIB
@@ -354,7 +371,7 @@ def main(args=None):
     if "c3" in which:
         for lg in range(12, 29):
             size = 1 << lg
-            for algo in ("ring", "tree", "oneshot", "direct", "fused"):
+            for algo in ("ring", "ring_folded", "tree", "oneshot", "direct", "fused"):
                 if algo == "oneshot" and size > 64 * MIB:
                     continue
                 # chunks of a partition (size / 8) for the partitioned algorithms and for trees above

@@ -48,3 +48,27 @@ def test_the_printed_line_is_short(tmp_path, capsys):
     short, full = json.loads(out), json.loads((tmp_path / "detail.json").read_text())
     assert full == line and "detail" not in short and "all" not in short["small_allreduce"]
     assert set(line) - set(short) == {"detail"} and abs(short["value"] / line["value"] - 1) < 1e-5
+
+
+def test_a_ring_whose_partial_sums_stay_on_the_sms_moves_inputs_and_outputs():
+    """The op list of a ring counts every hop: bytes that a folded ring, or one with its hops in shared memory, never moves."""
+    import types
+
+    import bench_suite as S
+    from paper_2609_36954_b200 import binding as B
+    R, n, es = 8, 1 << 20, 2
+    comm = B.pl_comm_create_planner(R, B.PL_BF16)  # on the op queues: hops through memory
+    s = B.pl_schedule_build(comm, B.PL_REDUCE_SCATTER, B.PL_ALGO_RING, n, 65536, None)
+    try:
+        info = B.pl_schedule_info(s)
+        ins, outs = R * n * es, n * es
+        assert info.bytes_written > 4 * outs
+        for algo in ("ring", "ring_folded"):
+            assert S.moved_bytes(info, algo, R) == (info.bytes_read, info.bytes_written)
+            # what a GPU communicator reports for the same schedule
+            on_sms = types.SimpleNamespace(bytes_read=info.bytes_read, bytes_written=info.bytes_written, hbm_bytes=ins + outs,
+                                           in_bytes=info.in_bytes, out_bytes=info.out_bytes)
+            assert S.moved_bytes(on_sms, algo, R) == (ins, outs)
+    finally:
+        B.pl_schedule_destroy(s)
+        B.pl_comm_destroy(comm)
