@@ -12,19 +12,25 @@ pytestmark = pytest.mark.gpu
 R, LAYERS = 4, 2
 
 
+def in_clusters(info):
+    """A ring that hops through shared memory: the tile's slots of a CTA per rank and nothing else (tiles have none, or a barrier beside them)."""
+    return info.smem_bytes > 0 and info.smem_bytes % info.stage_bytes == 0 and info.grid % R == 0
+
+
 class Chain:
-    """x -> fused all-reduce (tiles) -> ring (clusters) -> two layers (`n` decides: one cluster, or flags) -> reduce-scatter
+    """x -> fused all-reduce (tiles) -> ring (clusters and, every second turn, folded) -> two layers (`n` decides: one cluster, or flags) -> reduce-scatter
     (tiles) -> all-gather (tiles); with the sum S of the inputs the result is R^3 S on every rank."""
 
     def __init__(self, n, turns):
         self.ses, self.n = Session(R, "i32"), n
         a = self.ses.build(B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n, 1 << 20)
-        b = self.ses.build(B.PL_ALLREDUCE, B.PL_ALGO_RING, n, 65536)
+        b = [self.ses.build(B.PL_ALLREDUCE, B.PL_ALGO_RING, n, 65536, flags=f) for f in (B.PL_OPT_RING_HOPS, 0)]
         c = self.ses.build_layers(B.PL_ALGO_AUTO, n // LAYERS, LAYERS)
         d = self.ses.build(B.PL_REDUCE_SCATTER, B.PL_ALGO_DIRECT, n, 1 << 20)
         e = self.ses.build(B.PL_ALLGATHER, B.PL_ALGO_DIRECT, n // R, 1 << 20)
-        for s in (a, b, d, e):
+        for s in (a, *b, d, e):
             assert B.pl_schedule_info(s).stages == 1  # not on the queues
+        assert [in_clusters(B.pl_schedule_info(s)) for s in b] == [True, False]
         rng = np.random.default_rng(n)
         x = [rng.integers(-2 ** 31, 2 ** 31, (turns, n)).astype(np.int32) for _ in range(R)]
         with np.errstate(over="ignore"):
@@ -39,7 +45,7 @@ class Chain:
             info = B.pl_schedule_info(s)
             return s, B.make_bufs([t.data_ptr() for t in i], [t.data_ptr() for t in o], list(info.in_bytes)[:R], list(info.out_bytes)[:R])
 
-        self.calls = [[bufs(a, dx[t], y), bufs(b, y, z), bufs(c, z, w), bufs(d, w, u), bufs(e, u, self.out[t])] for t in range(turns)]
+        self.calls = [[bufs(a, dx[t], y), bufs(b[t % 2], y, z), bufs(c, z, w), bufs(d, w, u), bufs(e, u, self.out[t])] for t in range(turns)]
 
     def run(self):
         for turn in self.calls:
@@ -95,8 +101,9 @@ def test_executors_whose_launches_wait_for_nobody_run_beside_one_another():
     n = 1 << 20
     ses = Session(R, "i32")
     try:
-        scheds = [ses.build(B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n, 1 << 20), ses.build(B.PL_ALLREDUCE, B.PL_ALGO_RING, n, 65536),
-                  ses.build_layers(B.PL_ALGO_AUTO, 1024, 8)]
+        scheds = [ses.build(B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n, 1 << 20),
+                  ses.build(B.PL_ALLREDUCE, B.PL_ALGO_RING, n, 65536, flags=B.PL_OPT_RING_HOPS), ses.build_layers(B.PL_ALGO_AUTO, 1024, 8)]
+        assert in_clusters(B.pl_schedule_info(scheds[1]))
         assert B.pl_schedule_info(scheds[0]).grid + B.pl_schedule_info(scheds[1]).grid > 1000 and B.pl_schedule_info(scheds[2]).grid <= 16
         jobs = []
         for s in scheds:

@@ -43,12 +43,22 @@ def test_gathering_rings(R, dtype, units):
     same_bits(R, dtype, build(B.PL_ALLGATHER, 16 * units // SIZE[dtype]), "tiles" if R == 2 or (units <= 65536 and units * R <= 8 * 65536) else "queues")
 
 
-def test_broken_wait_times_out():
+def in_clusters(info):
+    """Hops through shared memory: a CTA per rank with the tile's slots and nothing else (tiles have none, or a barrier beside them)."""
+    return info.smem_bytes > 0 and info.smem_bytes % info.stage_bytes == 0
+
+
+FORMS = pytest.mark.parametrize("flags", [0, B.PL_OPT_RING_HOPS], ids=["folded", "clusters"])
+
+
+@FORMS
+def test_broken_wait_times_out(flags):
     """The fault hook moves the schedule to the op queues, whose waits it edits."""
     R, n = 4, 4096
     comm = B.pl_comm_create(R, DT["f32"])
-    s = build(B.PL_ALLREDUCE, n)(comm, B.make_opts(timeout_ns=20_000_000))
+    s = build(B.PL_ALLREDUCE, n)(comm, B.make_opts(timeout_ns=20_000_000, flags=flags))
     try:
+        assert in_clusters(B.pl_schedule_info(s)) == bool(flags)
         t = [torch.ones(n, device="cuda") for _ in range(2 * R)]
         size = [4 * n] * R
         bufs = B.make_bufs([x.data_ptr() for x in t[:R]], [x.data_ptr() for x in t[R:]], size, size)
@@ -65,14 +75,17 @@ def test_broken_wait_times_out():
         B.pl_comm_destroy(comm)
 
 
-def test_a_ring_in_clusters_uploads_no_op_list():
+@FORMS
+def test_a_ring_without_queues_uploads_no_op_list(flags):
     R, n = 16, 32 * 1024 * 1024  # 64 MiB of bf16 per rank in chunks of 64 KiB: 30,720 ops
     comm = B.pl_comm_create(R, DT["bf16"])
-    scheds = [build(B.PL_ALLREDUCE, n)(comm, None)]
+    opts = B.make_opts(flags=flags)
+    scheds = [build(B.PL_ALLREDUCE, n)(comm, opts)]
     try:
         torch.cuda.synchronize()
         free = torch.cuda.mem_get_info()[0]
-        scheds += [build(B.PL_ALLREDUCE, n)(comm, None) for _ in range(6)]
+        scheds += [build(B.PL_ALLREDUCE, n)(comm, opts) for _ in range(6)]
+        assert all(in_clusters(B.pl_schedule_info(s)) == bool(flags) for s in scheds)
         assert len(B.pl_schedule_dump(scheds[0])) >= 30720 and B.pl_schedule_info(scheds[0]).scratch_bytes == 0
         assert free - torch.cuda.mem_get_info()[0] < 4 << 20  # an op list takes 3 MiB
     finally:
