@@ -550,7 +550,7 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
     if (reduce && !(flags & PL_OPT_RING_HOPS)) {
       ring_plan(comm->R, rq.coll == PL_ALLREDUCE, part, &S->flat_spans);
       lay_flat(true, rq.coll == PL_ALLREDUCE);
-      S->folded = S->flat;
+      S->folded = S->flat_launch.folded = S->flat;
     }
     S->ring = !S->folded && ring_shape(comm->R, comm->dtype, reduce, rq.coll != PL_REDUCE_SCATTER, part, rq.chunk_bytes, comm->sm_count, &S->ring_launch) &&
               ring_prepare(comm->dtype, comm->R, S->ring_launch) > 0;

@@ -131,7 +131,10 @@ struct FlatUnits {
 // bf16, us: 4 x 4 MiB 9.5 -> 8.9, 8 x 1.6 MiB 9.3 -> 9.0, 8 x 4 MiB 18.1 -> 17.2, 16 x 4 MiB 33.6 -> 31.9; fp32 8 x 2 MiB 11.1 -> 10.2);
 // without one the bursts are slower where inputs and outputs take 20 to 40 MB of L2 (8 x 2 MiB 6.4 / 8.2, 16 x 1 MiB
 // 6.9 / 8.3, while 16 x 2 MiB 13.0 / 12.2), so it goes with HOOK.
-template <int DT, int NR, bool HOOK, bool ALL, bool EXACT>
+// FOLDED: the sum starts with a rank that the span names, so the pointer of every load is looked up at run time.  Where it is not,
+// the pointers are constants (looked up in every sum: one-shot 6 x 8 MiB bf16 33.8 -> 35.8 us, fp32 43.7 -> 46.5, reduce-scatter 2 x 8 MiB
+// with residual 5.0 -> 5.9).
+template <int DT, int NR, bool HOOK, bool ALL, bool EXACT, bool FOLDED>
 __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const __grid_constant__ FlatParams P) {
   constexpr int U = FlatUnits<NR, HOOK>::value;
   if (P.release) pdl_launch_dependents();
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
     in_off[j] = (t.span.src_off + t.first + u) * 16ull;
   }
   uint4 q[U][NR];
-  const uint32_t first = first_rank(t.span);
+  const uint32_t first = FOLDED ? first_rank(t.span) : 0u;
   // one test of the hint for all loads (in front of each: 16 x 2 MiB 15.1 us, so 13.0; 8 x 2 MiB 7.4 / 6.4)
   auto load = [&](auto ld) {
 #pragma unroll
@@ -160,7 +163,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
 #pragma unroll
       for (int s = 0; s < NR; ++s)
         if (EXACT || (live[j] && s < (int)R)) {
-          const uint32_t rank = first + s < R ? first + s : first + s - R;
+          const uint32_t rank = !FOLDED ? (uint32_t)s : first + s < R ? first + s : first + s - R;
           q[j][s] = ld(static_cast<const char*>(P.in[rank]) + in_off[j]);
         }
   };
@@ -376,9 +379,10 @@ cudaError_t launch(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream
   return cudaLaunchKernelEx(&cfg, kernel, P);
 }
 
-template <int DT, int NR, bool HOOK, bool EXACT>
+template <int DT, int NR, bool HOOK, bool EXACT, bool FOLDED = false>
 cudaError_t launch_all(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
-  return F.all ? launch<pl_flat_reduce_kernel<DT, NR, HOOK, true, EXACT>>(P, F, stream) : launch<pl_flat_reduce_kernel<DT, NR, HOOK, false, EXACT>>(P, F, stream);
+  return F.all ? launch<pl_flat_reduce_kernel<DT, NR, HOOK, true, EXACT, FOLDED>>(P, F, stream)
+               : launch<pl_flat_reduce_kernel<DT, NR, HOOK, false, EXACT, FOLDED>>(P, F, stream);
 }
 template <int DT, int NR, bool HOOK>
 cudaError_t launch_reduce(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
@@ -386,6 +390,9 @@ cudaError_t launch_reduce(const FlatParams& P, const FlatLaunch& F, cudaStream_t
     if (P.n_ranks == NR) return launch_all<DT, NR, true, true>(P, F, stream);
     if (P.n_ranks == 3) return launch_all<DT, 3, true, true>(P, F, stream);
     if (P.n_ranks == 6) return launch_all<DT, 6, true, true>(P, F, stream);
+  }
+  if constexpr (!HOOK) {
+    if (F.folded) return launch_all<DT, NR, false, false, true>(P, F, stream);
   }
   return launch_all<DT, NR, HOOK, false>(P, F, stream);
 }

@@ -154,6 +154,7 @@ struct FlatParams {
 static_assert(cheap_params(sizeof(FlatParams)), "launch cost");
 struct FlatLaunch {  // host side: which kernel, how many CTAs
   bool reduce, all, bulk;  // all: every rank is a destination
+  bool folded = false;     // spans start with a rank of their own
   int units = 1;           // units per thread of a register copy
   bool release = true;
   uint32_t tile, blocks = 0, smem_bytes;
