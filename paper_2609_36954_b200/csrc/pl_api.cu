@@ -536,7 +536,6 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
     S->flat_launch.blocks = (uint32_t)blocks;
     S->flat_launch.release = flat_release(reduce, all, S->flat_launch.bulk, blocks);
     S->flat_is_run = units > 0 && flat_run(S->flat_spans, &S->flat_run);
-    if (S->flat_is_run) S->flat_run.blocks = (uint32_t)(blocks / S->flat_spans.size());
     S->flat = units > 0 && blocks <= 0x7FFFFFFFull;
     if (S->flat) S->pol.idle_count = 0;
   };

@@ -49,26 +49,26 @@ struct Tile {
   uint32_t units;
 };
 
-// The tile of this CTA.  A run is worked out from the parameters: no load stands in front of a tile's own
-// (8 x 1 MiB all-reduce 5.05 -> 4.82 us, 2 x 8 MiB reduce-scatter + all-gather 9.88 -> 9.50, 8 x 16 MiB the same), and nothing is
-// uploaded.
+// The tile of this CTA.  A run is worked out from the parameters: nothing is uploaded, and no load stands in front of a
+// tile's own.  The span is the second dimension of the grid (dealt in the same order; found by a division it cost more than the
+// load: one-shot 6 x 2 MiB bf16 7.73 us, 8.06 by division, 8.53 from memory; reduce-scatter 8 x 1 MiB 1.74, 1.88, 2.01).
 // Else every warp finds the span whose blocks contain it (lane i looks at spans i, i + 32, ...); spans are written
 // when the schedule is built, so this may run ahead of the wait for the launch in front.
 __device__ __forceinline__ Tile my_tile(const FlatParams& P) {
   const uint32_t b = blockIdx.x, lane = threadIdx.x & 31u;
-  uint32_t k = 0;
   if (!P.spans) {
+    const uint32_t k = blockIdx.y;
     Tile t;
-    if (P.n_spans > 1) k = b / P.run.blocks;
     t.span.src_off = k * P.run.src_step;
     t.span.dst_off = k * P.run.dst_step;
     t.span.units = P.run.units;
-    t.span.first_block = k * P.run.blocks;
+    t.span.first_block = 0;
     t.span.ranks = P.run.ranks + k * P.run.rank_step;
-    t.first = (uint64_t)(b - t.span.first_block) * P.tile;
+    t.first = (uint64_t)b * P.tile;
     t.units = (uint32_t)min((uint64_t)P.tile, t.span.units - t.first);
     return t;
   }
+  uint32_t k = 0;
   if (P.n_spans > 1) {
     uint32_t below = 0;  // spans that start at or before this block
     for (uint32_t i = 0; i < P.n_spans; i += 32)
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(32) pl_flat_bulk_copy_kernel(const __grid_cons
 template <void (*kernel)(const FlatParams)>
 cudaError_t launch(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(F.blocks);
+  cfg.gridDim = P.spans ? dim3(F.blocks) : dim3(F.blocks / P.n_spans, P.n_spans);
   cfg.blockDim = dim3((unsigned)F.threads);
   cfg.dynamicSmemBytes = F.smem_bytes;
   cfg.stream = stream;

@@ -134,8 +134,7 @@ static_assert(sizeof(FlatSpan) == 32, "FlatSpan layout");
 // the inputs and outputs, and its `ranks` are k rank steps on from the first one's.
 struct FlatRun {
   uint64_t units, src_step, dst_step;
-  uint32_t blocks;  // CTAs of a span
-  uint32_t ranks, rank_step, pad;
+  uint32_t ranks, rank_step;
 };
 struct FlatParams {
   const void* in[PL_MAX_RANKS];
@@ -149,7 +148,8 @@ struct FlatParams {
   int* status;
   unsigned long long timeout_ns;
   FlatRun run;             // the spans, if `spans` is null
-  uint32_t release, pad;   // register sums and copies: release the launch behind at the start
+  uint32_t release;        // register sums and copies: release the launch behind at the start
+  uint32_t pad[3];
 };
 static_assert(cheap_params(sizeof(FlatParams)), "launch cost");
 struct FlatLaunch {  // host side: which kernel, how many CTAs
@@ -272,7 +272,7 @@ pl_status_t validate(const Lowered& L, int R, std::string* err, bool bulk_datapa
 // The ops of a schedule without flags as spans; false if they are not of the forms a span describes.
 // `reduce` / `all` receive the one kind of op the schedule holds.  first_block is left to the caller.
 bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans, bool* reduce, bool* all);
-// True if the spans are a run; `blocks` of it is left to the caller.
+// True if the spans are a run.
 bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run);
 // flat_plan() for a reducing ring (a partition's chain of hops is one sum per unit); empty without units.
 void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* spans);

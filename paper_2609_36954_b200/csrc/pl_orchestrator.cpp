@@ -1324,7 +1324,7 @@ void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* s
 bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run) {
   const FlatSpan& a = spans[0];
   const FlatSpan& b = spans.size() > 1 ? spans[1] : a;
-  *run = FlatRun{a.units, b.src_off, b.dst_off, 0, a.ranks, b.ranks - a.ranks, 0};
+  *run = FlatRun{a.units, b.src_off, b.dst_off, a.ranks, b.ranks - a.ranks};
   if (spans.size() == 1) run->src_step = run->dst_step = 0;
   for (size_t k = 0; k < spans.size(); ++k) {
     const FlatSpan& f = spans[k];
