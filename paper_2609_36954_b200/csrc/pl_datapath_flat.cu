@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "pl_device.cuh"
 #include "pl_internal.h"
@@ -130,11 +131,16 @@ struct FlatUnits {
 // tile is then loaded from its last one and not stored.  With a processing phase that is faster at every size (residual,
 // bf16, us: 4 x 4 MiB 9.5 -> 8.9, 8 x 1.6 MiB 9.3 -> 9.0, 8 x 4 MiB 18.1 -> 17.2, 16 x 4 MiB 33.6 -> 31.9; fp32 8 x 2 MiB 11.1 -> 10.2);
 // without one the bursts are slower where inputs and outputs take 20 to 40 MB of L2 (8 x 2 MiB 6.4 / 8.2, 16 x 1 MiB
-// 6.9 / 8.3, while 16 x 2 MiB 13.0 / 12.2), so it goes with HOOK.
+// 6.9 / 8.3, while 16 x 2 MiB 13.0 / 12.2; measured with the launch behind released early), so it goes with HOOK.
 // FOLDED: the sum starts with a rank that the span names, so the pointer of every load is looked up at run time.  Where it is not,
 // the pointers are constants (looked up in every sum: one-shot 6 x 8 MiB bf16 33.8 -> 35.8 us, fp32 43.7 -> 46.5, reduce-scatter 2 x 8 MiB
 // with residual 5.0 -> 5.9).
-template <int DT, int NR, bool HOOK, bool ALL, bool EXACT, bool FOLDED>
+// HINT: the loads carry the evict-first hint.  Known when compiled, but for sums of more than 8 ranks to one rank, which test for it in
+// front of every load: that keeps the loads of up to 16 sources in front of the first addition (us, so / as an argument /
+// one test for all loads: one-shot 12 x 2 MiB int32 24.0 / 30.8 / 34.2, 16 x 2 MiB bf16 49.2 / 51.3 / 52.9, reduce-scatter 12 x 1 MiB bf16 2.01 / 2.36
+// / 2.50, though 16 x 4 MiB 13.8 / 13.0 / 12.9; up to 8 ranks: one-shot 8 x 2 MiB bf16 12.1 / 11.6 / 12.0, reduce-scatter 8 x 4 MiB
+// fp32 8.3 / 7.1 / 7.1, and to every rank 16 x 2 MiB 15.1 / 13.4 / 13.3, 12 x 4 KiB 2.35 / 2.51 / 2.60).
+template <int DT, int NR, bool HOOK, bool ALL, bool EXACT, bool FOLDED, bool HINT>
 __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const __grid_constant__ FlatParams P) {
   constexpr int U = FlatUnits<NR, HOOK>::value;
   if (P.release) pdl_launch_dependents();
@@ -142,7 +148,9 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
   const uint32_t R = EXACT ? (uint32_t)NR : (uint32_t)P.n_ranks, to = dst_rank(t.span);
   const bool residual = HOOK && (P.hook & PL_HOOK_RESIDUAL);
   const uint32_t out_b = (HOOK && DT == PL_BF16 && (P.hook & PL_HOOK_F32_OUT)) ? 32u : 16u;
-  const uint64_t policy = (P.hints & 1u) ? ptx::policy_evict_first() : 0ull;
+  constexpr bool kTested = NR > 8 && !ALL && !EXACT;
+  const bool hint = kTested ? (P.hints & 1u) != 0 : HINT;
+  const uint64_t policy = hint ? ptx::policy_evict_first() : 0ull;
   pdl_wait();
   uint64_t in_off[U], at[U];  // byte offset of the unit in every source, unit index in the destination
   bool live[U];
@@ -156,7 +164,6 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
   }
   uint4 q[U][NR];
   const uint32_t first = FOLDED ? first_rank(t.span) : 0u;
-  // one test of the hint for all loads (in front of each: 16 x 2 MiB 15.1 us, so 13.0; 8 x 2 MiB 7.4 / 6.4)
   auto load = [&](auto ld) {
 #pragma unroll
     for (int j = 0; j < U; ++j)
@@ -167,7 +174,8 @@ __global__ void __launch_bounds__(kFlatThreads, 2) pl_flat_reduce_kernel(const _
           q[j][s] = ld(static_cast<const char*>(P.in[rank]) + in_off[j]);
         }
   };
-  if (P.hints & 1u) load([&](const char* src) { return ld16_hint(src, policy); });
+  if constexpr (kTested) load([&](const char* src) { return hint ? ld16_hint(src, policy) : ld16(src); });
+  else if (hint) load([&](const char* src) { return ld16_hint(src, policy); });
   else load([](const char* src) { return ld16(src); });
   // second operands: of 8 ranks at a time when the results go to every rank (16 of them and 16
   // sources would not fit the registers), else the one of the destination
@@ -381,8 +389,13 @@ cudaError_t launch(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream
 
 template <int DT, int NR, bool HOOK, bool EXACT, bool FOLDED = false>
 cudaError_t launch_all(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
-  return F.all ? launch<pl_flat_reduce_kernel<DT, NR, HOOK, true, EXACT, FOLDED>>(P, F, stream)
-               : launch<pl_flat_reduce_kernel<DT, NR, HOOK, false, EXACT, FOLDED>>(P, F, stream);
+  auto by_hint = [&](auto all) {
+    if constexpr (all() || NR <= 8 || EXACT) {
+      if (P.hints & 1u) return launch<pl_flat_reduce_kernel<DT, NR, HOOK, all(), EXACT, FOLDED, true>>(P, F, stream);
+    }
+    return launch<pl_flat_reduce_kernel<DT, NR, HOOK, all(), EXACT, FOLDED, false>>(P, F, stream);
+  };
+  return F.all ? by_hint(std::true_type{}) : by_hint(std::false_type{});
 }
 template <int DT, int NR, bool HOOK>
 cudaError_t launch_reduce(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
