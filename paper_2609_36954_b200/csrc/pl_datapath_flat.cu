@@ -399,15 +399,19 @@ cudaError_t launch_all(const FlatParams& P, const FlatLaunch& F, cudaStream_t st
 }
 template <int DT, int NR, bool HOOK>
 cudaError_t launch_reduce(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
-  if constexpr (HOOK) {
-    if (P.n_ranks == NR) return launch_all<DT, NR, true, true>(P, F, stream);
-    if (P.n_ranks == 3) return launch_all<DT, 3, true, true>(P, F, stream);
-    if (P.n_ranks == 6) return launch_all<DT, 6, true, true>(P, F, stream);
+  if constexpr (HOOK) {  // EXACT for 2, 3, 4, 6, 8 and 16 ranks, the counts it was measured at; another takes the next bound's
+    if constexpr (NR == 4) {
+      if (P.n_ranks == 3) return launch_all<DT, 3, true, true>(P, F, stream);
+    }
+    if constexpr (NR == 8) {
+      if (P.n_ranks == 6) return launch_all<DT, 6, true, true>(P, F, stream);
+    }
+    if (NR <= 4 || P.n_ranks == NR) return launch_all<DT, NR, true, true>(P, F, stream);
+  } else if (F.folded) {
+    return launch_all<DT, NR, false, false, true>(P, F, stream);
   }
-  if constexpr (!HOOK) {
-    if (F.folded) return launch_all<DT, NR, false, false, true>(P, F, stream);
-  }
-  return launch_all<DT, NR, HOOK, false>(P, F, stream);
+  if constexpr (!HOOK || NR > 4) return launch_all<DT, NR, HOOK, false>(P, F, stream);
+  else return cudaErrorInvalidValue;  // not reached
 }
 template <int DT, bool HOOK>
 cudaError_t launch_dt(const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
