@@ -1074,21 +1074,18 @@ pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index) {
     return PL_OK;
   }
   if (s->ring || s->folded) {  // they read no wait entries: from here on the op queues execute the schedule
-    const bool ring = s->ring, folded = s->folded;
-    char* const spans = s->d_blob;
-    s->d_blob = nullptr;
+    const bool ring = s->ring, folded = s->folded;  // nothing of either is on the device (the spans of a folded ring are a run)
     s->ring = s->folded = s->flat = false;
     flatten(s, s->comm->dtype);
     const pl_status_t st = upload(s, s->comm->R);
     if (st != PL_OK) {
       if (s->d_blob) cudaFree(s->d_blob);
-      s->d_blob = spans;
+      s->d_blob = nullptr;
       s->sync_bytes = 0;
       s->ring = ring;
       s->folded = s->flat = folded;
       return st;
     }
-    if (spans) cudaFree(spans);
     fill_info(s, s->comm->R);
   }
   const size_t pos = (size_t)s->topo_to_dev[op_index];

@@ -269,7 +269,7 @@ LayerKernel kernel_t(int R, bool full) {
       case 8: return exact(std::integral_constant<int, 8>{});
       case 12: return exact(std::integral_constant<int, 12>{});
       case 16: return exact(std::integral_constant<int, 16>{});
-      default: return pl_layers_kernel<DT, NR, false, CLUSTER, false, false>;
+      default: return pl_layers_kernel<DT, PL_MAX_RANKS, false, CLUSTER, false, false>;  // 9 to 15 but for 12
     }
   }
 }
