@@ -501,6 +501,13 @@ pl_status_t pl_schedule_debug_drop_wait(pl_schedule_t s, size_t op_index);
  * exercise the bounded-wait path without hanging a GPU. */
 pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index);
 
+/* TEST HOOK: raise the device-resident epoch of a schedule that runs layer by layer with flags, as if an execute had
+ * gone by without its signals: every CTA of the next execute waits for more than will come and gives up at the time
+ * limit.  Where pl_schedule_debug_break_wait has such a schedule run a kernel with that hook in it, this one leaves the
+ * kernel as it ships.  No execute of the schedule may be in flight; pl_comm_reset undoes it.
+ * Errors: PL_ERR_INVALID_ARG (any other schedule, or another device current), PL_ERR_CUDA. */
+pl_status_t pl_schedule_debug_raise_epoch(pl_schedule_t s);
+
 pl_status_t pl_schedule_destroy(pl_schedule_t s);
 
 /* ---- datapath ---------------------------------------------------------------------- */

@@ -102,6 +102,7 @@ EXPORTS = [
     "pl_comm_last_error", "pl_probe_hbm",
     "pl_schedule_build", "pl_schedule_build_v", "pl_schedule_build_layers", "pl_schedule_build_rooted", "pl_schedule_info",
     "pl_schedule_dump", "pl_schedule_validate", "pl_schedule_debug_break_wait", "pl_schedule_debug_drop_wait",
+    "pl_schedule_debug_raise_epoch",
     "pl_schedule_trace_read", "pl_schedule_destroy",
     "pl_execute", "pl_execute_host", "pl_execute_host_async", "pl_comm_host_fence", "pl_comm_host_sync", "pl_comm_host_stats", "pl_comm_tune",
     "pl_moe_plan_create", "pl_moe_plan_destroy", "pl_moe_dispatch", "pl_moe_combine", "pl_moe_plan_read",
@@ -145,6 +146,7 @@ def load():
         "pl_schedule_validate": [vp, C.c_char_p, sz],
         "pl_schedule_debug_break_wait": [vp, sz],
         "pl_schedule_debug_drop_wait": [vp, sz],
+        "pl_schedule_debug_raise_epoch": [vp],
         "pl_schedule_trace_read": [vp, vp, sz, vp],
         "pl_schedule_destroy": [vp],
         "pl_execute": [vp, P(pl_bufs_t), vp],
@@ -311,6 +313,10 @@ def pl_schedule_validate(s):
 
 def pl_schedule_debug_break_wait(s, op_index):
     _check(load().pl_schedule_debug_break_wait(s, op_index), "pl_schedule_debug_break_wait")
+
+
+def pl_schedule_debug_raise_epoch(s):
+    _check(load().pl_schedule_debug_raise_epoch(s), "pl_schedule_debug_raise_epoch")
 
 
 def pl_schedule_trace_read(s, n_ops, stream=0):

@@ -1101,6 +1101,15 @@ pl_status_t pl_schedule_debug_break_wait(pl_schedule_t s, size_t op_index) {
   return PL_OK;
 }
 
+pl_status_t pl_schedule_debug_raise_epoch(pl_schedule_t s) {
+  if (!s || !s->layer_kernel || s->layer_cluster || !s->d_blob || !on_comm_device(s->comm)) return PL_ERR_INVALID_ARG;
+  unsigned long long epoch = 0;
+  if (cudaMemcpy(&epoch, s->d_blob + s->off_epoch, sizeof(epoch), cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
+  ++epoch;
+  if (cudaMemcpy(s->d_blob + s->off_epoch, &epoch, sizeof(epoch), cudaMemcpyHostToDevice) != cudaSuccess) { cudaGetLastError(); return PL_ERR_CUDA; }
+  return PL_OK;
+}
+
 pl_status_t pl_schedule_destroy(pl_schedule_t s) {
   if (!s) return PL_ERR_INVALID_ARG;
   if (s->d_blob) cudaFree(s->d_blob);

@@ -94,6 +94,36 @@ def test_layers_trace_and_time_out(nbytes):
         ses.close()
 
 
+# the kernels for a number of ranks and the one for any other, as they ship: every CTA of an execute waits for signals of
+# one that never ran, gives up, and says so; after a reset the schedule runs again
+@pytest.mark.parametrize("R,dtype", [(8, "bf16"), (9, "f32"), (16, "i32")])
+def test_layers_that_time_out_in_the_kernel_that_ships(R, dtype):
+    n, layers = 16 * 1024 * R // SIZE[dtype], 4
+    ses = Session(R, dtype)
+    try:
+        s = ses.build_layers(B.PL_ALGO_DIRECT_FUSED, n, layers, timeout_ns=20_000_000)
+        assert B.pl_schedule_info(s).grid > 16  # with flags
+        x = [(np.arange(n * layers) % 89 + r).astype(np.int32) for r in range(R)]
+        x = [gen.f32_to_bf16_bits(a.astype(np.float32)) if dtype == "bf16" else a.astype(np.float32 if dtype == "f32" else np.int32) for a in x]
+        want, _ = ses.execute(s, x, repeats=2)
+        B.pl_schedule_debug_raise_epoch(s)
+        with pytest.raises(AssertionError, match="device status 6"):
+            ses.execute(s, x)
+        st = B.pl_comm_status(ses.comm)
+        grid = B.pl_schedule_info(s).grid
+        # third execute, counted as the fourth; layer 1 waits for layer 0, which all CTAs have written
+        assert st.expected == 4 * grid and st.observed == 3 * grid and B.pl_schedule_dump(s)[st.op].layer == 1
+        B.pl_comm_reset(ses.comm, stream_handle())
+        torch.cuda.synchronize()
+        again, _ = ses.execute(s, x, repeats=2)
+        assert all(np.array_equal(a, b) for a, b in zip(want, again))
+        for other in (ses.build_layers(B.PL_ALGO_DIRECT_FUSED, 64 * R, layers), ses.build(B.PL_ALLREDUCE, B.PL_ALGO_DIRECT_FUSED, n, 1 << 20)):
+            with pytest.raises(B.PurlinError):  # one cluster; tiles: no epoch of this kind
+                B.pl_schedule_debug_raise_epoch(other)
+    finally:
+        ses.close()
+
+
 # tiny messages with everything left to the library: the layer executor where the message has a vector for
 # every rank, packets where it has not; the same bits as packets asked for
 @pytest.mark.parametrize("R,dtype,nbytes,want", [
@@ -134,19 +164,21 @@ def test_layers_of_many_ranks_that_stream_run_on_the_register_executor():
 # kernels for a fixed number of ranks, and the one for any other: slices that do not fill a warp, end inside one, and take
 # several turns of a thread, as one cluster and with flags, against the register executor (a grid asked for): the same bits
 @pytest.mark.parametrize("R", [2, 3, 4, 5, 6, 7, 8, 9, 12, 16])
-@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "i32"])
 @pytest.mark.parametrize("units", [1, 33, 149, 2055])
 def test_layers_by_number_of_ranks(R, dtype, units):
-    layers, es = 3, {"bf16": 2, "f32": 4}[dtype]
+    layers, es = 3, SIZE[dtype]
     n = 16 * units * R // es
     ses = Session(R, dtype)
     try:
-        x = [torch.randn(n * layers, device="cuda", generator=torch.Generator("cuda").manual_seed(r)).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
-             for r in range(R)]
-        outs = []
+        x = [torch.randn(n * layers, device="cuda", generator=torch.Generator("cuda").manual_seed(r)) for r in range(R)]
+        x = [(t * 2 ** 30).to(torch.int32) if dtype == "i32" else t.to(torch.bfloat16 if dtype == "bf16" else torch.float32) for t in x]
+        outs, threads = [], []
         for kw in ({}, {"n_ctas": R}):
             s = ses.build_layers(B.PL_ALGO_DIRECT_FUSED, n, layers, **kw)
             outs.append(ses.execute(s, None, repeats=2, d_ins=x)[0])
+            threads.append(B.pl_schedule_info(s).threads)
+        assert threads[0] < 512 == threads[1]  # as many as a slice needs here, the default of the queues there
         for a, b in zip(*outs):
             assert np.array_equal(a, b)
     finally:
