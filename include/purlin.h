@@ -38,8 +38,8 @@
  *     (pl_schedule_info reports each grid): launches that each hold part of the SMs could
  *     otherwise starve each other until the wait limit reports PL_ERR_TIMEOUT.  CTAs wait on one
  *     another in schedules with flags (n_flags > 0) that run on queues or layer by layer.
- *     Schedules without flags do not, nor do rings and layers that run in thread-block clusters
- *     (waits inside a cluster only, whose CTAs are resident together): their grids may be larger
+ *     Schedules without flags do not, nor do rings that are folded, nor rings and layers that run in
+ *     thread-block clusters (waits inside a cluster only, whose CTAs are resident together): their grids may be larger
  *     than the GPU and count nothing here.  A MoE dispatch of more than 1024 routing entries per
  *     source waits too (one CTA per source and 256 tokens).  Issuing all executes on one stream
  *     is always safe.
@@ -128,8 +128,9 @@ typedef enum {
  *                         no partial sum leaves the thread); with PL_OPT_RING_HOPS, and for a
  *                         gathering ring, they go through the shared memory of thread-block
  *                         clusters where that is faster than the op queues.  In both cases
- *                         the info has that launch, no scratch, and the bytes of inputs and
- *                         outputs; the op list still states which rank adds what, in order.
+ *                         the info has that launch, no scratch, and in hbm_bytes the inputs and
+ *                         outputs; bytes_read, bytes_written and the op list still count every
+ *                         hop and state which rank adds what, in order.
  *   PL_ALGO_TREE          all-reduce only: binomial reduce to a root, binomial broadcast from it;
  *                         the root of chunk c is rank c mod R (rank 0 for a one-chunk message).
  * Ring and tree are not in the paper (its only pattern is the direct pull); they are the
@@ -488,7 +489,8 @@ pl_status_t pl_schedule_validate(pl_schedule_t s, char* msg, size_t msg_cap);
  * before its signal was released; the bulk-copy executor stamps the end only for ops that
  * signal, others read 0).  Needs PL_OPT_TRACE at build (PL_ERR_INVALID_ARG otherwise).
  * Synchronises `stream`.  Useful to see where a schedule's time goes and to check on the real
- * device that every waiter started after all of its signallers ended. */
+ * device that every waiter started after all of its signallers ended.  A traced schedule runs on the op queues or,
+ * layer by layer, in a kernel with the stamps in its loop: slower than what runs without the option. */
 pl_status_t pl_schedule_trace_read(pl_schedule_t s, uint64_t* out, size_t cap_entries, void* stream);
 
 /* TEST HOOK: remove the first wait edge of op `op_index` from the host copy of the schedule,
