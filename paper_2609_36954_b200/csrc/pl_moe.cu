@@ -481,8 +481,10 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
   const int p = counts ? (int)min(blockIdx.x, (uint32_t)R - 1u) : (int)((blockIdx.x - counters) / groups);
   const int t0 = counts ? 0 : (int)((blockIdx.x - counters - (uint32_t)p * groups) * Q.rows);
   const int nrows = min((int)Q.rows, T - t0), Kd = g.K, n_tgt = nrows * Kd;  // Kd: entries per token (DEDUP: ranks)
-  // The launch behind is set up as the CTAs exit: released here its CTAs took the room of this one's (dispatch and combine,
-  // deduplicated, 8 x 8 tokens of 14 KiB 10.3 -> 9.8 us, 8 x 64 25.5 -> 25.0; top-8, 8 x 64 29.6 -> 29.3).
+  // Deduplicated the launch behind is set up as the CTAs exit.  Dispatch and combine in turn, us, released here / at the exit, 8 ranks: top-2
+  // 64 tokens of 1 KiB 8.3 / 7.5 one by one, 7.9 / 7.2 in a graph, top-8 8 of 4 KiB 8.9 / 8.4 and 7.8 / 8.2, top-8 64 of 14 KiB 22.1 / 21.5 and 21.3 / 21.6; else
+  // released: top-2 8 tokens of 1 KiB 6.7 / 6.9 and 5.2 / 5.4, top-8 8 of 1 KiB 6.7 / 6.8 and 5.5 / 6.0, top-8 64 of 14 KiB 26.0 / 25.8 and 25.7 / 25.8.
+  if constexpr (!DEDUP) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid < 16) s_cnt[tid] = s_total[tid] = 0;
   if (tid == 0) {
     s_bad = 0;
