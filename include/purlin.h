@@ -125,9 +125,10 @@ typedef enum {
  *                         data as compensated fp32 pairs (PL_F32X2), of int32 data in int32.
  *                         With nothing about the launch asked for, a reducing ring's hops are folded
  *                         into one chain of additions per element, in ring order (same bits, but
- *                         no partial sum leaves the thread); with PL_OPT_RING_HOPS, and for a
- *                         gathering ring, they go through the shared memory of thread-block
- *                         clusters where that is faster than the op queues.  In both cases
+ *                         no partial sum leaves the thread); with PL_OPT_RING_HOPS, for a gathering
+ *                         ring, and for a reduce-scatter of two ranks of 16 to 296 KiB they go
+ *                         through the shared memory of thread-block clusters where that is
+ *                         faster than the op queues.  In both cases
  *                         the info has that launch, no scratch, and in hbm_bytes the inputs and
  *                         outputs; bytes_read, bytes_written and the op list still count every
  *                         hop and state which rank adds what, in order.

@@ -540,13 +540,13 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
     if (S->flat) S->pol.idle_count = 0;
   };
   // A ring with nothing about the launch asked for.  (A processing phase is the queue executors' business.)  With every
-  // rank's buffers in one memory a thread can make all hops of a unit: faster than hops through memory at every size
-  // measured, 2 to 16 ranks (2 x 64 KiB 2.5 us both, 8 x 64 MiB 237 / 87 us; the others in pl_datapath_flat.cu).  An
+  // rank's buffers in one memory a thread can make all hops of a unit: faster than hops at nearly every size,
+  // 2 to 16 ranks (8 x 64 MiB 237 / 87 us; the others in pl_datapath_flat.cu, the exception at ring_folds()).  An
   // all-gather has no partial sums to keep, and goes as the direct one if that is what is wanted.
   if (!comm->planner && rq.algo == PL_ALGO_RING && !hook && !S->trace && all_default && rq.n_layers == 0) {
     const bool reduce = rq.coll != PL_ALLGATHER;
     const uint64_t part = rq.count_per_rank * (uint64_t)elem_size(comm->dtype) / (reduce ? (uint64_t)comm->R : 1ull) / 16;
-    if (reduce && !(flags & PL_OPT_RING_HOPS)) {
+    if (reduce && !(flags & PL_OPT_RING_HOPS) && ring_folds(comm->R, rq.coll == PL_ALLREDUCE, part, comm->sm_count)) {
       ring_plan(comm->R, rq.coll == PL_ALLREDUCE, part, &S->flat_spans);
       lay_flat(true, rq.coll == PL_ALLREDUCE);
       S->folded = S->flat_launch.folded = S->flat;

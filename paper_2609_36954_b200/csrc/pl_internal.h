@@ -276,6 +276,8 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
 bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run);
 // flat_plan() for a reducing ring (a partition's chain of hops is one sum per unit); empty without units.
 void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* spans);
+// True where a reducing ring goes as one chain of additions per unit (else its hops are kept).
+bool ring_folds(int R, bool gather, uint64_t part_units, int sm_count);
 // True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
 // tma: the policy picked the bulk-copy datapath (the working set streams from HBM).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes);

@@ -1314,6 +1314,14 @@ bool flat_plan(const Lowered& L, int R, int dtype, std::vector<FlatSpan>* spans,
   return !spans->empty();
 }
 
+// A reduce-scatter of two ranks is one hop, and with one small CTA per SM (ring_shape()) the cluster makes it sooner than a few
+// tiles of four units per thread.  us in a graph, hop / folded, by KiB per rank: bf16 8 0.99 / 0.96, 32 1.03 / 1.33, 128 1.03 / 1.37, 256
+// 1.09 / 1.40, 512 1.74 / 1.42; fp32 8 1.07 / 0.99, 16 1.09 / 1.16, 256 1.20 / 1.60, 512 1.74 / 1.60; launched one by one the same.  Its all-reduce is ahead
+// folded at every size (4 KiB 1.53 / 0.99, 256 KiB 1.94 / 1.57).
+bool ring_folds(int R, bool gather, uint64_t part_units, int sm_count) {
+  return R > 2 || gather || part_units < 512 || 2 * part_units > 128ull * sm_count;
+}
+
 void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* spans) {
   spans->clear();
   if (!part_units) return;

@@ -23,6 +23,7 @@ def rules(tmp_path_factory):
     u64, i, u32, p = C.c_uint64, C.c_int, C.c_uint32, C.c_void_p
     L.t_flat_plan.argtypes = [i, i, i, i, u64, u64, p, i, u32, p, i, p, p]
     L.t_queues_faster.argtypes = [i, i, u32, i, i, i, i, u64]
+    L.t_ring_folds.argtypes = [i, i, u64]
     L.t_combine_by_parts.argtypes = [u64, u32, i, u64]
     L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
     L.t_layers.argtypes = [i, u64, i]
@@ -100,6 +101,12 @@ def ring(rules, R, dtype, coll, nbytes, chunk=MIB):
     (16, "f32", "ar", 16, 256, 1), (16, "bf16", "ar", 64, 1024, 1), (8, "f32", "ar", 256, 1024, 1), (2, "u8", "ag", 1, 64, 1), (2, "u8", "ag", 2, 64, 0)])
 def test_rings_that_stay_on_the_queues(rules, R, dtype, coll, mib, kib, clusters):
     assert (ring(rules, R, dtype, coll, mib * MIB, kib << 10)[1] > 0) == clusters
+
+
+# ranks, units of a partition: the one hop of two ranks stays in clusters while they are one small CTA per SM
+@pytest.mark.parametrize("R,gather,units,folds", [(2, 0, 511, 1), (2, 0, 512, 0), (2, 0, 8192, 0), (2, 0, 9472, 0), (2, 0, 9473, 1), (2, 1, 2048, 1), (3, 0, 2048, 1), (8, 0, 2048, 1)])
+def test_the_hop_of_two_ranks_is_kept_where_it_is_faster(rules, R, gather, units, folds):
+    assert rules.t_ring_folds(R, gather, units) == folds
 
 
 @pytest.mark.parametrize("R", [2, 3, 5, 8, 12, 16])
