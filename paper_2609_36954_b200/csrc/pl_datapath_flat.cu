@@ -455,21 +455,6 @@ FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, u
   return F;
 }
 
-// Else the launch behind is set up as the CTAs exit.  Released at the start its CTAs take the room that is left, and in a
-// grid of middle size they then share SMs while others idle, once launches are enqueued faster than the GPU finishes
-// them.  us, released / not, back to back in a CUDA graph: sums to every rank 8 x 16 KiB (4 CTAs) 1.95 / 2.03, 2 x 128 KiB (8)
-// 1.79 / 1.85, 8 x 64 KiB (16) 2.09 / 2.02, 8 x 128 KiB (32) 2.31 / 2.05, 4 x 512 KiB (64) 2.52 / 1.90, 8 x 512 KiB (128) 3.56 / 2.15; launched one
-// by one 8 x 1 MiB (256) 4.85 / 3.02, 8 x 2 MiB (512) 6.4 / 5.2, 8 x 8 MiB (2048) 21.9 / 22.0.  Sums to one rank (one-shot) 4 x 16 KiB
-// (8) 1.38 / 1.61, 4 x 128 KiB (64) 1.48 / 1.63, 8 x 64 KiB (128) 1.94 / 1.81, 4 x 512 KiB (256) 2.30 / 2.02, 4 x 1 MiB (512) 2.35 / 2.75, 8 x 1
-// MiB (2048) 6.26 / 6.45.  Copies to every rank 8 x 4 KiB (8) 0.91 / 1.30, 4 x 128 KiB (32) 1.19 / 1.40, 8 x 256 KiB (64) 1.83 / 1.70, 8 x
-// 512 KiB (128) 3.53 / 1.73.  Copies to one rank read their span from memory first (all-to-all-v 8 x 2 MiB 5.0 / 5.4), the bulk-copy
-// forms are the same or 1 % slower without: they always release.
-bool flat_release(bool reduce, bool all, bool bulk, uint64_t blocks) {
-  if (bulk || (!reduce && !all)) return true;
-  if (all) return blocks <= (reduce ? 8 : 32);
-  return blocks <= 64 || blocks >= 512;
-}
-
 cudaError_t launch_flat(int dtype, const FlatParams& P, const FlatLaunch& F, cudaStream_t stream) {
   if (!F.reduce) {
     if (F.bulk) return F.all ? launch<pl_flat_bulk_copy_kernel<true>>(P, F, stream) : launch<pl_flat_bulk_copy_kernel<false>>(P, F, stream);

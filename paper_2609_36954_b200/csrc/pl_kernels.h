@@ -27,7 +27,6 @@ bool layers_cluster_fits(int dtype, int R, bool hook, int grid, int threads);
 
 // schedules without flags, one CTA per tile
 FlatLaunch flat_launch(int R, bool reduce, bool all, bool bulk, uint32_t hook, uint64_t total_units, int sm_count);
-bool flat_release(bool reduce, bool all, bool bulk, uint64_t blocks);
 cudaError_t launch_flat(int dtype, const FlatParams& P, const FlatLaunch& F, cudaStream_t stream);
 
 // ring schedules, a cluster per tile.  ring_prepare: clusters that can be resident at once (0: none)

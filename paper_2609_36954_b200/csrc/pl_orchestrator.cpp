@@ -1342,6 +1342,24 @@ bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run) {
   return true;
 }
 
+// Which launches without queues release the one behind them at their start; else it is set up as their CTAs exit.  Released early its
+// CTAs take the room that is left, and in a grid of middle size they then share SMs while others idle, once launches are enqueued
+// faster than the GPU finishes them.  us in a CUDA graph, released / not.
+// Sums to every rank: bf16 8 x 4 KiB (1 CTA) 1.73 / 1.64, 8 x 32 KiB (8) 1.78 / 1.69, 4 x 512 KiB (64) 2.52 / 1.90, 8 x 512 KiB (128) 3.56 / 2.15, 8 x 2
+// MiB (512) 5.33 / 4.99, fp32 5.38 / 5.14, 3 x 3 MiB with residual (768) 3.49 / 3.08; from two waves of two CTAs per SM on it gains a little: 8 x 4 MiB
+// (1024) 11.74 / 11.84, 8 x 8 MiB (2048) 21.85 / 21.94, 16 x 4 MiB (1024) 23.16 / 23.20.
+// Copies to every rank: 8 x 4 KiB gathered (8) 1.05 / 0.89, 4 x 128 KiB (32) 1.15 / 1.10, 8 x 256 KiB (64) 1.53 / 1.39, 8 x 2 MiB (512) 4.53 / 3.35, 8 x 4 MiB (1024) 6.65 /
+// 6.23; beyond one wave, once 24 MiB are written, the stores of one launch cover the start of the next: 8 x 5 MiB (1280) 8.56 / 8.71, 8 x 6 MiB 10.06 /
+// 10.36, 12 x 6 MiB 14.23 / 14.61, 4 x 5 MiB (1280) 4.25 / 3.91, 4 x 6 MiB (1536) 5.14 / 5.19, 2 x 8 MiB (2048) 3.60 / 3.42, 2 x 12 MiB (3072) 6.80 / 6.88.
+// Sums to one rank (one-shot): 8 x 4 KiB (8) 1.30 / 1.16, 4 x 16 KiB (8) 1.25 / 1.13, 4 x 64 KiB (32) 1.32 / 1.23, 16 x 16 KiB (64) 2.03 / 1.88, 8 x 64 KiB (128) 1.94 /
+// 1.81, 4 x 512 KiB (256) 2.30 / 2.02, 8 x 256 KiB (512) 2.22 / 2.32, 4 x 1 MiB (512) 2.35 / 2.75, 8 x 1 MiB (2048) 6.26 / 6.45.  Copies to one rank 8 x 2 MiB
+// (all-to-all-v) 5.0 / 5.4; the bulk-copy forms are the same or 1 % slower without: they always release.
+bool flat_release(int R, bool reduce, bool all, bool bulk, uint64_t blocks) {
+  if (bulk || (!reduce && !all)) return true;
+  if (reduce) return blocks >= (all ? 1024 : 512);
+  return blocks > 8 * 148 && blocks * (uint64_t)R * kFlatThreads * 16 >= (24u << 20);
+}
+
 // A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a short
 // one (8 x 1 MiB 7.0 us, flat 7.5, with residual 7.1 / 8.0; 4 x 1 MiB 4.7 / 6.4; at 4 x 4 MiB flat is ahead,
 // 11.3 / 12.8), and a streaming one without residual (8 x 64 MiB 267 us, flat 286; 4 x 64 MiB 139 / 148; 16 x
