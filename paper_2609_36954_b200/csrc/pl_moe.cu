@@ -401,6 +401,7 @@ __global__ void __launch_bounds__(256) moe_derive_ranks_kernel(const __grid_cons
 struct SmallParams {
   uint32_t rows;            // tokens per CTA
   int K0, epr0;             // DEDUP: slots per token and experts per rank of the routing
+  uint32_t release;         // release the launch behind at the start
   int32_t* ridx;            // DEDUP: distinct destination ranks per token, padded with -1, and the slots on each
   int32_t* rmask;
   uint64_t pad[4];
@@ -481,10 +482,7 @@ __global__ void __launch_bounds__(kSmallThreads) moe_small_kernel(const __grid_c
   const int p = counts ? (int)min(blockIdx.x, (uint32_t)R - 1u) : (int)((blockIdx.x - counters) / groups);
   const int t0 = counts ? 0 : (int)((blockIdx.x - counters - (uint32_t)p * groups) * Q.rows);
   const int nrows = min((int)Q.rows, T - t0), Kd = g.K, n_tgt = nrows * Kd;  // Kd: entries per token (DEDUP: ranks)
-  // Deduplicated the launch behind is set up as the CTAs exit.  Dispatch and combine in turn, us, released here / at the exit, 8 ranks: top-2
-  // 64 tokens of 1 KiB 8.3 / 7.5 one by one, 7.9 / 7.2 in a graph, top-8 8 of 4 KiB 8.9 / 8.4 and 7.8 / 8.2, top-8 64 of 14 KiB 22.1 / 21.5 and 21.3 / 21.6; else
-  // released: top-2 8 tokens of 1 KiB 6.7 / 6.9 and 5.2 / 5.4, top-8 8 of 1 KiB 6.7 / 6.8 and 5.5 / 6.0, top-8 64 of 14 KiB 26.0 / 25.8 and 25.7 / 25.8.
-  if constexpr (!DEDUP) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!DEDUP && Q.release) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid < 16) s_cnt[tid] = s_total[tid] = 0;
   if (tid == 0) {
     s_bad = 0;
@@ -1088,7 +1086,12 @@ static int launch_dispatch(pl_moe_plan_t plan, const DispatchPtrs& P, const MoeG
   return launched + 1;
 }
 
-static bool launch_small(const DispatchPtrs& P, const MoeGeo& g, const SmallParams& Q, bool dedup, cudaStream_t cs) {
+// The launch behind is released early where few bytes are written; else, and deduplicated, it is set up as the CTAs exit.  Dispatch and
+// combine in turn, us, released / not, one by one and in a graph: top-2 8 x 8 tokens of 1 KiB 6.7 / 6.9 and 5.2 / 5.4, top-8 8 x 8 of 1 KiB 6.7 / 6.8 and 5.5
+// / 6.0, top-2 4 x 256 of 4 KiB 11.3 / 11.5 and 11.0 / 11.3; from 12 MiB of rows on 4 x 64 top-8 of 14 KiB 14.15 / 13.88 and 13.5 / 13.6, 8 x 64 26.0 / 25.8 and 25.65 /
+// 25.84, top-2 8 x 64 10.8 / 10.5 and 10.2 / 10.3; deduplicated top-2 8 x 64 of 1 KiB 8.3 / 7.5 and 7.9 / 7.2, top-8 8 x 8 of 4 KiB 8.9 / 8.4 and 7.8 / 8.2.
+static bool launch_small(const DispatchPtrs& P, const MoeGeo& g, SmallParams Q, bool dedup, cudaStream_t cs) {
+  Q.release = (uint64_t)g.R * g.T * g.K * g.row_bytes < (12ull << 20);
   const dim3 grid((unsigned)g.R * (((unsigned)g.T + Q.rows - 1) / Q.rows) + (unsigned)g.R + 1u);
   return launch_after(true, dedup ? moe_small_kernel<true> : moe_small_kernel<false>, grid, kSmallThreads, 128 + (size_t)Q.rows * g.row_bytes, cs, P, g, Q);
 }
@@ -1110,7 +1113,7 @@ pl_status_t pl_moe_dispatch(pl_moe_plan_t plan, const void* const* x, const int3
     P.meta[r] = recv_meta ? recv_meta[r] : nullptr;
   }
   if (plan->small_rows) {
-    if (!launch_small(P, g, SmallParams{plan->small_rows, g.K, g.epr, nullptr, nullptr}, false, static_cast<cudaStream_t>(stream))) return PL_ERR_CUDA;
+    if (!launch_small(P, g, SmallParams{plan->small_rows, g.K, g.epr, 0, nullptr, nullptr}, false, static_cast<cudaStream_t>(stream))) return PL_ERR_CUDA;
     g_launches.fetch_add(1);
     plan->dispatched = true;
     return PL_OK;
@@ -1209,7 +1212,7 @@ pl_status_t pl_moe_dispatch_dedup(pl_moe_plan_t plan, const void* const* x, cons
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   if (plan->small_rows_dedup) {
     for (int r = 0; r < g.R; ++r) P.idx[r] = topk_idx[r];
-    if (!launch_small(P, d, SmallParams{plan->small_rows_dedup, g.K, g.epr, plan->d_ridx, plan->d_rmask}, true, cs)) return PL_ERR_CUDA;
+    if (!launch_small(P, d, SmallParams{plan->small_rows_dedup, g.K, g.epr, 0, plan->d_ridx, plan->d_rmask}, true, cs)) return PL_ERR_CUDA;
     g_launches.fetch_add(1);
     plan->dispatched_dedup = true;
     return PL_OK;
