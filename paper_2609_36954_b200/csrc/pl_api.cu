@@ -534,8 +534,8 @@ pl_status_t build_common(pl_comm_t comm, BuildRequest rq, const pl_sched_opts_t*
       blocks += (f.units + S->flat_launch.tile - 1) / S->flat_launch.tile;
     }
     S->flat_launch.blocks = (uint32_t)blocks;
-    S->flat_launch.release = flat_release(comm->R, reduce, all, S->flat_launch.bulk, blocks);
     S->flat_is_run = units > 0 && flat_run(S->flat_spans, &S->flat_run);
+    S->flat_launch.release = flat_release(comm->R, reduce, all, S->flat_launch.bulk, S->flat_is_run, blocks);
     S->flat = units > 0 && blocks <= 0x7FFFFFFFull;
     if (S->flat) S->pol.idle_count = 0;
   };

@@ -279,7 +279,7 @@ void ring_plan(int R, bool gather, uint64_t part_units, std::vector<FlatSpan>* s
 // True where a reducing ring goes as one chain of additions per unit (else its hops are kept).
 bool ring_folds(int R, bool gather, uint64_t part_units, int sm_count);
 // True if a launch of tiles releases the one behind it at its start.
-bool flat_release(int R, bool reduce, bool all, bool bulk, uint64_t blocks);
+bool flat_release(int R, bool reduce, bool all, bool bulk, bool run, uint64_t blocks);
 // True where the op queues run a schedule that flat_plan() accepts faster than one CTA per tile.
 // tma: the policy picked the bulk-copy datapath (the working set streams from HBM).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes);

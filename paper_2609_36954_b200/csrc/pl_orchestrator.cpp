@@ -1354,8 +1354,10 @@ bool flat_run(const std::vector<FlatSpan>& spans, FlatRun* run) {
 // Sums to one rank (one-shot): 8 x 4 KiB (8) 1.30 / 1.16, 4 x 16 KiB (8) 1.25 / 1.13, 4 x 64 KiB (32) 1.32 / 1.23, 16 x 16 KiB (64) 2.03 / 1.88, 8 x 64 KiB (128) 1.94 /
 // 1.81, 4 x 512 KiB (256) 2.30 / 2.02, 8 x 256 KiB (512) 2.22 / 2.32, 4 x 1 MiB (512) 2.35 / 2.75, 8 x 1 MiB (2048) 6.26 / 6.45.  Copies to one rank 8 x 2 MiB
 // (all-to-all-v) 5.0 / 5.4; the bulk-copy forms are the same or 1 % slower without: they always release.
-bool flat_release(int R, bool reduce, bool all, bool bulk, uint64_t blocks) {
-  if (bulk || (!reduce && !all)) return true;
+// Tiles that read their span from memory (no run) do so ahead of the wait for the launch in front, if they are there by then: few of them are released
+// (all-gather-v 2 x 64 KiB 1.03 / 1.23, 4 x 64 KiB 1.10 / 1.37).
+bool flat_release(int R, bool reduce, bool all, bool bulk, bool run, uint64_t blocks) {
+  if (bulk || (!reduce && !all) || (!run && blocks <= 32)) return true;
   if (reduce) return blocks >= (all ? 1024 : 512);
   return blocks > 8 * 148 && blocks * (uint64_t)R * kFlatThreads * 16 >= (24u << 20);
 }

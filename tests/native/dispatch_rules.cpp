@@ -49,7 +49,7 @@ int t_queues_faster(int R, int dtype, uint32_t hook, int algo, int reduce, int a
 
 int t_ring_folds(int R, int gather, uint64_t part_units) { return ring_folds(R, gather, part_units, 148); }
 
-int t_flat_release(int R, int reduce, int all, int bulk, uint64_t blocks) { return flat_release(R, reduce, all, bulk, blocks); }
+int t_flat_release(int R, int reduce, int all, int bulk, int run, uint64_t blocks) { return flat_release(R, reduce, all, bulk, run, blocks); }
 
 int t_combine_by_parts(uint64_t n_tok, uint32_t units, int topk, uint64_t turns) { return combine_by_parts(n_tok, units, topk, turns); }
 

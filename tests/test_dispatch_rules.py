@@ -24,7 +24,7 @@ def rules(tmp_path_factory):
     L.t_flat_plan.argtypes = [i, i, i, i, u64, u64, p, i, u32, p, i, p, p]
     L.t_queues_faster.argtypes = [i, i, u32, i, i, i, i, u64]
     L.t_ring_folds.argtypes = [i, i, u64]
-    L.t_flat_release.argtypes = [i, i, i, i, u64]
+    L.t_flat_release.argtypes = [i, i, i, i, i, u64]
     L.t_combine_by_parts.argtypes = [u64, u32, i, u64]
     L.t_small_dispatch_rows.argtypes = [i, i, i, i, i, u64]
     L.t_layers.argtypes = [i, u64, i]
@@ -67,8 +67,9 @@ def test_all_gather_of_many_ranks_stays_on_the_queues_where_they_are_faster(rule
     (8, 0, 1, 8, 0), (8, 0, 1, 1184, 0), (8, 0, 1, 1280, 1), (4, 0, 1, 1280, 0), (4, 0, 1, 1536, 1), (2, 0, 1, 2048, 0), (2, 0, 1, 3072, 1),
     (8, 0, 0, 1, 1), (8, 0, 0, 300, 1), (8, 0, 0, 4096, 1)])
 def test_grids_that_release_the_launch_behind_them(rules, R, reduce, every, blocks, release):
-    assert rules.t_flat_release(R, reduce, every, 0, blocks) == release
-    assert rules.t_flat_release(R, reduce, every, 1, blocks)  # bulk copies
+    assert rules.t_flat_release(R, reduce, every, 0, 1, blocks) == release
+    assert rules.t_flat_release(R, reduce, every, 0, 0, blocks) == (release or blocks <= 32)  # spans read from memory
+    assert rules.t_flat_release(R, reduce, every, 1, 1, blocks)  # bulk copies
 
 
 # tokens of all ranks, KiB of a row, slots: a combine that reads about 200 MB or more takes whole rows in turn
