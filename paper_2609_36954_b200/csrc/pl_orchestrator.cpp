@@ -793,8 +793,8 @@ void a2a_direct_staged(Emitter& em, const Geo& g, uint64_t capacity) {
 }  // namespace
 
 // One cluster while it has at most 256 KiB of inputs to read per layer (16 KiB per CTA): at
-// R = 8 a 16 KiB layer takes 1.22 us as a cluster and 1.66 us with flags, 32 KiB 1.59-2.03
-// (the two values are two B200s) against 1.95, 64 KiB 2.16-2.24 against 1.96.  With flags as many
+// R = 8 a 16 KiB layer takes 1.13 us as a cluster, 32 KiB 1.42, 40 KiB 1.71 against 1.69 with flags, 48 KiB 1.75 / 1.70, 64 KiB 2.09 /
+// 1.71; fp32 32 KiB 1.61, 40 KiB 1.63 / 1.83, 48 KiB 1.79 / 1.83, 64 KiB 2.18 / 1.84.  With flags as many
 // CTAs as there are slices of at least 32 units: 16, 32, 64 or 128 made no difference at 64 KiB
 // and above as long as every SM has a slice at the large end (1 MiB: 128 CTAs 3.6 us, 64 CTAs 5 us).
 // Lines of the next layer's inputs are asked into L2 ahead while they and what this layer writes have room there.
@@ -1362,10 +1362,10 @@ bool flat_release(int R, bool reduce, bool all, bool bulk, bool run, uint64_t bl
   return blocks > 8 * 148 && blocks * (uint64_t)R * kFlatThreads * 16 >= (24u << 20);
 }
 
-// A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a short
-// one (8 x 1 MiB 7.0 us, flat 7.5, with residual 7.1 / 8.0; 4 x 1 MiB 4.7 / 6.4; at 4 x 4 MiB flat is ahead,
-// 11.3 / 12.8), and a streaming one without residual (8 x 64 MiB 267 us, flat 286; 4 x 64 MiB 139 / 148; 16 x
-// 64 MiB 549 / 570; with residual flat is ahead, 325 / 505).
+// A fused all-reduce of bf16 with fp32 output keeps the queues where their wider stores win: a streaming one without residual
+// (8 x 64 MiB 268 us, flat 285; 4 x 64 MiB 138 / 146; 16 x 64 MiB 549 / 570; with residual flat is ahead, 325 / 505), and a short one.
+// The short line was measured while flat launches of middle size released the one behind them early; in a graph it is now, queues / flat, 8
+// x 1 MiB 6.3 / 6.3 us, with residual 10.4 / 6.8, 8 x 64 KiB 3.0 / 3.3, 8 x 512 KiB 4.5 / 3.6, 4 x 1 MiB 3.9 / 3.5, 2 x 2 MiB 4.9 / 3.4: it may move down.
 // A one-shot all-reduce reads every input once per rank.  Flat, the tiles go out destination by
 // destination, so every sweep passes over all inputs; the op list has the destinations of a chunk next
 // to one another, which lets all reads but the first hit L2 when the inputs do not fit it.  us, queues /
@@ -1376,12 +1376,12 @@ bool flat_release(int R, bool reduce, bool all, bool bulk, bool run, uint64_t bl
 // With a processing phase the register queues of bf16 take twice as long; the bulk-copy queues are ahead where
 // their ranks divide the SMs evenly (residual 8 x 16 156 / 189, 12 x 64 1365 / 1565, 14 x 64 2191 / 2088, 3 x 64 170 / 142; fp32
 // output 8 x 64 663 / 743, 16 x 64 2773 / 2661; both 8 x 64 633 / 818, 14 x 64 2212 / 2199).  Float sums of 12 and 16 ranks leave half
-// of flat's registers idle while 144 queues divide evenly among them: 12 x 768 KiB bf16 10 / 14, 12 x 3 MiB 47 / 52, 16 x
-// 512 KiB 12.3 / 14.1, while 13 ranks take 16.4 / 15.1 and 73 / 58.
+// of flat's registers idle while 144 queues divide evenly among them: 12 x 768 KiB bf16 9.1 / 12.8, 12 x 3 MiB 45.7 / 49.5, 16 x
+// 512 KiB 10.1 / 13.2, fp32 14.4 / 17.5, while 13 ranks take 16.4 / 15.1 and 73 / 58.
 // An all-gather of more than 8 ranks stores every unit more than 8 times; between 10 and 36 MiB written the
-// queues, which keep 144 CTAs at it, are ahead (us, queues / flat: 16 x 768 KiB 3.7 / 8.5, 1 MiB 4.3 / 9.4, 2 MiB 7.8 /
-// 11.1, 3 MiB 10.0 / 11.4, 4 MiB 13.2 / 14.0; 14 x 1 MiB 4.1 / 8.5; 12 x 1 MiB 3.7 / 7.1, 4 MiB 10.3 / 10.9); below both
-// are bound by the launch, above by HBM (16 x 8 MiB 26.7 / 23.5).
+// queues keep 144 CTAs at it, which was ahead while flat launches of middle size released the one behind them early (16 x 1 MiB 4.3 /
+// 9.4 us).  In a graph it is now, queues / flat, 16 x 640 KiB 2.9 / 3.1, 768 KiB 3.1 / 3.25, 1 MiB 3.7 / 3.35, 2 MiB 7.1 / 6.1; 14 x 1 MiB 3.7 / 3.2; 12 x 1 MiB 3.3 / 2.8, 3 MiB
+// 7.3 / 7.1: the line may move down; above it both are bound by HBM (16 x 8 MiB 26.7 / 23.5).
 bool queues_faster(int R, int dtype, uint32_t hook, int algo, bool reduce, bool all, bool tma, uint64_t message_bytes) {
   const uint64_t inputs = message_bytes * (uint64_t)R, mib = 1u << 20;
   if (!reduce) return all && !tma && R > 8 && inputs >= 10 * mib && inputs <= 36 * mib;  // a gathered message: bytes written
